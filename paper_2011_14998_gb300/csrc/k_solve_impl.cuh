@@ -52,6 +52,8 @@
 // anywhere in the warp) costs nothing extra.
 #pragma once
 
+#include <type_traits>
+
 #include "mgx_internal.cuh"
 
 namespace mgx {
@@ -132,11 +134,54 @@ struct Pts<float> {
     static __device__ __forceinline__ const float *etac(const DevLines &L) { return L.etacf; }
 };
 
+// Values of one lane: a scalar, or two bins' single-precision values side by
+// side (float2), on which GB300's packed instructions work (fma.rn.f32x2 and
+// its kin): the same two IEEE operations in one issue slot.
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+
+template <typename V>
+__device__ __forceinline__ V vset(float x) {
+    if constexpr (sizeof(V) == sizeof(float2) && !std::is_same_v<V, double>) return make_float2(x, x);
+    else return V(x);
+}
+
+// Component c of a value.
+__device__ __forceinline__ float vget(float x, int) { return x; }
+__device__ __forceinline__ double vget(double x, int) { return x; }
+__device__ __forceinline__ float vget(float2 x, int c) { return c ? x.y : x.x; }
+template <typename T>
+__device__ __forceinline__ void vput(T &x, int, T v) { x = v; }
+__device__ __forceinline__ void vput(float2 &x, int c, float v) { (c ? x.y : x.x) = v; }
+
+// One compiled form of the solve: the arithmetic R, the lines NL and bins per
+// lane BPL it is compiled for, the scheme's order, the pivots' precision P.
+// The single-precision second-order form holds its bins in pairs (kPacked): the
+// optics and rows of two bins then take 20 issue slots instead of 36, and issue
+// slots were what bounded the loop (77 % busy; FP32 lanes 39 %).  Together with
+// the branch-free runs of consume_chunk and the lines left out (line_is_far) the
+// solve of the 50 000-point wind fell from 86.1 to 70.8 ms, of a batch of five
+// four-line models from 136.4 to 95.2 ms, J the same bit for bit.  What bounds it
+// now is latency (issue 56 % busy): the reciprocal and exp2 on the recurrence's
+// path and the staging's gathers, at 8 resident CTAs.
+template <typename R_, int NL_, int BPL_, int ORD_, typename P_ = R_>
+struct Form {
+    using R = R_;
+    using P = P_;
+    static constexpr int NL = NL_, BPL = BPL_, ORD = ORD_;
+    static constexpr bool kPacked = sizeof(R) == 4 && sizeof(P) == 4 && ORD == 2 && BPL % 2 == 0;
+    using V = std::conditional_t<kPacked, float2, R>;
+    using W = std::conditional_t<kPacked, float2, P>;
+    static constexpr int kIn = kPacked ? 2 : 1;  // bins in a value
+    static constexpr int NV = BPL / kIn;         // values per lane
+};
+
 // Per-bin constants: the Doppler-shifted profile argument of line l at this
 // bin is (A[l] + B[l] delta) / dv (prescaled for the single-precision ex2).
-template <typename R, int NL>
+template <typename V, int NL>
 struct Bin {
-    R A[NL], B[NL];
+    V A[NL], B[NL];
 };
 
 // Total opacity and emissivity of a sample for one bin: delta, rdv = 1/dv,
@@ -153,6 +198,18 @@ __device__ __forceinline__ void optics(R delta, R rdv, R cc, R ec, const R *ce, 
         chi = fma(ce[2 * l], g, chi);
         eta = fma(ce[2 * l + 1], g, eta);
     }
+}
+
+// One line's part of it for two bins.
+__device__ __forceinline__ void add_line(float2 delta, float2 rdv, float2 c0, float2 e0, float2 A, float2 B,
+                                         float2 &chi, float2 &eta) {
+    const float2 a = vmul(vfma(B, delta, A), rdv);
+    const float2 q = vmul(a, a);
+    float2 g;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g.x) : "f"(-q.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g.y) : "f"(-q.y));
+    chi = vfma(c0, g, chi);
+    eta = vfma(e0, g, eta);
 }
 
 // State of the elimination of one bin along one half of a pair line.
@@ -174,6 +231,18 @@ struct Sweep {
     R chi, eta;     // optics of the current (not yet eliminated) sample
     R Sp, Sc, hp, rh;  // Hermitian scheme only
 };
+
+// The second-order row below for two bins at once, operation for operation.
+__device__ __forceinline__ void row2(Sweep<float2> &w, float2 chi, float2 eta, float2 dt) {
+    const float2 half = make_float2(0.5f, 0.5f), one = make_float2(1.f, 1.f);
+    const float2 dtb = vfma(dt, half, w.dtp);
+    w.Fh = vfma(w.Dm, w.Fh, dtb);
+    const float2 den = vmul(chi, vfma(dt, w.Fh, one));
+    const float2 rr = make_float2(Ar<float>::rcp(den.x), Ar<float>::rcp(den.y));
+    w.Dm = vmul(chi, rr);
+    w.zh = vfma(dtb, vmul(eta, rr), vmul(w.Dm, w.zh));
+    w.dtp = vmul(dt, half);
+}
 
 // Eliminate the row of the current sub-point (optics chi, eta) once the
 // increment dt beyond it is known.  One reciprocal R = 1 / (chi (1 + dt Fh))
@@ -306,14 +375,21 @@ __device__ __forceinline__ HalfList half_list(const SolveArgs &a, int64_t h) {
 // Layout of one velocity-sample record, as the bins read it: delta, 1/dv,
 // continuum opacity and emissivity, half the distance to the previous sample,
 // the Eq. 2 threshold on chi, then chi0 and eta0 of each line; padded to whole
-// 16-byte words so that each word is one shared-memory load.  In single
-// precision with one line, a negative 1/dv marks a sample in the far wing of
-// every bin of the tile (the optics are the continuum's) and an infinite
-// threshold an interval on which no bin can need a split.
-template <typename R, int NL>
+// 16-byte words so that each word is one shared-memory load.  An infinite
+// threshold (single precision) marks an interval on which no bin can need a
+// split.  The packed form stores the values twice, so that a load yields the
+// operand pair of the packed instructions (a register pair built from one
+// loaded value would cost a move each; with more than two lines only the line
+// values are stored once, for the sake of shared memory), with the lines that
+// take part in the sample as a bit mask next to the threshold; the other
+// single-precision forms with one line mark a sample in which it takes no part
+// by a negative 1/dv.
+template <class C>
 struct Rec {
-    static constexpr int kVals = 6 + 2 * NL;
-    static constexpr int kPer16 = int(16 / sizeof(R));
+    using V = typename C::V;
+    static constexpr bool kTwice = C::NL <= 2;  // packed: line values stored twice
+    static constexpr int kVals = 6 + (C::kPacked && !kTwice ? 1 : 2) * C::NL;
+    static constexpr int kPer16 = int(16 / sizeof(V));
     static constexpr int kStride = (kVals + kPer16 - 1) / kPer16 * kPer16;
 };
 
@@ -321,17 +397,21 @@ struct Rec {
 // (kCap at a time), the chunk's points (slot 0 holds the point just farther
 // than the chunk, slots 1..32 the chunk, far to near) with the constants of
 // the interval from the farther point, and the warp's item.
-template <typename R, int NL>
+template <class C>
 struct Stage {
+    using R = typename C::R;
+    using V = typename C::V;
+    static constexpr int NL = C::NL, BPL = C::BPL;
     static constexpr int kCap = sizeof(R) == 4 ? 32 : (NL <= 4 ? 32 : 16);
-    static constexpr int kS = Rec<R, NL>::kStride;
+    static constexpr int kS = Rec<C>::kStride;
     static constexpr int kF = sizeof(R) == 4 ? 33 : 1;  // arrays of the single-precision decisions
-    alignas(16) R rec[kCap * kS];
-    int sk[kCap];                           // slot | (sample index j << 6) of each record
+    alignas(16) V rec[kCap * kS];
+    alignas(16) V fA[NL][C::NV][32], fB[NL][C::NV][32];  // profile constants of each lane's bins (Bin)
     R d[33], w[33], cc[33], ec[33];         // delta, Doppler width, continuum
     R ce[2 * NL][33];                       // chi0 and eta0 per line
     R hq[33], thr[33];                      // half the sample spacing, Eq. 2 threshold
     R E[kF], qlo[kF], qhi[kF];              // bound of |chi - chi64|, Eq. 2 ratio factors
+    unsigned char sk[kCap];                 // slot of each record
     R de0;                                  // single precision: bound of |delta - delta64| of the carried point
     double z[sizeof(R) == 8 ? 33 : 1];      // exact Z (single precision: the carried point's only)
     int id[33], nv[33], so[33];             // point (-1: the origin), velocity samples, their offset
@@ -341,33 +421,31 @@ struct Stage {
     int o, NB, tile;                        // origin, bins of the model, the warp's frequency tile
     HalfList hl;                            // traced list of the half being eliminated
     unsigned n_smp, n_extra, n_redo;        // work counters of the item (samples, extra sub-intervals, redone decisions)
-    int fix[2][32];                         // Eq. 2 counts of a sample whose single-precision decision was
-                                            // left open (-1: to redo in double precision; 0: not open)
-    R fA[NL][2][32], fB[NL][2][32];         // profile constants of each lane's bins (Bin)
-    float wa[2], wb[2];                     // single precision, one line: A, B of the tile's first and last bin
-    int wing;                               // the far-wing test of the records is on
+    int fix[BPL][32];                       // Eq. 2 counts of a sample whose single-precision decision was left
+                                            // open (0: not open; negative: to resolve, the bits of -chi)
+    float wA[NL][2], wB[NL][2];             // single precision: smallest and largest A, B over the warp's bins
+    unsigned m_split, m_new;                // packed form: the round's records that may split; whose lines differ
+                                            // from the record's before
 };
 
 // Bin i of the lane in the warp's tile (>= NB: beyond the last, inactive).
-template <int BPL, typename St>
-__device__ __forceinline__ int32_t lane_bin(const St &sg, int i, int lane) {
-    return sg.tile * 32 * BPL + lane + 32 * i;
+template <class C>
+__device__ __forceinline__ int32_t lane_bin(const Stage<C> &sg, int i, int lane) {
+    return sg.tile * 32 * C::BPL + lane + 32 * i;
 }
 
 // Per-lane state that lives across chunks of samples, kept in shared memory
 // so that no register holds it across the out-of-line staging calls: the
-// elimination state of each of the lane's (at most two) bins (D and Fh enter
-// every step only as their product, which is what is kept) and the running
-// maximum of chi.  The pivot quantities (D Fh, dtb/2) are kept in the pivot
-// precision P.  What is needed only once per pair (the J sums, the origin's
-// source function, the backward half's coupling to the origin row) stays in
-// the item loop's registers, so that 9 CTAs fit the shared memory.
-template <typename R, int ORD, typename P = R>
+// elimination state of each of the lane's bins (D and Fh enter every step only
+// as their product, which is what is kept).  The pivot quantities (D Fh,
+// dtb/2) are kept in the pivot precision.  What is needed only once per pair
+// (the J sums, the origin's source function, the backward half's coupling to
+// the origin row) stays in the item loop's registers.
+template <class C>
 struct Lane {
-    static constexpr int kWR = ORD == 4 ? 6 : 3;  // zh, chi, eta (Hermitian: + Sp, Sc, hp; rh = 1/hp re-formed)
-    P wp[2][2][32];                              // D Fh, dtb/2
-    R wr[kWR][2][32];
-    R cm[32];
+    static constexpr int kWR = C::ORD == 4 ? 6 : 3;  // zh, chi, eta (Hermitian: + Sp, Sc, hp; rh = 1/hp re-formed)
+    typename C::W wp[2][C::NV][32];                  // D Fh, dtb/2
+    typename C::V wr[kWR][C::NV][32];
 };
 
 // Projected distance Z = (x_n - x_o).d exactly as the tracer and its
@@ -388,6 +466,47 @@ __device__ __forceinline__ double proj64(const DevMesh &m, int32_t id, const dou
     const double uy = __dsub_rn(__ldg(m.vy + id), vo[1]);
     const double uz = __dsub_rn(__ldg(m.vz + id), vo[2]);
     return __dadd_rn(__dadd_rn(__dmul_rn(ux, d0), __dmul_rn(uy, d1)), __dmul_rn(uz, d2));
+}
+
+// Bound of |delta32 - delta64| of point id (-1: the origin) along d: the operands
+// rounded to single, then three products and two sums.
+template <class C>
+__device__ __forceinline__ float delta_bound(const Stage<C> &sg, float vx, float vy, float vz, float f0, float f1,
+                                             float f2) {
+    return kDeltaErr * ((fabsf(vx) + fabsf(sg.vor[0])) * fabsf(f0) + (fabsf(vy) + fabsf(sg.vor[1])) * fabsf(f1) +
+                        (fabsf(vz) + fabsf(sg.vor[2])) * fabsf(f2));
+}
+
+// Bound E of |chi32 - chi64| at every sample of the interval to the point in
+// `slot` (both ends included), from the errors of delta (dea, deb at its ends,
+// interpolation), dv, the profile constants, the profile argument, ex2 and the
+// sums:
+//   |g32 - g64| <= 0.7142 |da'| + 0.7358 rho + u/e + eps_ex2
+// (0.7142 = max |d/da 2^(-a^2)|, 0.7358 = max |a d/da 2^(-a^2)|).  The error
+// of a grows with |A|; far: the |a| beyond which bins need not be covered
+// (infinite: every bin of the warp is).
+template <class C>
+__device__ __forceinline__ float opacity_bound(const Stage<C> &sg, int slot, float dea, float deb, float far) {
+    const int pa = slot - 1;
+    const float k6 = 6.f * kU + kERcp;  // interpolation in single precision
+    const float wa = sg.w[pa], wb = sg.w[slot], ada = fabsf(sg.d[pa]), adb = fabsf(sg.d[slot]);
+    const float dmax = fmaxf(ada, adb);
+    const float edi = dea + deb + k6 * (ada + adb);
+    const float rdvmin = 1.f / fminf(wa, wb);
+    const float rho = kERcp + k6 * (wa + wb) * rdvmin + 4.f * kU;
+    const float wfar = far * fmaxf(wa, wb);
+    float E = 0.f, csum = fmaxf(sg.cc[pa], sg.cc[slot]);
+#pragma unroll
+    for (int l = 0; l < C::NL; ++l) {
+        const float Am = fminf(sg.Am[l], sg.Bm[l] * dmax + wfar);
+        const float dA = (3.f * kU * (Am + sg.Bm[l] * dmax) + sg.Bm[l] * edi) * rdvmin * (1.f + rho);
+        const float Eg = 0.7142f * dA + 0.7358f * rho * 1.001f + 0.3679f * kU + kEEx2 + 2.f * dA * dA;
+        const float c0a = sg.ce[2 * l][pa], c0b = sg.ce[2 * l][slot], c0m = fmaxf(c0a, c0b);
+        E += c0m * Eg + k6 * (c0a + c0b) + kU * c0m;
+        csum += c0m;
+    }
+    E += k6 * (sg.cc[pa] + sg.cc[slot]) + kU * fmaxf(sg.cc[pa], sg.cc[slot]) + float(C::NL + 1) * kU * csum;
+    return E * 1.0625f;
 }
 
 // ---- double-precision redo of the single-precision form's decisions ------
@@ -471,9 +590,11 @@ __device__ __noinline__ int redo_n_inter(const DevMesh &m, const DevLines &Ln, c
 // Point q of the half (q < cnt: traced entry cnt-1-q, far end first; q == cnt:
 // the origin) into `slot`; its exact Z and (single precision) the bound of
 // its delta's error are also returned, for the interval to it.
-template <typename R, int NL>
-__device__ __forceinline__ void stage_point(const DevMesh &m, const DevLines &Ln, Stage<R, NL> &sg, int32_t q,
-                                            int32_t cnt, int slot, int sign, double &zq, R &deq) {
+template <class C>
+__device__ __forceinline__ void stage_point(const DevMesh &m, const DevLines &Ln, Stage<C> &sg, int32_t q, int32_t cnt,
+                                            int slot, int sign, double &zq, typename C::R &deq) {
+    using R = typename C::R;
+    constexpr int NL = C::NL;
     const HalfList &hl = sg.hl;
     const double sgn = double(sign);
     const int32_t L = Ln.L;
@@ -494,8 +615,7 @@ __device__ __forceinline__ void stage_point(const DevMesh &m, const DevLines &Ln
             const float vx = __ldg(Pts<R>::vx(m) + id), vy = __ldg(Pts<R>::vy(m) + id), vz = __ldg(Pts<R>::vz(m) + id);
             const float ux = vx - sg.vor[0], uy = vy - sg.vor[1], uz = vz - sg.vor[2];
             d = fmaf(uz, f2, fmaf(uy, f1, ux * f0));
-            de = kDeltaErr * ((fabsf(vx) + fabsf(sg.vor[0])) * fabsf(f0) + (fabsf(vy) + fabsf(sg.vor[1])) * fabsf(f1) +
-                              (fabsf(vz) + fabsf(sg.vor[2])) * fabsf(f2));
+            de = delta_bound<C>(sg, vx, vy, vz, f0, f1, f2);
         }
     }
     sg.id[slot] = q < cnt ? id : -1;
@@ -518,10 +638,12 @@ __device__ __forceinline__ void stage_point(const DevMesh &m, const DevLines &Ln
 // the constants of Eq. 2 with the bound on the opacity's error.  za, zb are
 // the exact Z of the farther and the nearer point, dea, deb the bounds of
 // their deltas' errors (single precision).
-template <typename R, int NL>
-__device__ __forceinline__ int stage_interval(const DevMesh &m, const DevLines &Ln, const SolveArgs &a,
-                                              Stage<R, NL> &sg, int slot, int sign, double za, double zb, R dea,
-                                              R deb) {
+template <class C>
+__device__ __forceinline__ int stage_interval(const DevMesh &m, const DevLines &Ln, const SolveArgs &a, Stage<C> &sg,
+                                              int slot, int sign, double za, double zb, typename C::R dea,
+                                              typename C::R deb) {
+    using R = typename C::R;
+    constexpr int NL = C::NL;
     const int pa = slot - 1;
     if constexpr (sizeof(R) == 8) {
         // as defined: ceil(|delta_b - delta_a| / (dv_max min(dv_a, dv_b))) when that exceeds one
@@ -566,37 +688,16 @@ __device__ __forceinline__ int stage_interval(const DevMesh &m, const DevLines &
         const float ds = float(za - zb);  // distance increment, differenced in double
         const float rn = 1.f / float(nv);
         const float hs = ds * rn;
-        // Bound E of |chi32 - chi64| at every sample of the interval (both
-        // ends included), from the errors of delta (de, interpolation), dv,
-        // the profile constants, the profile argument, ex2 and the sums:
-        //   |g32 - g64| <= 0.7142 |da'| + 0.7358 rho + u/e + eps_ex2
-        // (0.7142 = max |d/da 2^(-a^2)|, 0.7358 = max |a d/da 2^(-a^2)|).
-        const float k6 = 6.f * kU + kERcp;  // interpolation in single precision
-        const float ada = fabsf(da), adb = fabsf(db);
-        const float dmax = fmaxf(ada, adb);
-        const float edi = dea + deb + k6 * (ada + adb);
-        const float rdvmin = 1.f / fminf(wa, wb);
-        const float rho = kERcp + k6 * (wa + wb) * rdvmin + 4.f * kU;
-        float E = 0.f, csum = fmaxf(sg.cc[pa], sg.cc[slot]);
-#pragma unroll
-        for (int l = 0; l < NL; ++l) {
-            const float dA = (3.f * kU * (sg.Am[l] + sg.Bm[l] * dmax) + sg.Bm[l] * edi) * rdvmin * (1.f + rho);
-            const float Eg = 0.7142f * dA + 0.7358f * rho * 1.001f + 0.3679f * kU + kEEx2 + 2.f * dA * dA;
-            const float c0a = sg.ce[2 * l][pa], c0b = sg.ce[2 * l][slot], c0m = fmaxf(c0a, c0b);
-            E += c0m * Eg + k6 * (c0a + c0b) + kU * c0m;
-            csum += c0m;
-        }
-        E += k6 * (sg.cc[pa] + sg.cc[slot]) + kU * fmaxf(sg.cc[pa], sg.cc[slot]) + float(NL + 1) * kU * csum;
-        E *= 1.0625f;
+        const float E = opacity_bound<C>(sg, slot, dea, deb, INFINITY);
         // Eq. 2: n_inter = max(1, ceil(fl(fl(chi64 ds64) / dtau_max))); ds64, the
         // definition's sample spacing, is within (3u + rho_s) of hs, rho_s the
         // rounding of its interpolated distances (8 u64 max|Z| / hs)
         const float zmax = float(fmax(za, zb));
         const float kap = 15.f * kU + 9.0e-16f * zmax / hs + 1e-15f;
         const float dtm = float(a.dtau_max);
-        const float qs = hs * float(1.0 / a.dtau_max);
         sg.hq[slot] = 0.5f * hs;
         sg.thr[slot] = (dtm / hs) * (1.f - kap) - E * (1.f + 4.f * kU);
+        const float qs = hs * float(1.0 / a.dtau_max);
         sg.qlo[slot] = qs * (1.f - kap);
         sg.qhi[slot] = qs * (1.f + kap);
         sg.E[slot] = E;
@@ -604,69 +705,113 @@ __device__ __forceinline__ int stage_interval(const DevMesh &m, const DevLines &
     }
 }
 
-// Record of sample s_abs of the chunk (relative to its first) into record s_rec.
-template <typename R, int NL>
-__device__ __forceinline__ void gen_sample(Stage<R, NL> &sg, int s_abs, int s_rec, int nch, int sign,
-                                           double dtau_max) {
-    constexpr int kS = Stage<R, NL>::kS;
-    int lo = 1, hi = nch;  // the last slot whose samples start at or before s_abs
+// Whether line l takes no part in a sample of single precision, bit for bit:
+// every bin of the warp gets chi = fma(c0, g, chi) = chi and eta likewise.
+// A and B of the warp's bins lie in [wA[0], wA[1]] and [wB[0], wB[1]], and
+// rounding is monotone, so fl(fl(B delta + A) rdv) of every bin lies between
+// the same expression at the ends.  With |a| >= t on one side of zero,
+// g <= 2^-t^2 (1 + kEEx2), and a product c0 g below half an ulp of chi, at
+// least 2^-25 cc, rounds away: t^2 = 25.05 + log2(c0 / cc), likewise for eta,
+// the margin covering lg2.approx, rcp.approx and this evaluation.  From
+// |a| = 12.1 on ex2.approx.ftz(-a^2) is exactly 0, whatever the ratios.  On
+// the 50 000-point wind the far wing then starts at |a'| of about 6.2
+// instead of 12.1.
+__device__ __forceinline__ bool line_is_far(float dl, float rdv, float cc, float ec, float c0, float e0,
+                                            const float *wA, const float *wB) {
+    if (c0 == 0.f && e0 == 0.f) return true;
+    const float lo = fmaf(dl >= 0.f ? wB[0] : wB[1], dl, wA[0]) * rdv;
+    const float hi = fmaf(dl >= 0.f ? wB[1] : wB[0], dl, wA[1]) * rdv;
+    const float re = e0 > 0.f ? e0 * Ar<float>::rcp(ec) : 0.f;
+    const float x = fmaxf(fmaxf(c0 * Ar<float>::rcp(cc), re), 1e-30f);
+    const float t = fminf(sqrtf(fmaxf(25.05f + __log2f(x), 0.f)) * 1.0001f, 12.1f);
+    return lo >= t || hi <= -t;
+}
+
+// The slot whose interval holds sample s_abs of the chunk: the last one whose
+// samples start at or before it.
+template <class C>
+__device__ __forceinline__ int slot_of(const Stage<C> &sg, int s_abs, int nch) {
+    int lo = 1, hi = nch;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (sg.so[mid] <= s_abs) lo = mid;
         else hi = mid - 1;
     }
-    const int k = lo, nv = sg.nv[k], j = s_abs - sg.so[k] + 1;
-    R *o = sg.rec + s_rec * kS;
-    sg.sk[s_rec] = k | (j << 6);
+    return lo;
+}
+
+// Record of sample s_abs of the chunk (relative to its first) into record s_rec.
+// Returns (packed form) the mask of the lines that take part, bit 31 set when some bin may need a split.
+template <class C>
+__device__ __forceinline__ unsigned gen_sample(Stage<C> &sg, int s_abs, int s_rec, int nch, int sign,
+                                               double dtau_max) {
+    using R = typename C::R;
+    constexpr int NL = C::NL;
+    constexpr int kS = Stage<C>::kS;
+    const int k = slot_of<C>(sg, s_abs, nch), nv = sg.nv[k], j = s_abs - sg.so[k] + 1;
+    sg.sk[s_rec] = (unsigned char)k;
     if constexpr (sizeof(R) == 4) {
         const int pa = k - 1;
-        float wv;
+        float wv, dl, cc, ec, ce[2 * NL];
         if (j == nv) {
-            o[0] = sg.d[k];
+            dl = sg.d[k];
             wv = sg.w[k];
-            o[2] = sg.cc[k];
-            o[3] = sg.ec[k];
+            cc = sg.cc[k];
+            ec = sg.ec[k];
 #pragma unroll
-            for (int c = 0; c < 2 * NL; ++c) o[6 + c] = sg.ce[c][k];
+            for (int c = 0; c < 2 * NL; ++c) ce[c] = sg.ce[c][k];
         } else {
             const float t = float(j) * (1.f / float(nv));  // rn of the interval, formed again
-            o[0] = fmaf(sg.d[k] - sg.d[pa], t, sg.d[pa]);
+            dl = fmaf(sg.d[k] - sg.d[pa], t, sg.d[pa]);
             wv = fmaf(sg.w[k] - sg.w[pa], t, sg.w[pa]);
-            o[2] = fmaf(sg.cc[k] - sg.cc[pa], t, sg.cc[pa]);
-            o[3] = fmaf(sg.ec[k] - sg.ec[pa], t, sg.ec[pa]);
+            cc = fmaf(sg.cc[k] - sg.cc[pa], t, sg.cc[pa]);
+            ec = fmaf(sg.ec[k] - sg.ec[pa], t, sg.ec[pa]);
 #pragma unroll
-            for (int c = 0; c < 2 * NL; ++c) o[6 + c] = fmaf(sg.ce[c][k] - sg.ce[c][pa], t, sg.ce[c][pa]);
+            for (int c = 0; c < 2 * NL; ++c) ce[c] = fmaf(sg.ce[c][k] - sg.ce[c][pa], t, sg.ce[c][pa]);
         }
-        o[1] = Ar<float>::rcp(wv);
-        if constexpr (NL == 1) {
-            // far wing: when every bin's profile argument a = fl(fl(B delta + A) rdv)
-            // has a^2 >= 128, ex2.approx.ftz(-a^2) is exactly 0 and the optics are
-            // the continuum's (bit for bit).  A and B rise with the bin, so over the
-            // tile B delta + A lies in [min(tf, tl) - W, max(tf, tl) + W] with
-            // W = (B_last - B_first) |delta|; |a| >= 12.1 leaves margin for every
-            // rounding.  The record carries the outcome as a negative 1/dv.
-            if (sg.wing) {
-                const float dl = o[0];
-                const float tf = fmaf(sg.wb[0], dl, sg.wa[0]), tl = fmaf(sg.wb[1], dl, sg.wa[1]);
-                const float W = 1.01f * (sg.wb[1] - sg.wb[0]) * fabsf(dl);
-                const float lo = (fminf(tf, tl) - W) * o[1], hi = (fmaxf(tf, tl) + W) * o[1];
-                if (lo >= 12.1f || hi <= -12.1f) o[1] = -o[1];
+        const float rdv = Ar<float>::rcp(wv);
+        // no bin can split anywhere on the interval when the largest opacity any
+        // sample of it (or the point before it) can reach, continuum plus line
+        // centres (the profile is at most 1; interpolation and the fused sums
+        // round within (4 + NL) u), stays below the threshold: the record says so
+        // with an infinite threshold and the step skips the vote
+        float thr = sg.thr[k];
+        float cb = fmaxf(sg.cc[pa], sg.cc[k]);
+#pragma unroll
+        for (int l = 0; l < NL; ++l) cb += fmaxf(sg.ce[2 * l][pa], sg.ce[2 * l][k]);
+        if (cb * (1.f + (8 + 2 * NL) * kU) <= thr) thr = INFINITY;
+        unsigned on = 0;  // the lines that take part
+#pragma unroll
+        for (int l = 0; l < NL; ++l)
+            if (!line_is_far(dl, rdv, cc, ec, ce[2 * l], ce[2 * l + 1], sg.wA[l], sg.wB[l])) on |= 1u << l;
+        if constexpr (C::kPacked) {
+            float4 *o = reinterpret_cast<float4 *>(sg.rec + s_rec * kS);
+            o[0] = make_float4(dl, dl, rdv, rdv);
+            o[1] = make_float4(cc, cc, ec, ec);
+            o[2] = make_float4(sg.hq[k], sg.hq[k], thr, __uint_as_float(on));
+#pragma unroll
+            for (int l = 0; l < NL; ++l) {
+                if constexpr (Rec<C>::kTwice)
+                    o[3 + l] = make_float4(ce[2 * l], ce[2 * l], ce[2 * l + 1], ce[2 * l + 1]);
+                else
+                    reinterpret_cast<float2 *>(o + 3)[l] = make_float2(ce[2 * l], ce[2 * l + 1]);
             }
-        }
-        o[4] = sg.hq[k];
-        o[5] = sg.thr[k];
-        if constexpr (NL == 1) {
-            // no bin can split anywhere on the interval when the largest opacity any
-            // sample of it (or the point before it) can reach, continuum plus line
-            // centre (the profile is at most 1; interpolation and the fused sums
-            // round within 4u), stays below the threshold: the record says so
-            // with an infinite threshold and the step skips the vote
-            const float cb = fmaxf(sg.cc[pa], sg.cc[k]) + fmaxf(sg.ce[0][pa], sg.ce[0][k]);
-            if (cb * (1.f + 8.f * kU) <= o[5]) o[5] = INFINITY;
+            return on | (thr != INFINITY ? 0x80000000u : 0u);
+        } else {
+            R *o = sg.rec + s_rec * kS;
+            o[0] = dl;
+            o[1] = NL == 1 && on == 0 ? -rdv : rdv;
+            o[2] = cc;
+            o[3] = ec;
+            o[4] = sg.hq[k];
+            o[5] = thr;
+#pragma unroll
+            for (int c = 0; c < 2 * NL; ++c) o[6 + c] = ce[c];
         }
     } else {
         // the definition's layout: samples interpolated from the earlier point
         // along +r with t = i / nv, exact end points; ds between consecutive samples
+        R *o = sg.rec + s_rec * kS;
         const bool bwd = sign < 0;
         const double sgn = double(sign);
         const int b0 = bwd ? k - 1 : k, b1 = bwd ? k : k - 1;
@@ -689,12 +834,13 @@ __device__ __forceinline__ void gen_sample(Stage<R, NL> &sg, int s_abs, int s_re
         o[4] = 0.5 * ds;
         o[5] = (dtau_max / ds) * (1.0 - 0x1p-40);  // chi below this gives n_inter = 1
     }
+    return 0u;
 }
 
-template <typename R, int NL>
-__device__ __forceinline__ void load_rec(const R *src, R (&v)[Stage<R, NL>::kS]) {
-    constexpr int kS = Stage<R, NL>::kS;
-    if constexpr (sizeof(R) == 4) {
+template <class C>
+__device__ __forceinline__ void load_rec(const typename C::V *src, typename C::V (&v)[Stage<C>::kS]) {
+    constexpr int kS = Stage<C>::kS;
+    if constexpr (sizeof(typename C::V) == 4) {
 #pragma unroll
         for (int c = 0; c < kS / 4; ++c) {
             const float4 t = reinterpret_cast<const float4 *>(src)[c];
@@ -717,14 +863,15 @@ __device__ __forceinline__ void load_rec(const R *src, R (&v)[Stage<R, NL>::kS])
 // threshold.  Double precision: as defined.  Single precision: certified from
 // the bound E; 0 when the bound leaves the integer open (the caller has it
 // redone in double precision).
-template <typename R, int NL>
-__device__ __forceinline__ int n_inter(R cm, R hq, int s, const Stage<R, NL> &sg, const SolveArgs &a) {
+template <class C>
+__device__ __forceinline__ int n_inter(typename C::R cm, typename C::R hq, int k, const Stage<C> &sg,
+                                       const SolveArgs &a) {
+    using R = typename C::R;
     int n;
     if constexpr (sizeof(R) == 8) {
         const double nr = ceil((cm * (hq + hq)) / a.dtau_max);
         n = nr > double(kMaxSubdiv) ? kMaxSubdiv + 1 : nr <= 1.0 ? 1 : int(nr);
     } else {
-        const int k = sg.sk[s] & 63;
         const float E = sg.E[k];
         const float nhi = ceilf((cm + E) * sg.qhi[k]);
         if (nhi <= 1.f) return 1;
@@ -740,18 +887,44 @@ __device__ __forceinline__ int n_inter(R cm, R hq, int s, const Stage<R, NL> &sg
 }
 
 // The Eq. 2 counts of sample s that its single-precision bound left open
-// (sg.fix[i][lane] == -1), redone in double precision into sg.fix.  Out of
-// line and outside the elimination loop, which it interrupts only for such a
-// sample: a call inside the loop would cost the loop its registers.
-template <typename R, int NL>
-__device__ __noinline__ void resolve_n_inter(Stage<R, NL> &sg, const DevMesh &m, const DevLines &Ln,
-                                             const SolveArgs &a, int sign, int s, int32_t bin0, int32_t bin1) {
+// (sg.fix[i][lane] < 0), resolved into sg.fix: by a tighter bound, which leaves
+// out the bins on which the line has no part (|a| >= 12.1, g = 0 in single
+// precision and below 2^-146 in double), else in double precision.  With
+// several lines the loop's bound carries their distance, hundreds of widths:
+// on a two-line octree of 20 000 leaves the tighter one decides two thirds of
+// the 5.6e5 open counts of a pass.  Out of line and outside the elimination
+// loop, which it interrupts only for such a sample: a call inside the loop
+// would cost the loop its registers.
+template <class C>
+__device__ __noinline__ void resolve_n_inter(Stage<C> &sg, const DevMesh &m, const DevLines &Ln, const SolveArgs &a,
+                                             int sign, int s_abs) {
     const int lane = threadIdx.x & 31;
-    const int sk = sg.sk[s], k = sk & 63, j = sk >> 6;
+    const int k = sg.sk[s_abs % Stage<C>::kCap], j = s_abs - sg.so[k] + 1;
 #pragma unroll 1
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < C::BPL; ++i) {
         if (sg.fix[i][lane] >= 0) continue;
-        const int32_t b = i == 0 ? bin0 : bin1;
+        if constexpr (sizeof(typename C::R) == 4) {
+            const float cm = __int_as_float(sg.fix[i][lane] & 0x7fffffff);
+            const float f0 = float(sg.r[0]), f1 = float(sg.r[1]), f2 = float(sg.r[2]);
+            float de[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int id = sg.id[k - 1 + e];
+                de[e] = id < 0 ? 0.f : delta_bound<C>(sg, __ldg(m.vxf + id), __ldg(m.vyf + id), __ldg(m.vzf + id), f0, f1, f2);
+            }
+            const float E = opacity_bound<C>(sg, k, de[0], de[1], 12.25f);
+            const float nhi = ceilf((cm + E) * sg.qhi[k]), nlo = ceilf((cm - E) * sg.qlo[k]);
+            if (nhi <= 1.f || nlo == nhi) {
+                int n = nhi <= 1.f ? 1 : nhi > float(kMaxSubdiv) ? kMaxSubdiv + 1 : int(nhi);
+                if (n > kMaxSubdiv) {
+                    dev_fail(a.status, kDevSubdivLimit);
+                    n = kMaxSubdiv;
+                }
+                sg.fix[i][lane] = n;
+                continue;
+            }
+        }
+        const int32_t b = lane_bin<C>(sg, i, lane);
         int n = redo_n_inter(m, Ln, sg.r, sg.vo, sg.o, double(sign), sg.id[k - 1], sg.id[k], sg.nv[k], j,
                              b < sg.NB ? b : sg.NB - 1, a.dtau_max);
         if (n > kMaxSubdiv) {
@@ -764,23 +937,186 @@ __device__ __noinline__ void resolve_n_inter(Stage<R, NL> &sg, const DevMesh &m,
     __syncwarp();
 }
 
-// One velocity sample (record v, index s of the round) for every bin of the
+// The split counts (Eq. 2) of the lane's bins at a sample where some bin of
+// the warp may need more than one.  Returns false, with the open bins marked
+// in sg.fix, when a single-precision count is left open somewhere in the warp.
+template <class C>
+__device__ __forceinline__ bool split_counts(typename C::R hq, typename C::R thr, int s_abs, bool fixed,
+                                             Stage<C> &sg, const SolveArgs &a, const typename C::V (&chi_q)[C::NV],
+                                             const Sweep<typename C::V, typename C::W> (&w)[C::NV],
+                                             int (&nis)[C::BPL]) {
+    using R = typename C::R;
+    const int lane = threadIdx.x & 31;
+    const int k = sg.sk[s_abs % Stage<C>::kCap];
+    bool open = false;
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) {
+        const R cm = fmax(vget(w[i / C::kIn].chi, i % C::kIn), vget(chi_q[i / C::kIn], i % C::kIn));
+        int n = 1;
+        if (cm > thr) {
+            n = (fixed && sg.fix[i][lane] > 0) ? sg.fix[i][lane] : n_inter<C>(cm, hq, k, sg, a);
+            open |= n == 0;
+        }
+        nis[i] = n;
+        if constexpr (sizeof(R) == 4) {
+            if (n == 0) nis[i] = __float_as_int(-cm);
+        }
+    }
+    if constexpr (sizeof(R) == 4) {
+        if (__any_sync(kFull, open)) {
+#pragma unroll
+            for (int i = 0; i < C::BPL; ++i) sg.fix[i][lane] = nis[i] < 0 ? nis[i] : 0;
+            __syncwarp();
+            return false;
+        }
+    }
+    if (a.counters) {  // (uniform) only while profiling
+        unsigned extra = 0;
+#pragma unroll
+        for (int i = 0; i < C::BPL; ++i)
+            if (lane_bin<C>(sg, i, lane) < sg.NB) extra += unsigned(nis[i] - 1);
+        extra = __reduce_add_sync(kFull, extra);
+        if (lane == 0) sg.n_extra += extra;
+    }
+    return true;
+}
+
+// Packed form: words of a record, as pairs.
+__device__ __forceinline__ void load_pair(const float2 *src, float2 &a, float2 &b) {
+    const float4 t = *reinterpret_cast<const float4 *>(src);
+    a = make_float2(t.x, t.y);
+    b = make_float2(t.z, t.w);
+}
+
+// Packed form: the part of line l in a sample (record src) for every bin of
+// the lane, A and B its profile constants.
+template <class C>
+__device__ __forceinline__ void one_line(const float2 *src, int l, float2 delta, float2 rdv, const float2 (&A)[C::NV],
+                                         const float2 (&B)[C::NV], float2 (&chi_q)[C::NV], float2 (&eta_q)[C::NV]) {
+    float2 c0, e0;
+    if constexpr (Rec<C>::kTwice) {
+        load_pair(src + 6 + 2 * l, c0, e0);
+    } else {
+        const float2 t = src[6 + l];
+        c0 = make_float2(t.x, t.x);
+        e0 = make_float2(t.y, t.y);
+    }
+#pragma unroll
+    for (int i = 0; i < C::NV; ++i) add_line(delta, rdv, c0, e0, A[i], B[i], chi_q[i], eta_q[i]);
+}
+
+// Packed form: total opacity and emissivity of a sample for every bin of the
+// lane, over the lines that take part (mask `on`, uniform over the warp).
+template <class C>
+__device__ __forceinline__ void all_lines(const float2 *src, unsigned on, const Stage<C> &sg, float2 (&chi_q)[C::NV],
+                                          float2 (&eta_q)[C::NV]) {
+    const int lane = threadIdx.x & 31;
+    float2 delta, rdv, cc, ec;
+    load_pair(src, delta, rdv);
+    load_pair(src + 2, cc, ec);
+#pragma unroll
+    for (int i = 0; i < C::NV; ++i) {
+        chi_q[i] = cc;
+        eta_q[i] = ec;
+    }
+#pragma unroll 1
+    for (; on; on &= on - 1) {
+        const int l = C::NL == 1 ? 0 : __ffs(on) - 1;
+        float2 A[C::NV], B[C::NV];
+#pragma unroll
+        for (int i = 0; i < C::NV; ++i) {
+            A[i] = sg.fA[l][i][lane];
+            B[i] = sg.fB[l][i][lane];
+        }
+        one_line<C>(src, l, delta, rdv, A, B, chi_q, eta_q);
+    }
+}
+
+// Packed form: the rows of a sample without sub-intervals (hq: half its spacing).
+template <class C>
+__device__ __forceinline__ void rows_to(float2 hq, const float2 (&chi_q)[C::NV], const float2 (&eta_q)[C::NV],
+                                        Sweep<float2> (&w)[C::NV]) {
+#pragma unroll
+    for (int i = 0; i < C::NV; ++i) {
+        row2(w[i], w[i].chi, w[i].eta, vmul(hq, vadd(w[i].chi, chi_q[i])));
+        w[i].chi = chi_q[i];
+        w[i].eta = eta_q[i];
+    }
+}
+
+// Packed form: one velocity sample (record src, sample s_abs of the chunk) of an
+// interval on which some bin may need sub-intervals (Eq. 2, chi and eta
+// linear).  Returns false, with nothing changed but the bins marked in sg.fix,
+// when a count is left open somewhere in the warp; once it has been redone the
+// sample is stepped again with `fixed` set, taking the counts from sg.fix.
+template <class C>
+__device__ __forceinline__ bool split_step(const float2 *src, int s_abs, bool fixed, Stage<C> &sg,
+                                           const SolveArgs &a, Sweep<float2> (&w)[C::NV]) {
+    float2 hq, tm;
+    load_pair(src + 4, hq, tm);
+    const float thr = tm.x;
+    float2 chi_q[C::NV], eta_q[C::NV];
+    all_lines<C>(src, __float_as_uint(tm.y), sg, chi_q, eta_q);
+    float cm = 0.f;
+#pragma unroll
+    for (int i = 0; i < C::NV; ++i)
+        cm = fmaxf(cm, fmaxf(fmaxf(w[i].chi.x, w[i].chi.y), fmaxf(chi_q[i].x, chi_q[i].y)));
+    if (!__any_sync(kFull, cm > thr)) {
+        rows_to<C>(hq, chi_q, eta_q, w);
+        return true;
+    }
+    int nis[C::BPL];
+    if (!split_counts<C>(hq.x, thr, s_abs, fixed, sg, a, chi_q, w, nis)) return false;
+    // the sub-intervals of both bins of a value side by side, each bin taking its first n
+#pragma unroll
+    for (int i = 0; i < C::NV; ++i) {
+        const int nx = nis[2 * i], ny = nis[2 * i + 1], n = nx > ny ? nx : ny;
+        const float2 rni = make_float2(1.f / float(nx), 1.f / float(ny));
+        const float2 hh = vmul(hq, rni);
+        const float2 c0 = w[i].chi, e0 = w[i].eta;
+        const float2 dchi = make_float2((chi_q[i].x - c0.x) * rni.x, (chi_q[i].y - c0.y) * rni.y);
+        const float2 deta = make_float2((eta_q[i].x - e0.x) * rni.x, (eta_q[i].y - e0.y) * rni.y);
+        float2 cprev = c0, eprev = e0;
+#pragma unroll 1
+        for (int k = 1; k <= n; ++k) {
+            const float2 fk = make_float2(float(k), float(k));
+            float2 ck = vfma(dchi, fk, c0), ek = vfma(deta, fk, e0);
+            if (k >= nx) ck.x = chi_q[i].x, ek.x = eta_q[i].x;
+            if (k >= ny) ck.y = chi_q[i].y, ek.y = eta_q[i].y;
+            Sweep<float2> t = w[i];
+            row2(t, cprev, eprev, vmul(hh, vadd(cprev, ck)));
+            if (k <= nx) w[i].Fh.x = t.Fh.x, w[i].Dm.x = t.Dm.x, w[i].dtp.x = t.dtp.x, w[i].zh.x = t.zh.x;
+            if (k <= ny) w[i].Fh.y = t.Fh.y, w[i].Dm.y = t.Dm.y, w[i].dtp.y = t.dtp.y, w[i].zh.y = t.zh.y;
+            cprev = ck;
+            eprev = ek;
+        }
+        w[i].chi = chi_q[i];
+        w[i].eta = eta_q[i];
+    }
+    return true;
+}
+
+// The other forms: one velocity sample (record v, sample s_abs of the chunk) for every bin of the
 // lane: line optics, Eq. 2 sub-intervals with linear chi and eta, elimination
 // rows.  When no bin of the warp can need sub-intervals (the common case) the
 // rows run as straight-line code, so the bins' chains interleave.  Single
-// precision tests "possibly more than one sub-interval" on the lane's running
-// maximum of chi over its bins (cmax: the previous sample's, updated here)
-// against the certified threshold; double precision per bin.  Returns false,
-// with nothing changed, when a single-precision count is left open somewhere
-// in the warp (sg.fix marks it); once it has been redone the sample is
-// stepped again with `fixed` set, taking the counts from sg.fix.
-template <typename R, int NL, int BPL, int ORD, typename P>
-__device__ __forceinline__ bool sample_step(const R (&v)[Stage<R, NL>::kS], int s, bool fixed, Stage<R, NL> &sg,
-                                            const SolveArgs &a, R &cmax, const Bin<R, NL> (&f)[BPL],
-                                            const bool (&act)[BPL], Sweep<R, P> (&w)[BPL]) {
+// precision tests "possibly more than one sub-interval" on the lane's maximum
+// of chi over its bins (this sample's and the previous one's) against the
+// certified threshold; double precision per bin.  Returns false, with nothing
+// changed, when a single-precision count is left open somewhere in the warp
+// (sg.fix marks it); once it has been redone the sample is stepped again with
+// `fixed` set, taking the counts from sg.fix.
+template <class C>
+__device__ __forceinline__ bool sample_step(const typename C::V (&v)[Stage<C>::kS], int s_abs, bool fixed, Stage<C> &sg,
+                                            const SolveArgs &a, const Bin<typename C::V, C::NL> (&f)[C::NV],
+                                            Sweep<typename C::V, typename C::W> (&w)[C::NV]) {
+    using R = typename C::R;
+    using P = typename C::P;
+    constexpr int NL = C::NL;
+    constexpr int BPL = C::BPL, ORD = C::ORD;
     const R dl = v[0], rdv = v[1], hq = v[4], thr = v[5];
     R chi_q[BPL], eta_q[BPL];
-    if (sizeof(R) == 4 && NL == 1 && rdv < R(0)) {  // far wing of every bin: the continuum (as ex2 gives 0)
+    if (sizeof(R) == 4 && NL == 1 && rdv < R(0)) {  // the line takes no part: the continuum
 #pragma unroll
         for (int i = 0; i < BPL; ++i) {
             chi_q[i] = v[2];
@@ -791,12 +1127,14 @@ __device__ __forceinline__ bool sample_step(const R (&v)[Stage<R, NL>::kS], int 
         for (int i = 0; i < BPL; ++i) optics<R, NL>(dl, rdv, v[2], v[3], v + 6, f[i], chi_q[i], eta_q[i]);
     }
     bool go;  // no bin needs a split (n_inter = 1 for all)
-    R cq = chi_q[0];
     if constexpr (sizeof(R) == 4) {
+        go = thr == R(INFINITY);  // uniform (the warp's record): no bin of the interval can split
+        if (!go) {
+            R cm = fmax(w[0].chi, chi_q[0]);
 #pragma unroll
-        for (int i = 1; i < BPL; ++i) cq = fmax(cq, chi_q[i]);
-        // an infinite threshold (uniform: the warp's record) means no bin of the interval can split
-        go = (NL == 1 && thr == R(INFINITY)) || !__any_sync(kFull, fmax(cmax, cq) > thr);
+            for (int i = 1; i < BPL; ++i) cm = fmax(cm, fmax(w[i].chi, chi_q[i]));
+            go = !__any_sync(kFull, cm > thr);
+        }
     } else {
         bool split = false;
 #pragma unroll
@@ -813,30 +1151,10 @@ __device__ __forceinline__ bool sample_step(const R (&v)[Stage<R, NL>::kS], int 
             w[i].eta = eta_q[i];
             w[i].Sc = Sq;
         }
-        cmax = cq;
         return true;
     }
-    const int lane = threadIdx.x & 31;
     int nis[BPL];
-    bool open = false;
-#pragma unroll
-    for (int i = 0; i < BPL; ++i) {
-        const R cm = fmax(w[i].chi, chi_q[i]);
-        int n = 1;
-        if (cm > thr) {
-            n = (fixed && sg.fix[i][lane] > 0) ? sg.fix[i][lane] : n_inter<R, NL>(cm, hq, s, sg, a);
-            open |= n == 0;
-        }
-        nis[i] = n;
-    }
-    if constexpr (sizeof(R) == 4) {
-        if (__any_sync(kFull, open)) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) sg.fix[i][lane] = (i < BPL && nis[i < BPL ? i : 0] == 0) ? -1 : 0;
-            __syncwarp();
-            return false;
-        }
-    }
+    if (!split_counts<C>(hq, thr, s_abs, fixed, sg, a, chi_q, w, nis)) return false;
 #pragma unroll
     for (int i = 0; i < BPL; ++i) {
         const int ni = nis[i];
@@ -861,24 +1179,24 @@ __device__ __forceinline__ bool sample_step(const R (&v)[Stage<R, NL>::kS], int 
         w[i].chi = chi_q[i];
         w[i].eta = eta_q[i];
         w[i].Sc = Sq;
-        if (act[i] && ni > 1) atomicAdd(&sg.n_extra, unsigned(ni - 1));
     }
-    cmax = cq;
     return true;
 }
 
 // The lane's sweep state to and from shared memory (D Fh kept as one value,
 // read back as Fh = D Fh, D = 1).
-template <typename R, int BPL, int ORD, typename P>
-__device__ __forceinline__ void put_sweep(Lane<R, ORD, P> &ln, const Sweep<R, P> (&w)[BPL], int lane) {
+template <class C>
+__device__ __forceinline__ void put_sweep(Lane<C> &ln, const Sweep<typename C::V, typename C::W> (&w)[C::NV],
+                                          int lane) {
 #pragma unroll
-    for (int i = 0; i < BPL; ++i) {
-        ln.wp[0][i][lane] = w[i].Dm * w[i].Fh;
+    for (int i = 0; i < C::NV; ++i) {
+        if constexpr (C::kPacked) ln.wp[0][i][lane] = vmul(w[i].Dm, w[i].Fh);
+        else ln.wp[0][i][lane] = w[i].Dm * w[i].Fh;
         ln.wp[1][i][lane] = w[i].dtp;
         ln.wr[0][i][lane] = w[i].zh;
         ln.wr[1][i][lane] = w[i].chi;
         ln.wr[2][i][lane] = w[i].eta;
-        if constexpr (ORD == 4) {
+        if constexpr (C::ORD == 4) {
             ln.wr[3][i][lane] = w[i].Sp;
             ln.wr[4][i][lane] = w[i].Sc;
             ln.wr[5][i][lane] = w[i].hp;
@@ -886,38 +1204,40 @@ __device__ __forceinline__ void put_sweep(Lane<R, ORD, P> &ln, const Sweep<R, P>
     }
 }
 
-template <typename R, int BPL, int ORD, typename P>
-__device__ __forceinline__ void get_sweep(const Lane<R, ORD, P> &ln, Sweep<R, P> (&w)[BPL], int lane) {
+template <class C>
+__device__ __forceinline__ void get_sweep(const Lane<C> &ln, Sweep<typename C::V, typename C::W> (&w)[C::NV],
+                                          int lane) {
+    using V = typename C::V;
+    using R = typename C::R;
 #pragma unroll
-    for (int i = 0; i < BPL; ++i) {
+    for (int i = 0; i < C::NV; ++i) {
         w[i].Fh = ln.wp[0][i][lane];
-        w[i].Dm = P(1);
+        w[i].Dm = vset<typename C::W>(1.f);
         w[i].dtp = ln.wp[1][i][lane];
         w[i].zh = ln.wr[0][i][lane];
         w[i].chi = ln.wr[1][i][lane];
         w[i].eta = ln.wr[2][i][lane];
-        if constexpr (ORD == 4) {
+        if constexpr (C::ORD == 4) {
             w[i].Sp = ln.wr[3][i][lane];
             w[i].Sc = ln.wr[4][i][lane];
             w[i].hp = ln.wr[5][i][lane];
             // the reciprocal of the last increment, formed again as the row formed it
             w[i].rh = w[i].hp < R(0) ? R(0) : Ar<R>::rcp(w[i].hp);
         } else {
-            w[i].Sp = w[i].Sc = w[i].hp = w[i].rh = R(0);
+            w[i].Sp = w[i].Sc = w[i].hp = w[i].rh = vset<V>(0.f);
         }
     }
 }
 
-template <typename R, int NL, int BPL>
-__device__ __forceinline__ void get_bins(const Stage<R, NL> &sg, Bin<R, NL> (&f)[BPL], bool (&act)[BPL], int lane) {
+template <class C>
+__device__ __forceinline__ void get_bins(const Stage<C> &sg, Bin<typename C::V, C::NL> (&f)[C::NV], int lane) {
 #pragma unroll
-    for (int i = 0; i < BPL; ++i) {
+    for (int i = 0; i < C::NV; ++i) {
 #pragma unroll
-        for (int l = 0; l < NL; ++l) {
+        for (int l = 0; l < C::NL; ++l) {
             f[i].A[l] = sg.fA[l][i][lane];
             f[i].B[l] = sg.fB[l][i][lane];
         }
-        act[i] = lane_bin<BPL>(sg, i, lane) < sg.NB;
     }
 }
 
@@ -930,44 +1250,120 @@ __device__ __forceinline__ void get_bins(const Stage<R, NL> &sg, Bin<R, NL> (&f)
 // (one call per chunk): its loop then gets a register allocation of its own,
 // unaffected by the calls of the code around it.  pend: a sample whose open
 // counts have been redone into sg.fix (-1: none).
-template <typename R, int NL, int BPL, int ORD, typename P>
-__device__ __noinline__ int consume_chunk(Stage<R, NL> &sg, Lane<R, ORD, P> &ln, const SolveArgs &a, int total,
-                                          int nch, int sign, int pos, int pend, bool fresh) {
-    constexpr int kS = Stage<R, NL>::kS, kCap = Stage<R, NL>::kCap;
+template <class C>
+__device__ __noinline__ int consume_chunk(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, int total, int nch, int sign,
+                                          int pos, int pend, bool fresh) {
+    constexpr int kS = Stage<C>::kS, kCap = Stage<C>::kCap;
     const int lane = threadIdx.x & 31;
-    Sweep<R, P> w[BPL];
-    Bin<R, NL> f[BPL];
-    bool act[BPL];
-    get_sweep<R, BPL, ORD, P>(ln, w, lane);
-    get_bins<R, NL, BPL>(sg, f, act, lane);
-    R cmax = ln.cm[lane];
+    Sweep<typename C::V, typename C::W> w[C::NV];
+    Bin<typename C::V, C::NL> f[C::NV];
+    get_sweep<C>(ln, w, lane);
+    if constexpr (!C::kPacked) get_bins<C>(sg, f, lane);
     int r0 = pos / kCap * kCap, s = pos - r0;
 #pragma unroll 1
     for (; r0 < total; r0 += kCap, s = 0, fresh = true) {
         const int nr = total - r0 < kCap ? total - r0 : kCap;
-        if (fresh) {
-#pragma unroll 1
-            for (int q = lane; q < nr; q += 32) gen_sample<R, NL>(sg, r0 + q, q, nch, sign, a.dtau_max);
-            __syncwarp();
-        }
+        if constexpr (C::kPacked) {
+            // the round in runs of records on which no bin can split and the same lines take
+            // part, so that the loops over the common classes (no line, one line) hold no
+            // branch and the compiler interleaves one sample's optics with another's rows
+            static_assert(kCap == 32, "one record per lane");
+            unsigned m_split, m_new;
+            if (fresh) {
+                const unsigned cls = lane < nr ? gen_sample<C>(sg, r0 + lane, lane, nch, sign, a.dtau_max) : 0u;
+                const unsigned up = __shfl_up_sync(kFull, cls, 1);
+                m_split = __ballot_sync(kFull, cls >> 31);
+                m_new = __ballot_sync(kFull, ((cls ^ up) & 0x7fffffffu) != 0u);
+                if (lane == 0) {
+                    sg.m_split = m_split;
+                    sg.m_new = m_new;
+                }
+                __syncwarp();
+            } else {
+                m_split = sg.m_split;
+                m_new = sg.m_new;
+            }
+            while (s < nr) {
+                const float2 *src = sg.rec + s * kS;
+                if ((m_split >> s) & 1u) {
+                    if (!split_step<C>(src, r0 + s, r0 + s == pend, sg, a, w)) break;
+                    ++s;
+                    continue;
+                }
+                // the run ends at the next record that may split or has other lines
+                const unsigned next = (m_split | m_new) & (0xfffffffeu << s);
+                const int e = next ? min(__ffs(int(next)) - 1, nr) : nr;
+                const float2 *end = sg.rec + e * kS;
+                s = e;
+                const unsigned on = __float_as_uint(src[5].y);
+                float2 chi_q[C::NV], eta_q[C::NV];
+                if (on == 0u) {
 #pragma unroll 2
-        for (; s < nr; ++s) {
-            R v[kS];
-            load_rec<R, NL>(sg.rec + s * kS, v);
-            if (!sample_step<R, NL, BPL, ORD, P>(v, s, r0 + s == pend, sg, a, cmax, f, act, w)) break;
+                    for (; src < end; src += kS) {
+                        float2 cc, ec;
+                        load_pair(src + 2, cc, ec);
+#pragma unroll
+                        for (int i = 0; i < C::NV; ++i) {
+                            chi_q[i] = cc;
+                            eta_q[i] = ec;
+                        }
+                        rows_to<C>(src[4], chi_q, eta_q, w);
+                    }
+                } else if (C::NL == 1 || (on & (on - 1)) == 0u) {
+                    const int l = C::NL == 1 ? 0 : __ffs(int(on)) - 1;
+                    float2 A[C::NV], B[C::NV];
+#pragma unroll
+                    for (int i = 0; i < C::NV; ++i) {
+                        A[i] = sg.fA[l][i][lane];
+                        B[i] = sg.fB[l][i][lane];
+                    }
+#pragma unroll 2
+                    for (; src < end; src += kS) {
+                        float2 delta, rdv, cc, ec;
+                        load_pair(src, delta, rdv);
+                        load_pair(src + 2, cc, ec);
+#pragma unroll
+                        for (int i = 0; i < C::NV; ++i) {
+                            chi_q[i] = cc;
+                            eta_q[i] = ec;
+                        }
+                        one_line<C>(src, l, delta, rdv, A, B, chi_q, eta_q);
+                        rows_to<C>(src[4], chi_q, eta_q, w);
+                    }
+                } else {
+#pragma unroll 1
+                    for (; src < end; src += kS) {
+                        all_lines<C>(src, on, sg, chi_q, eta_q);
+                        rows_to<C>(src[4], chi_q, eta_q, w);
+                    }
+                }
+            }
+        } else {
+            if (fresh) {
+#pragma unroll 1
+                for (int q = lane; q < nr; q += 32) gen_sample<C>(sg, r0 + q, q, nch, sign, a.dtau_max);
+                __syncwarp();
+            }
+#pragma unroll 2
+            for (; s < nr; ++s) {
+                typename C::V v[kS];
+                load_rec<C>(sg.rec + s * kS, v);
+                if (!sample_step<C>(v, r0 + s, r0 + s == pend, sg, a, f, w)) break;
+            }
         }
         if (s < nr) break;
         __syncwarp();
     }
-    put_sweep<R, BPL, ORD, P>(ln, w, lane);
-    ln.cm[lane] = cmax;
+    put_sweep<C>(ln, w, lane);
     __syncwarp();
     return r0 < total ? r0 + s : total;
 }
 
 // Copy the point data of slot `from` into slot 0 (the next chunk's farther point).
-template <typename R, int NL>
-__device__ __forceinline__ void carry_slot(Stage<R, NL> &sg, int from) {
+template <class C>
+__device__ __forceinline__ void carry_slot(Stage<C> &sg, int from) {
+    using R = typename C::R;
+    constexpr int NL = C::NL;
     sg.d[0] = sg.d[from];
     sg.w[0] = sg.w[from];
     sg.cc[0] = sg.cc[from];
@@ -983,9 +1379,10 @@ __device__ __forceinline__ void carry_slot(Stage<R, NL> &sg, int from) {
 // their velocity samples.  Returns the chunk's number of samples.  Called once
 // per 32 points and kept out of line, so that its double-precision and bound
 // arithmetic does not add to the registers of the elimination loop.
-template <typename R, int NL>
-__device__ __noinline__ int stage_chunk(const DevMesh &m, const DevLines &Ln, const SolveArgs &a, Stage<R, NL> &sg,
+template <class C>
+__device__ __noinline__ int stage_chunk(const DevMesh &m, const DevLines &Ln, const SolveArgs &a, Stage<C> &sg,
                                         int32_t qb, int32_t cnt, int sign) {
+    using R = typename C::R;
     const int lane = threadIdx.x & 31;
     const int32_t npt = cnt + 1;
     const int nch = npt - qb < 32 ? int(npt - qb) : 32;
@@ -993,7 +1390,7 @@ __device__ __noinline__ int stage_chunk(const DevMesh &m, const DevLines &Ln, co
     const int32_t q = qb + lane;
     double zq = 0.0;
     R deq = R(0);
-    if (lane < nch) stage_point<R, NL>(m, Ln, sg, q, cnt, slot, sign, zq, deq);
+    if (lane < nch) stage_point<C>(m, Ln, sg, q, cnt, slot, sign, zq, deq);
     // the farther point's Z and delta bound: the previous lane's, or the carried point's for lane 0
     double zf = __shfl_up_sync(kFull, zq, 1);
     R def = __shfl_up_sync(kFull, deq, 1);
@@ -1009,7 +1406,7 @@ __device__ __noinline__ int stage_chunk(const DevMesh &m, const DevLines &Ln, co
         }
     }
     int nvk = 0;  // the far end (q = 0) starts the line: no interval
-    if (lane < nch && q > 0) nvk = stage_interval<R, NL>(m, Ln, a, sg, slot, sign, zf, zq, def, deq);
+    if (lane < nch && q > 0) nvk = stage_interval<C>(m, Ln, a, sg, slot, sign, zf, zq, def, deq);
     int incl = nvk;
 #pragma unroll
     for (int sh = 1; sh < 32; sh <<= 1) {
@@ -1029,92 +1426,96 @@ __device__ __noinline__ int stage_chunk(const DevMesh &m, const DevLines &Ln, co
 // Eliminate one half of a pair line (direction sign r) from its far end up to
 // (excluding) the origin row.  Leaves the origin row's coupling (D Fh, zh)
 // and the last optical-depth increment in the lane's sweep state.
-template <typename R, int NL, int BPL, int ORD, typename P>
-__device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs &a, Stage<R, NL> &sg,
-                           Lane<R, ORD, P> &ln, int sign) {
-    constexpr int kCap = Stage<R, NL>::kCap;
+template <class C>
+__device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs &a, Stage<C> &sg, Lane<C> &ln,
+                           int sign) {
+    using R = typename C::R;
+    using V = typename C::V;
+    constexpr int NL = C::NL;
     const int lane = threadIdx.x & 31;
     {
-        Sweep<R, P> w[BPL];
+        Sweep<V, typename C::W> w[C::NV];
 #pragma unroll
-        for (int i = 0; i < BPL; ++i) {
-            w[i].Fh = P(1);
-            w[i].Dm = P(1);
-            w[i].zh = R(a.I_bdy);
-            w[i].dtp = P(0);
-            w[i].hp = R(-1);  // no row yet (Hermitian scheme)
-            w[i].Sp = w[i].Sc = w[i].rh = w[i].chi = w[i].eta = R(0);
+        for (int i = 0; i < C::NV; ++i) {
+            w[i].Fh = w[i].Dm = vset<typename C::W>(1.f);
+            w[i].dtp = vset<typename C::W>(0.f);
+            if constexpr (C::kPacked) w[i].zh = vset<V>(float(a.I_bdy));
+            else w[i].zh = R(a.I_bdy);
+            w[i].hp = vset<V>(-1.f);  // no row yet (Hermitian scheme)
+            w[i].Sp = w[i].Sc = w[i].rh = w[i].chi = w[i].eta = vset<V>(0.f);
         }
-        put_sweep<R, BPL, ORD, P>(ln, w, lane);
+        put_sweep<C>(ln, w, lane);
     }
     const int32_t cnt = sg.hl.cnt;
     __syncwarp();
     if (cnt == 0) return;
 #pragma unroll 1
     for (int32_t qb = 0; qb <= cnt; qb += 32) {
-        const int total = stage_chunk<R, NL>(m, Ln, a, sg, qb, cnt, sign);
+        const int total = stage_chunk<C>(m, Ln, a, sg, qb, cnt, sign);
         const int nch = cnt + 1 - qb < 32 ? int(cnt + 1 - qb) : 32;
         if (qb == 0) {  // the far end: its optics; its row follows with the first increment
-            Bin<R, NL> f[BPL];
-            bool act[BPL];
-            get_bins<R, NL, BPL>(sg, f, act, lane);
             R ce[2 * NL];
 #pragma unroll
             for (int c = 0; c < 2 * NL; ++c) ce[c] = sg.ce[c][1];
             const R rdv = Ar<R>::rcp(sg.w[1]);
-            R cmax = R(0);
 #pragma unroll
-            for (int i = 0; i < BPL; ++i) {
+            for (int i = 0; i < C::BPL; ++i) {
+                Bin<R, NL> f;
+#pragma unroll
+                for (int l = 0; l < NL; ++l) {
+                    f.A[l] = vget(sg.fA[l][i / C::kIn][lane], i % C::kIn);
+                    f.B[l] = vget(sg.fB[l][i / C::kIn][lane], i % C::kIn);
+                }
                 R chi, eta;
-                optics<R, NL>(sg.d[1], rdv, sg.cc[1], sg.ec[1], ce, f[i], chi, eta);
-                ln.wr[1][i][lane] = chi;
-                ln.wr[2][i][lane] = eta;
-                if constexpr (ORD == 4) ln.wr[4][i][lane] = Ar<R>::src(eta, chi);
-                cmax = i == 0 ? chi : fmax(cmax, chi);
+                optics<R, NL>(sg.d[1], rdv, sg.cc[1], sg.ec[1], ce, f, chi, eta);
+                vput(ln.wr[1][i / C::kIn][lane], i % C::kIn, chi);
+                vput(ln.wr[2][i / C::kIn][lane], i % C::kIn, eta);
+                if constexpr (C::ORD == 4) ln.wr[4][i][lane] = Ar<R>::src(eta, chi);
             }
-            ln.cm[lane] = cmax;
             __syncwarp();
         }
         int pos = 0, pend = -1;
         bool fresh = true;
 #pragma unroll 1
         for (;;) {
-            pos = consume_chunk<R, NL, BPL, ORD, P>(sg, ln, a, total, nch, sign, pos, pend, fresh);
+            pos = consume_chunk<C>(sg, ln, a, total, nch, sign, pos, pend, fresh);
             if (pos >= total) break;
-            resolve_n_inter<R, NL>(sg, m, Ln, a, sign, pos % kCap, lane_bin<BPL>(sg, 0, lane),
-                                   lane_bin<BPL>(sg, BPL - 1, lane));
+            resolve_n_inter<C>(sg, m, Ln, a, sign, pos);
             pend = pos;
             fresh = false;
         }
-        if (lane == 0) carry_slot<R, NL>(sg, nch);
+        if (lane == 0) carry_slot<C>(sg, nch);
         __syncwarp();
     }
 }
 
 // CTAs of 4 warps (2 in double precision, whose per-warp stage is twice as
 // large); the minimum resident CTAs per SM caps the registers
-// (65536 / (threads x CTAs)).  One line, second order: 9 CTAs (56 registers;
-// the shared staging of 9 CTAs, 24.5 KB each plus 1 KB reserved, fits 228 KB),
-// measured 4 % faster than 8 and 10 % faster than 7 on GB300 (the Hermitian
-// scheme: 3 % faster than 8).  Two lines: 8 CTAs (64 registers; 18 % faster
-// than 4 on the clump octree); three and four: 6 (80 registers; 11 % faster
-// than 4 on a four-line wind).
-template <typename R, int NL, int BPL, typename P = R>
+// (65536 / (threads x CTAs)).  The packed form: 8 for one line (64 registers,
+// 25 KB of shared memory each; the 50 000-point step takes 92.6 ms with 7, 89.9
+// with 8, 91.4 with 9, where the loop spills), 7 and 6 for two and four lines,
+// bounded by the staging.
+template <class C>
 struct Occ {
-    static constexpr int kWarps = sizeof(R) == 8 ? 2 : 4;
+    static constexpr int NL = C::NL;
+    static constexpr int kWarps = sizeof(typename C::R) == 8 ? 2 : 4;
     static constexpr int kThreads = 32 * kWarps;
     static constexpr int kMinBlocks =
-        sizeof(R) == 8 ? 1
-        : sizeof(P) == 8 ? (NL == 1 ? 4 : 2)
+        sizeof(typename C::R) == 8 ? 1
+        : sizeof(typename C::P) == 8 ? (NL == 1 ? 4 : 2)
+        : C::BPL == 4 ? 5
+        : C::kPacked ? (NL == 1 ? 8 : NL == 2 ? 7 : NL <= 4 ? 6 : 4)
         : (NL == 1 ? 9 : NL == 2 ? 8 : NL <= 4 ? 6 : 3);
 };
 
 // J of origin a.o_begin + oc for the bins of frequency tile `tile`, by one warp.
-template <typename R, int NL, int BPL, int ORD, typename P>
+template <class C>
 __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln, const DevRays &Rs,
-                                           const SolveArgs &a, int32_t oc, int32_t tile, Stage<R, NL> &sg,
-                                           Lane<R, ORD, P> &ln, int lane) {
-    static_assert(BPL <= 2, "the shared per-lane state holds two bins");
+                                           const SolveArgs &a, int32_t oc, int32_t tile, Stage<C> &sg, Lane<C> &ln,
+                                           int lane) {
+    using R = typename C::R;
+    using P = typename C::P;
+    constexpr int NL = C::NL, BPL = C::BPL, ORD = C::ORD;
     const int32_t o = a.o_begin + oc;
     const int32_t L = Ln.L, F = Ln.F, NB = L * F;
     const double dvo = Ln.dvw[o];
@@ -1143,10 +1544,8 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
     const R rdvo = Ar<R>::rcp(__ldg(Pts<R>::dvw(Ln) + o));
 
     // frequency of each bin of this lane and its profile constants
-    float am[NL], bm[NL];
     R So_[BPL];  // the source function at the origin of each bin
-#pragma unroll
-    for (int l = 0; l < NL; ++l) am[l] = bm[l] = 0.f;
+    float lA[NL][2], lB[NL][2];  // the smallest and largest A and B of each line over the lane's bins
 #pragma unroll
     for (int i = 0; i < BPL; ++i) {
         const int32_t b = tile * 32 * BPL + lane + 32 * i;
@@ -1160,39 +1559,38 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
             const double r = (lp < L) ? Ln.ratio[l * MGX_MAX_LINES + lp] : 1.0;
             f.A[lp] = R((kC * (r - 1.0) + r * ub) * Ar<R>::kArgScale);
             f.B[lp] = R(r * (1.0 + ub / kC) * Ar<R>::kArgScale);
-            sg.fA[lp][i][lane] = f.A[lp];
-            sg.fB[lp][i][lane] = f.B[lp];
-            am[lp] = fmaxf(am[lp], fabsf(float(f.A[lp])));
-            bm[lp] = fmaxf(bm[lp], fabsf(float(f.B[lp])));
+            vput(sg.fA[lp][i / C::kIn][lane], i % C::kIn, f.A[lp]);
+            vput(sg.fB[lp][i / C::kIn][lane], i % C::kIn, f.B[lp]);
+            const float fa = float(f.A[lp]), fb = float(f.B[lp]);
+            lA[lp][0] = i == 0 ? fa : fminf(lA[lp][0], fa);
+            lA[lp][1] = i == 0 ? fa : fmaxf(lA[lp][1], fa);
+            lB[lp][0] = i == 0 ? fb : fminf(lB[lp][0], fb);
+            lB[lp][1] = i == 0 ? fb : fmaxf(lB[lp][1], fb);
         }
         R chi_o, eta_o;
         optics<R, NL>(R(0), rdvo, __ldg(Pts<R>::chic(Ln) + o), __ldg(Pts<R>::etac(Ln) + o), oce, f, chi_o, eta_o);
         So_[i] = eta_o / chi_o;
     }
-    if constexpr (sizeof(R) == 4 && NL == 1) {
-        // the profile constants of the tile's first and last bin (the far-wing test of gen_sample)
-        __syncwarp();
-        if (lane == 0) {
-            const int32_t jl = (NB - 1 - tile * 32 * BPL) < 32 * BPL - 1 ? NB - 1 - tile * 32 * BPL : 32 * BPL - 1;
-            sg.wa[0] = sg.fA[0][0][0];
-            sg.wb[0] = sg.fB[0][0][0];
-            sg.wa[1] = sg.fA[0][jl / 32][jl % 32];
-            sg.wb[1] = sg.fB[0][jl / 32][jl % 32];
-            sg.wing = L == 1;
-        }
-    }
     if constexpr (sizeof(R) == 4) {
-        // largest |A|, |B| of each line over the warp's bins (the opacity bound of Eq. 2)
+        // the ranges of A and B over the warp's bins (line_is_far) and the largest
+        // |A|, |B| (the opacity bound of Eq. 2)
 #pragma unroll
         for (int lp = 0; lp < NL; ++lp) {
 #pragma unroll
             for (int sh = 16; sh > 0; sh >>= 1) {
-                am[lp] = fmaxf(am[lp], __shfl_xor_sync(kFull, am[lp], sh));
-                bm[lp] = fmaxf(bm[lp], __shfl_xor_sync(kFull, bm[lp], sh));
+                lA[lp][0] = fminf(lA[lp][0], __shfl_xor_sync(kFull, lA[lp][0], sh));
+                lA[lp][1] = fmaxf(lA[lp][1], __shfl_xor_sync(kFull, lA[lp][1], sh));
+                lB[lp][0] = fminf(lB[lp][0], __shfl_xor_sync(kFull, lB[lp][0], sh));
+                lB[lp][1] = fmaxf(lB[lp][1], __shfl_xor_sync(kFull, lB[lp][1], sh));
             }
             if (lane == 0) {
-                sg.Am[lp] = am[lp];
-                sg.Bm[lp] = bm[lp];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    sg.wA[lp][e] = lA[lp][e];
+                    sg.wB[lp][e] = lB[lp][e];
+                }
+                sg.Am[lp] = fmaxf(fabsf(lA[lp][0]), fabsf(lA[lp][1]));
+                sg.Bm[lp] = fmaxf(fabsf(lB[lp][0]), fabsf(lB[lp][1]));
             }
         }
     }
@@ -1211,12 +1609,13 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         if (lane < 3) sg.r[lane] = Rs.dir[3 * (level_offset(lev) + (ray & 0x0FFFFFFFu)) + lane];
         if (lane == 0) sg.hl = half_list(a, hb);
         __syncwarp();
-        half_sweep<R, NL, BPL, ORD, P>(m, Ln, a, sg, ln, -1);
+        half_sweep<C>(m, Ln, a, sg, ln, -1);
 #pragma unroll
         for (int i = 0; i < BPL; ++i) {  // the backward half's coupling to the origin row
-            cpD[i] = ln.wp[0][i][lane];  // D Fh
-            cpT[i] = ln.wp[1][i][lane];  // dtb / 2
-            cpZ[i] = ln.wr[0][i][lane];  // zh
+            const int v = i / C::kIn, c = i % C::kIn;
+            cpD[i] = vget(ln.wp[0][v][lane], c);  // D Fh
+            cpT[i] = vget(ln.wp[1][v][lane], c);  // dtb / 2
+            cpZ[i] = vget(ln.wr[0][v][lane], c);  // zh
             if constexpr (ORD == 4) {
                 cpH[i] = ln.wr[5][i][lane];  // hp
                 cpS[i] = ln.wr[3][i][lane];  // Sp
@@ -1224,13 +1623,21 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         }
         if (lane == 0) sg.hl = half_list(a, hb + 1);
         __syncwarp();
-        half_sweep<R, NL, BPL, ORD, P>(m, Ln, a, sg, ln, 1);
+        half_sweep<C>(m, Ln, a, sg, ln, 1);
         const double w2 = a.w2[lev];
-        Sweep<R, P> wf[BPL];
-        get_sweep<R, BPL, ORD, P>(ln, wf, lane);
 #pragma unroll
         for (int i = 0; i < BPL; ++i) {
-            Sweep<R, P> wb;
+            const int v = i / C::kIn, c = i % C::kIn;
+            Sweep<R, P> wf, wb;
+            wf.Fh = vget(ln.wp[0][v][lane], c);
+            wf.Dm = P(1);
+            wf.dtp = vget(ln.wp[1][v][lane], c);
+            wf.zh = vget(ln.wr[0][v][lane], c);
+            if constexpr (ORD == 4) {
+                wf.Sp = ln.wr[3][i][lane];
+                wf.hp = ln.wr[5][i][lane];
+                wf.rh = wf.hp < R(0) ? R(0) : Ar<R>::rcp(wf.hp);
+            }
             wb.Fh = cpD[i];
             wb.Dm = P(1);
             wb.dtp = cpT[i];
@@ -1241,8 +1648,8 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
                 wb.rh = wb.hp < R(0) ? R(0) : Ar<R>::rcp(wb.hp);
             }
             const R So = So_[i];
-            const R u = ORD == 4 ? origin_u4(wb, wf[i], So, R(a.I_bdy)) : origin_u2(wb, wf[i], So);
-            const int32_t b = lane_bin<BPL>(sg, i, lane);
+            const R u = ORD == 4 ? origin_u4(wb, wf, So, R(a.I_bdy)) : origin_u2(wb, wf, So);
+            const int32_t b = lane_bin<C>(sg, i, lane);
             if (a.u_out && b < NB) a.u_out[(int64_t(oc) * Rs.npairs + p) * NB + b] = double(u);
             const double xv = w2 * double(u);
             const double sum = js[i];
@@ -1256,7 +1663,7 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
     unsigned n_act = 0;
 #pragma unroll
     for (int i = 0; i < BPL; ++i) {
-        const int32_t b = lane_bin<BPL>(sg, i, lane);
+        const int32_t b = lane_bin<C>(sg, i, lane);
         if (b < NB) {
             a.J[int64_t(o) * NB + b] = js[i] + jc[i];
             ++n_act;
@@ -1278,29 +1685,31 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
 }
 
 // Grid-mapped launch: warp w of the grid solves item w = oc * n_tiles + tile.
-template <typename R, int NL, int BPL, int ORD, typename P>
-__global__ void __launch_bounds__(Occ<R, NL, BPL, P>::kThreads, (Occ<R, NL, BPL, P>::kMinBlocks))
+template <class C>
+__global__ void __launch_bounds__(Occ<C>::kThreads, (Occ<C>::kMinBlocks))
 k_solve(const __grid_constant__ DevMesh m, const __grid_constant__ DevLines Ln, const __grid_constant__ DevRays Rs,
         const __grid_constant__ SolveArgs a) {
-    __shared__ Stage<R, NL> stage[Occ<R, NL, BPL, P>::kWarps];  // one per warp
-    __shared__ Lane<R, ORD, P> lanes[Occ<R, NL, BPL, P>::kWarps];
+    extern __shared__ __align__(16) unsigned char smem[];
+    Stage<C> *stage = reinterpret_cast<Stage<C> *>(smem);  // one per warp
+    Lane<C> *lanes = reinterpret_cast<Lane<C> *>(smem + sizeof(Stage<C>) * Occ<C>::kWarps);
     const int lane = threadIdx.x & 31;
     const int64_t item = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
     const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles;
     if (item >= n_items) return;
-    solve_item<R, NL, BPL, ORD, P>(m, Ln, Rs, a, int32_t(item / a.n_tiles), int32_t(item % a.n_tiles),
-                                stage[threadIdx.x >> 5], lanes[threadIdx.x >> 5], lane);
+    solve_item<C>(m, Ln, Rs, a, int32_t(item / a.n_tiles), int32_t(item % a.n_tiles), stage[threadIdx.x >> 5],
+                  lanes[threadIdx.x >> 5], lane);
 }
 
 // Persistent launch over a work list of (model, origin, tile) items of many
 // models: each warp takes the next item from a global counter until the list
 // is exhausted.
-template <typename R, int NL, int BPL, int ORD, typename P>
-__global__ void __launch_bounds__(Occ<R, NL, BPL, P>::kThreads, (Occ<R, NL, BPL, P>::kMinBlocks))
+template <class C>
+__global__ void __launch_bounds__(Occ<C>::kThreads, (Occ<C>::kMinBlocks))
 k_solve_queue(const BatchSlot *__restrict__ slots, const uint2 *__restrict__ work, int64_t n_work,
               unsigned long long *__restrict__ next) {
-    __shared__ Stage<R, NL> stage[Occ<R, NL, BPL, P>::kWarps];
-    __shared__ Lane<R, ORD, P> lanes[Occ<R, NL, BPL, P>::kWarps];
+    extern __shared__ __align__(16) unsigned char smem[];
+    Stage<C> *stage = reinterpret_cast<Stage<C> *>(smem);
+    Lane<C> *lanes = reinterpret_cast<Lane<C> *>(smem + sizeof(Stage<C>) * Occ<C>::kWarps);
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long it = 0;
@@ -1309,68 +1718,70 @@ k_solve_queue(const BatchSlot *__restrict__ slots, const uint2 *__restrict__ wor
         if (it >= (unsigned long long)n_work) return;
         const uint2 w = work[it];  // x = model << 16 | tile, y = origin
         const BatchSlot &s = slots[w.x >> 16];
-        solve_item<R, NL, BPL, ORD, P>(s.m, s.Ln, s.R, s.a, int32_t(w.y), int32_t(w.x & 0xffffu), stage[threadIdx.x >> 5],
-                                    lanes[threadIdx.x >> 5], lane);
+        solve_item<C>(s.m, s.Ln, s.R, s.a, int32_t(w.y), int32_t(w.x & 0xffffu), stage[threadIdx.x >> 5],
+                      lanes[threadIdx.x >> 5], lane);
         __syncwarp();
     }
 }
 
+// Shared memory of a CTA of a solve kernel.
+template <class C>
+constexpr size_t solve_smem() {
+    static_assert(sizeof(Stage<C>) % 16 == 0 && sizeof(Lane<C>) % 16 == 0, "16-byte aligned records");
+    return (sizeof(Stage<C>) + sizeof(Lane<C>)) * Occ<C>::kWarps;
+}
+
 // Prefer the largest shared-memory carveout for a solve kernel (its resident
-// CTAs are bounded by their per-warp staging), once per kernel and process.
-template <typename K>
+// CTAs are bounded by their per-warp staging) and allow its shared memory, on
+// the current device.
+template <class C, typename K>
 void prefer_shared(K kernel) {
-    static bool done = false;
-    if (!done) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        done = true;
-    }
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(solve_smem<C>()));
+}
+
+template <class C>
+void launch_one(const DevMesh &m, const DevLines &Ln, const DevRays &R_, const SolveArgs &a, cudaStream_t st) {
+    const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles;
+    if (n_items == 0) return;
+    constexpr int tb = Occ<C>::kThreads;
+    const unsigned grid = unsigned((n_items * 32 + tb - 1) / tb);
+    prefer_shared<C>(k_solve<C>);
+    k_solve<C><<<grid, tb, solve_smem<C>(), st>>>(m, Ln, R_, a);
 }
 
 template <typename R, int BPL, int ORD, typename P = R>
 void launch_RB(const DevMesh &m, const DevLines &Ln, const DevRays &R_, const SolveArgs &a, cudaStream_t st) {
-    const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles;
-    if (n_items == 0) return;
-    constexpr int tb = Occ<R, 1, BPL, P>::kThreads;
-    const unsigned grid = unsigned((n_items * 32 + tb - 1) / tb);
-    if (Ln.L <= 1) {
-        prefer_shared(k_solve<R, 1, BPL, ORD, P>);
-        k_solve<R, 1, BPL, ORD, P><<<grid, tb, 0, st>>>(m, Ln, R_, a);
-    } else if (Ln.L <= 2) {
-        prefer_shared(k_solve<R, 2, BPL, ORD, P>);
-        k_solve<R, 2, BPL, ORD, P><<<grid, tb, 0, st>>>(m, Ln, R_, a);
-    } else if (Ln.L <= 4) {
-        prefer_shared(k_solve<R, 4, BPL, ORD, P>);
-        k_solve<R, 4, BPL, ORD, P><<<grid, tb, 0, st>>>(m, Ln, R_, a);
-    } else {
-        prefer_shared(k_solve<R, 8, BPL, ORD, P>);
-        k_solve<R, 8, BPL, ORD, P><<<grid, tb, 0, st>>>(m, Ln, R_, a);
-    }
+    if (Ln.L <= 1) launch_one<Form<R, 1, BPL, ORD, P>>(m, Ln, R_, a, st);
+    else if (Ln.L <= 2) launch_one<Form<R, 2, BPL, ORD, P>>(m, Ln, R_, a, st);
+    else if (Ln.L <= 4) launch_one<Form<R, 4, BPL, ORD, P>>(m, Ln, R_, a, st);
+    else launch_one<Form<R, 8, BPL, ORD, P>>(m, Ln, R_, a, st);
 }
 
-template <typename R, int BPL, int NL, int ORD, typename P = R>
-void launch_queue_NL(const BatchSlot *slots, const uint2 *work, int64_t n_work, unsigned long long *next,
-                     cudaStream_t st) {
+template <class C>
+void launch_queue_one(const BatchSlot *slots, const uint2 *work, int64_t n_work, unsigned long long *next,
+                      cudaStream_t st) {
     int dev = 0, sms = 152, per_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    constexpr int tb = Occ<R, NL, BPL, P>::kThreads, nw = Occ<R, NL, BPL, P>::kWarps;
-    prefer_shared(k_solve_queue<R, NL, BPL, ORD, P>);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_queue<R, NL, BPL, ORD, P>, tb, 0);
+    constexpr int tb = Occ<C>::kThreads, nw = Occ<C>::kWarps;
+    prefer_shared<C>(k_solve_queue<C>);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_queue<C>, tb, solve_smem<C>());
     if (per_sm < 1) per_sm = 1;
     int64_t grid = int64_t(sms) * per_sm;
     const int64_t need = (n_work + nw - 1) / nw;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    k_solve_queue<R, NL, BPL, ORD, P><<<unsigned(grid), tb, 0, st>>>(slots, work, n_work, next);
+    k_solve_queue<C><<<unsigned(grid), tb, solve_smem<C>(), st>>>(slots, work, n_work, next);
 }
 
 template <typename R, int BPL, int ORD, typename P = R>
 void launch_queue_RB(int max_lines, const BatchSlot *slots, const uint2 *work, int64_t n_work,
                      unsigned long long *next, cudaStream_t st) {
-    if (max_lines <= 1) launch_queue_NL<R, BPL, 1, ORD, P>(slots, work, n_work, next, st);
-    else if (max_lines <= 2) launch_queue_NL<R, BPL, 2, ORD, P>(slots, work, n_work, next, st);
-    else if (max_lines <= 4) launch_queue_NL<R, BPL, 4, ORD, P>(slots, work, n_work, next, st);
-    else launch_queue_NL<R, BPL, 8, ORD, P>(slots, work, n_work, next, st);
+    if (max_lines <= 1) launch_queue_one<Form<R, 1, BPL, ORD, P>>(slots, work, n_work, next, st);
+    else if (max_lines <= 2) launch_queue_one<Form<R, 2, BPL, ORD, P>>(slots, work, n_work, next, st);
+    else if (max_lines <= 4) launch_queue_one<Form<R, 4, BPL, ORD, P>>(slots, work, n_work, next, st);
+    else launch_queue_one<Form<R, 8, BPL, ORD, P>>(slots, work, n_work, next, st);
 }
 
 }  // namespace
@@ -1378,9 +1789,10 @@ void launch_queue_RB(int max_lines, const BatchSlot *slots, const uint2 *work, i
 template <int ORD>
 void launch_solve_ord(const DevMesh &m, const DevLines &Ln, const DevRays &R, const SolveArgs &a, int precision,
                       cudaStream_t st) {
-    const int bpl = solve_bins_per_lane(precision, Ln.L * Ln.F);
+    const int bpl = solve_bins_per_lane(precision, ORD, Ln.L, Ln.L * Ln.F);
     if (precision == MGX_FP64) launch_RB<double, 1, ORD>(m, Ln, R, a, st);
     else if (precision == MGX_FP32_DT64) launch_solve_dt64(m, Ln, R, a, bpl, st);
+    else if (ORD == 2 && bpl == 4) launch_one<Form<float, 1, ORD == 2 ? 4 : 2, ORD>>(m, Ln, R, a, st);
     else if (bpl == 2) launch_RB<float, 2, ORD>(m, Ln, R, a, st);
     else launch_RB<float, 1, ORD>(m, Ln, R, a, st);
 }
@@ -1392,6 +1804,8 @@ void launch_solve_queue_ord(int precision, int bins_per_lane, int max_lines, con
     if (precision == MGX_FP64) launch_queue_RB<double, 1, ORD>(max_lines, slots, work, n_work, next, st);
     else if (precision == MGX_FP32_DT64)
         launch_solve_queue_dt64(bins_per_lane, max_lines, slots, work, n_work, next, st);
+    else if (ORD == 2 && bins_per_lane == 4)
+        launch_queue_one<Form<float, 1, ORD == 2 ? 4 : 2, ORD>>(slots, work, n_work, next, st);
     else if (bins_per_lane == 2) launch_queue_RB<float, 2, ORD>(max_lines, slots, work, n_work, next, st);
     else launch_queue_RB<float, 1, ORD>(max_lines, slots, work, n_work, next, st);
 }

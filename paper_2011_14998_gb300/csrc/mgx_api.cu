@@ -963,7 +963,7 @@ mgx_status mgx_solve_J(mgx_ctx *ctx, int32_t model, const mgx_solve_params *p, v
         a.o_begin = o0;
         a.o_end = o1;
         {
-            const int64_t per = 32 * solve_bins_per_lane(p->precision, int32_t(NB));
+            const int64_t per = 32 * solve_bins_per_lane(p->precision, p->order, m->L, int32_t(NB));
             a.n_tiles = int32_t((NB + per - 1) / per);
         }
         a.offs = offs + h0;
@@ -1075,7 +1075,7 @@ mgx_status mgx_solve_u(mgx_ctx *ctx, int32_t model, const mgx_solve_params *p, i
     a.o_begin = o0;
     a.o_end = o1;
     {
-        const int64_t per = 32 * solve_bins_per_lane(p->precision, int32_t(NB));
+        const int64_t per = 32 * solve_bins_per_lane(p->precision, p->order, m->L, int32_t(NB));
         a.n_tiles = int32_t((NB + per - 1) / per);
     }
     a.offs = offs;
@@ -1230,7 +1230,7 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
         max_nb = std::max<int64_t>(max_nb, int64_t(m->L) * m->F);
         pl.max_lines = std::max(pl.max_lines, int(m->L));
     }
-    pl.bpl = solve_bins_per_lane(p->precision, int32_t(max_nb));
+    pl.bpl = solve_bins_per_lane(p->precision, p->order, pl.max_lines, int32_t(max_nb));
     if (p->precision != MGX_FP64 && pl.tune.bins_per_lane > 0) pl.bpl = pl.tune.bins_per_lane;
     std::vector<BatchGeom> geo(static_cast<size_t>(n_models));
     std::vector<int64_t> obase(static_cast<size_t>(n_models));
@@ -1433,10 +1433,12 @@ mgx_status mgx_autotune(mgx_ctx *ctx, const int32_t *models, int32_t n_models, c
     if (max_trials < 0 || (max_trials > 0 && !trials)) return fail(ctx, MGX_EINVAL, "autotune: bad trial buffer");
     if (!models || !p || n_models < 1) return fail(ctx, MGX_EINVAL, "autotune: bad model list or params");
     int64_t max_nb = 1;
+    int max_lines = 1;
     for (int32_t k = 0; k < n_models; ++k) {
         const Model *m = get_model(ctx, models[k]);
         if (!m) return fail(ctx, MGX_EINVAL, "autotune: no model %d", models[k]);
         max_nb = std::max<int64_t>(max_nb, int64_t(m->L) * m->F);
+        max_lines = std::max(max_lines, int(m->L));
     }
     DeviceGuard g(ctx->device);
     const mgx_tuning saved = ctx->tune;
@@ -1470,7 +1472,11 @@ mgx_status mgx_autotune(mgx_ctx *ctx, const int32_t *models, int32_t n_models, c
     };
     // start from the current tuning with its automatic fields made explicit
     mgx_tuning best = saved;
-    if (best.bins_per_lane == 0 && p->precision != MGX_FP64) best.bins_per_lane = solve_bins_per_lane(MGX_FP32, int32_t(max_nb));
+    // (four bins per lane, which only the automatic choice takes, stay automatic)
+    if (best.bins_per_lane == 0 && p->precision != MGX_FP64) {
+        const int b = solve_bins_per_lane(p->precision, p->order, max_lines, int32_t(max_nb));
+        if (b <= 2) best.bins_per_lane = b;
+    }
     if (best.trace_ctas_per_sm == 0) best.trace_ctas_per_sm = 7;
     if (best.tail_permille == 0) best.tail_permille = 20;
     double best_ms = 0.0;

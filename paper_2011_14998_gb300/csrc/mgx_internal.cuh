@@ -172,7 +172,7 @@ void launch_excess_totals(const int64_t *lens, int64_t n, unsigned long long *ou
 // ---- formal solution (k_solve.cu)
 // frequency bins per lane of the solve kernel; a chunk has
 // ceil(n_bins / (32 * bins_per_lane)) tiles per origin
-int solve_bins_per_lane(int precision, int32_t n_bins);
+int solve_bins_per_lane(int precision, int order, int32_t n_lines, int32_t n_bins);
 // order: 2 (second-order scheme) or 4 (Hermitian scheme)
 void launch_solve(const DevMesh &m, const DevLines &Ln, const DevRays &R, const SolveArgs &a,
                   int precision, int order, cudaStream_t st);

@@ -135,7 +135,7 @@ int noalloc_solve(int device, const DevMesh &m, const DevLines &Ln, const DevRay
         a.o_begin = int32_t(o0);
         a.o_end = int32_t(o0 + c);
         {
-            const int64_t per = 32 * solve_bins_per_lane(precision, int32_t(NB));
+            const int64_t per = 32 * solve_bins_per_lane(precision, order, Ln.L, int32_t(NB));
             a.n_tiles = int32_t((NB + per - 1) / per);
         }
         a.offs = offs;

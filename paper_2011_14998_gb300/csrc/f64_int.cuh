@@ -1,0 +1,133 @@
+// f64_int.cuh -- double-precision exp(-a^2) and division on the integer pipes.
+//
+// GB300 issues one double-precision warp instruction per SM quarter every 64
+// cycles or so (1.0 TFLOP/s), and an exponential or a division is a chain of
+// ten to twenty of them.  Both are evaluated here in 64-bit fixed point
+// instead (largest errors measured: 0.66 ulp below |a| = 8 and 0.64 ulp, rms
+// 0.294 and 0.291 where rounding alone gives 0.289), at about 85 and 45 issue
+// slots, while the double-precision pipe works on the elimination.
+// A 64-bit product's high half is three 32 x 32 -> 64 multiply-adds (the
+// low halves' product is dropped: an error below two units of the result).
+#pragma once
+
+#include <stdint.h>
+#include <string.h>
+
+#ifndef __CUDACC__
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#endif
+
+namespace mgx {
+
+// 2^(j/1024), j = 0..1023, in Q1.62, from integer square roots of two.
+struct Exp2Table {
+    uint64_t v[1024];
+    constexpr Exp2Table() : v() {
+        uint64_t root[10] = {};  // 2^(2^-k), k = 10..1, in Q1.62
+        unsigned __int128 x = (unsigned __int128)1 << 125;  // 2 in Q.124
+        for (int k = 1; k <= 10; ++k) {
+            uint64_t r = 0;  // floor(sqrt(x))
+            for (int b = 62; b >= 0; --b) {
+                const uint64_t t = r | (uint64_t(1) << b);
+                if ((unsigned __int128)t * t <= x) r = t;
+            }
+            root[10 - k] = r;
+            x = (unsigned __int128)r << 62;
+        }
+        for (int j = 0; j < 1024; ++j) {
+            uint64_t p = uint64_t(1) << 62;
+            for (int b = 0; b < 10; ++b)
+                if (j >> b & 1) p = uint64_t(((unsigned __int128)p * root[b] + ((unsigned __int128)1 << 61)) >> 62);
+            v[j] = p;
+        }
+    }
+};
+
+__host__ __device__ __forceinline__ uint32_t mul_hi32(uint32_t a, uint32_t b) {
+    return uint32_t((uint64_t(a) * b) >> 32);
+}
+
+// High half of a b for a, b < 2^63, low by at most two units.
+__host__ __device__ __forceinline__ uint64_t mul_hi63(uint64_t a, uint64_t b) {
+    const uint32_t ah = uint32_t(a >> 32), al = uint32_t(a), bh = uint32_t(b >> 32), bl = uint32_t(b);
+    uint64_t t = uint64_t(ah) * bl;
+    t += uint64_t(al) * bh;
+    return uint64_t(ah) * bh + (t >> 32);
+}
+
+__host__ __device__ __forceinline__ double bits_double(uint64_t b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double d;
+    memcpy(&d, &b, 8);
+    return d;
+#endif
+}
+
+__host__ __device__ __forceinline__ uint64_t double_bits(double d) {
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(d);
+#else
+    uint64_t b;
+    memcpy(&b, &d, 8);
+    return b;
+#endif
+}
+
+// 2^(-a^2) for |a| = A / 2^57 (Q7.57); 0 from |a| = 31 on (2^-961).
+// a^2 = n + f; 2^(-a^2) = 2^-(n+1) 2^(1-f), 1 - f = j/1024 + r: the table's
+// 2^(j/1024) times 1 + p(r), p the Taylor polynomial of 2^r - 1 to degree four
+// (r < 2^-10: the next term is below 2^-59).  a^2 carries 56 fraction bits
+// below |a| = 8 and 52 above, where g < 2^-64.
+__host__ __device__ __forceinline__ double exp2_neg_sq(uint64_t A, const uint64_t *tab) {
+    if (A >= (uint64_t(31) << 57)) return 0.0;
+    const bool small = A < (uint64_t(1) << 60);
+    const uint64_t M = A << (small ? 3 : 1);   // |a| / 8 or / 32 in Q0.63
+    const uint64_t Y = mul_hi63(M, M);         // a^2 / 64 or / 1024 in Q0.62
+    const uint32_t n = uint32_t(Y >> (small ? 56 : 52));
+    const uint64_t F = ~(Y << (small ? 8 : 12));  // 1 - f in Q0.64 (less 2^-64)
+    const uint64_t T = tab[F >> 54];
+    const uint64_t R = (F << 9) & 0x7fffffffffffffffull;  // 2^10 r in Q0.63
+    const uint32_t Rh = uint32_t(R >> 31);
+    // ln2^k / k! 2^(-10 (k-1)) for k = 4..1, scaled by 2^24, 2^24, 2^12, 1
+    const uint32_t v = mul_hi32(Rh, 645462u) + 3814213304u;
+    const uint64_t q = ((uint64_t(Rh) * v) >> 13) + 8862793787191474850ull;     // Q0.63
+    const uint64_t s = (mul_hi63(R, q) >> 11) + 6393154322601327830ull;        // Q0.63
+    const uint64_t m = T + (mul_hi63(T, mul_hi63(R, s)) >> 8);  // Q1.62
+    return bits_double(((m + 512) >> 10) + (uint64_t(1021 - n) << 52));
+}
+
+// e / t for finite e >= 0, t > 0: the mantissas' quotient from a
+// single-precision reciprocal and one fixed-point correction with its square.
+__host__ __device__ __forceinline__ double div_pos(double e, double t) {
+    const uint64_t be = double_bits(e), bt = double_bits(t);
+    const int xe = int(be >> 52), xt = int(bt >> 52), ex = xe - xt;
+    if (xe == 0 || xt == 0 || ex > 1000 || ex < -1000) return e / t;  // zero, subnormal or far out
+    const uint64_t hid = uint64_t(1) << 62, man = hid - 1;
+    const uint64_t me = ((be << 10) & man) | hid, mt = ((bt << 10) & man) | hid;  // Q1.62
+    const uint32_t tb = 0x3f800000u | (uint32_t(bt >> 29) & 0x7fffffu);
+    // the reciprocal of t's leading bits, lowered by 2^-21 so that 1 - t x is not negative
+#ifdef __CUDA_ARCH__
+    float x;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(__uint_as_float(tb)));
+    const uint32_t X = __float2uint_rz(x * 2147482624.0f);  // Q1.31
+#else
+    float x;
+    memcpy(&x, &tb, 4);
+    const uint32_t X = uint32_t(1.0f / x * 2147482624.0f);
+#endif
+    const uint64_t tx = uint64_t(uint32_t(mt >> 32)) * X + mul_hi32(uint32_t(mt), X);  // t x in Q2.61
+    const uint64_t qe = uint64_t(uint32_t(me >> 32)) * X + mul_hi32(uint32_t(me), X);
+    uint64_t d = (uint64_t(1) << 61) - tx;  // 1 - t x in [0, 2^-20)
+    const uint32_t dh = uint32_t(d >> 25);
+    d += (dh * dh) >> 11;                   // its square (the cube is below 2^-60)
+    const uint64_t s = qe + (mul_hi63(qe, d << 21) >> 18);  // Q2.61, in (1/2, 2)
+    const bool low = s < (uint64_t(1) << 61);
+    const uint64_t s2 = low ? s << 1 : s;
+    return bits_double(((s2 + 256) >> 9) + (uint64_t(int64_t(1022 + ex - int(low))) << 52));
+}
+
+}  // namespace mgx

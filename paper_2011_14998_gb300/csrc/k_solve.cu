@@ -5,11 +5,12 @@
 
 namespace mgx {
 
-// Bins per lane of the single-precision kernel: 2 when there are more bins than
-// lanes (the frequency-independent work is then shared by two bins), 4 in the
-// second-order form of one line when that takes no more bin slots than 2, else 1.
+// Bins per lane: 2 when there are more bins than lanes (the frequency-independent
+// work is then shared by two bins; the double-precision Hermitian form has one),
+// 4 in the single-precision second-order form of one line when that takes no
+// more bin slots than 2, else 1.
 int solve_bins_per_lane(int precision, int order, int32_t n_lines, int32_t n_bins) {
-    if (precision != MGX_FP32 && precision != MGX_FP32_DT64) return 1;
+    if (precision == MGX_FP64 && order == 4) return 1;
     if (precision == MGX_FP32 && order != 4 && n_lines == 1 && (n_bins + 127) / 128 * 2 == (n_bins + 63) / 64) return 4;
     return n_bins > 32 ? 2 : 1;
 }

@@ -54,6 +54,7 @@
 
 #include <type_traits>
 
+#include "f64_int.cuh"
 #include "mgx_internal.cuh"
 
 namespace mgx {
@@ -171,6 +172,8 @@ struct Form {
     using P = P_;
     static constexpr int NL = NL_, BPL = BPL_, ORD = ORD_;
     static constexpr bool kPacked = sizeof(R) == 4 && sizeof(P) == 4 && ORD == 2 && BPL % 2 == 0;
+    // the double-precision second-order form: exponentials and divisions on the integer pipes
+    static constexpr bool kInt = sizeof(R) == 8 && ORD == 2;
     using V = std::conditional_t<kPacked, float2, R>;
     using W = std::conditional_t<kPacked, float2, P>;
     static constexpr int kIn = kPacked ? 2 : 1;  // bins in a value
@@ -415,6 +418,9 @@ struct Stage {
     R de0;                                  // single precision: bound of |delta - delta64| of the carried point
     double z[sizeof(R) == 8 ? 33 : 1];      // exact Z (single precision: the carried point's only)
     int id[33], nv[33], so[33];             // point (-1: the origin), velocity samples, their offset
+    unsigned on[C::kInt ? kCap : 1];        // integer form: the lines that take part in each record
+    double span;                            // integer form, one line: x_span dvw_o, the bins' half-range in km/s
+    uint64_t uk[C::kInt && NL == 1 ? BPL : 1][32];  // and each lane's bins' place in it, (ub / span + 1) / 2, in Q0.63
     R Am[NL], Bm[NL];                       // largest |A|, |B| of each line over the warp's bins
     double r[3], xo[3], vo[3];              // pair direction, origin position and velocity (double)
     R vor[3];                               // origin velocity in the form's precision
@@ -424,7 +430,7 @@ struct Stage {
     int fix[BPL][32];                       // Eq. 2 counts of a sample whose single-precision decision was left
                                             // open (0: not open; negative: to resolve, the bits of -chi)
     float wA[NL][2], wB[NL][2];             // single precision: smallest and largest A, B over the warp's bins
-    unsigned m_split, m_new;                // packed form: the round's records that may split; whose lines differ
+    unsigned m_split, m_new, m_wild;        // packed and integer forms: the round's records that may split; whose lines differ
                                             // from the record's before
 };
 
@@ -660,6 +666,13 @@ __device__ __forceinline__ int stage_interval(const DevMesh &m, const DevLines &
             dev_fail(a.status, kDevSubdivLimit);
             nv = kMaxSubdiv;
         }
+        if constexpr (C::kInt) {
+            // the largest opacity any sample of the interval can reach
+            R cb = fmax(sg.cc[pa], sg.cc[slot]);
+#pragma unroll
+            for (int l = 0; l < NL; ++l) cb += fmax(sg.ce[2 * l][pa], sg.ce[2 * l][slot]);
+            sg.hq[slot] = cb * (1.0 + 0x1p-40);
+        }
         return nv;
     } else {
         const float da = sg.d[pa], db = sg.d[slot], wa = sg.w[pa], wb = sg.w[slot];
@@ -740,6 +753,110 @@ __device__ __forceinline__ int slot_of(const Stage<C> &sg, int s_abs, int nch) {
     return lo;
 }
 
+// The same for the double-precision integer form, where a product below half
+// an ulp is below 2^-54 of chi and the profile is taken as 0 from |a| = 31 on.
+// Evaluated in single precision; the margin on |a| covers its rounding.
+__device__ __forceinline__ bool line_is_far(double dl, double rdv, double cc, double ec, double c0, double e0,
+                                            const float *wA, const float *wB) {
+    if (c0 == 0.0 && e0 == 0.0) return true;
+    const float d = float(dl), rd = float(rdv), fc = float(cc), fe = float(ec), f0 = float(c0), g0 = float(e0);
+    const float lo = fmaf(d >= 0.f ? wB[0] : wB[1], d, wA[0]) * rd;
+    const float hi = fmaf(d >= 0.f ? wB[1] : wB[0], d, wA[1]) * rd;
+    const float mar = 1e-6f * (fmaxf(fabsf(wA[0]), fabsf(wA[1])) + fmaxf(fabsf(wB[0]), fabsf(wB[1])) * fabsf(d)) * rd;
+    float t = 31.f;
+    if (fc > 1e-30f && f0 < 1e30f && (g0 == 0.f || (fe > 1e-30f && g0 < 1e30f))) {
+        const float x = fmaxf(fmaxf(f0 * Ar<float>::rcp(fc), g0 > 0.f ? g0 * Ar<float>::rcp(fe) : 0.f), 1e-30f);
+        t = fminf(sqrtf(fmaxf(54.1f + __log2f(x), 0.f)) * 1.0001f + 1e-3f, 31.f);
+    }
+    return lo - mar >= t || hi + mar <= -t;
+}
+
+// Record of the integer form: a quarter of the distance to the previous sample,
+// eta_c / chi_c, chi_c, eta_c, the profile argument's two terms, then chi0 and
+// eta0 of each line.  One line: the argument of bin k is alpha + u_k gamma with
+// u_k = (ub_k / span + 1) / 2 (the bin's velocity ub within its range +-span),
+// alpha in Q6.57 and gamma scaled by the largest power
+// of two that keeps it below 2^63 (the shift back in its lowest three bits),
+// both from double products with their residuals, so that the cancellation
+// between them costs nothing.  More lines: delta and sqrt(log2 e) / dv.
+// Returns the mask of the lines that take part, bit 31 set when some bin may
+// need a split, bit 30 when the sample is outside what the fixed-point
+// arithmetic covers (plain_step takes it).
+constexpr unsigned kSplitBit = 0x80000000u, kWildBit = 0x40000000u, kLineBits = 0x3fffffffu;
+
+template <class C>
+__device__ __forceinline__ unsigned gen_sample_int(Stage<C> &sg, int k, int nv, int j, int s_rec, int sign,
+                                                   double dtau_max) {
+    constexpr int NL = C::NL;
+    double *o = sg.rec + s_rec * Stage<C>::kS;
+    // as the definition lays the samples out: interpolated from the earlier point along +r
+    const bool bwd = sign < 0;
+    const double sgn = double(sign);
+    const int b0 = bwd ? k - 1 : k, b1 = bwd ? k : k - 1;
+    const int i = bwd ? j : nv - j, ip = bwd ? j - 1 : nv - j + 1;
+    const double dn = double(nv);
+    const float rn = Ar<float>::rcp(float(nv));
+    auto frac = [&](int ii) -> double {  // ii / nv correctly rounded: the quotient with its residual added
+        if (nv == 1) return 0.0;
+        const double q = div_pos(double(ii), dn);
+        return fma(fma(-q, dn, double(ii)), double(rn), q);
+    };
+    const double ti = frac(i), tp = frac(ip);
+    auto at = [&](double x0, double x1, int ii, double t) -> double {
+        return ii == 0 ? x0 : ii == nv ? x1 : __dadd_rn(x0, __dmul_rn(__dsub_rn(x1, x0), t));
+    };
+    const double s0 = sgn * sg.z[b0], s1 = sgn * sg.z[b1];
+    const double ds = fabs(at(s0, s1, i, ti) - at(s0, s1, ip, tp));
+    const double dl = at(sg.d[b0], sg.d[b1], i, ti), wv = at(sg.w[b0], sg.w[b1], i, ti);
+    const double cc = at(sg.cc[b0], sg.cc[b1], i, ti), ec = at(sg.ec[b0], sg.ec[b1], i, ti);
+    const double rs = div_pos(Ar<float>::kArgScale, wv);
+    o[0] = 0.25 * ds;
+    o[1] = div_pos(ec, cc);
+    o[2] = cc;
+    o[3] = ec;
+    unsigned on = 0;
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const double c0 = at(sg.ce[2 * l][b0], sg.ce[2 * l][b1], i, ti);
+        const double e0 = at(sg.ce[2 * l + 1][b0], sg.ce[2 * l + 1][b1], i, ti);
+        o[6 + 2 * l] = c0;
+        o[7 + 2 * l] = e0;
+        if (!line_is_far(dl, rs, cc, ec, c0, e0, sg.wA[l], sg.wB[l])) on |= 1u << l;
+    }
+    const double top = sg.hq[k];  // bound of chi on the interval
+    unsigned cls = on;
+    if (!(top * ds <= dtau_max * (1.0 - 0x1p-38))) cls |= kSplitBit;
+    bool wild = !(top * ds < 1e60) || !(cc > 1e-150);
+    if constexpr (NL == 1) {
+        if (on) {
+            // gamma = 2 span (1 + delta/c) rs, alpha = delta rs - gamma / 2
+            const double G = sg.span, q = G * (1.0 / kC);
+            const double G1 = fma(q, dl, G), G1l = fma(q, dl, G - G1);
+            const double gh = G1 * rs, gl = fma(G1, rs, -gh) + G1l * rs;
+            const double ah = dl * rs, al = fma(dl, rs, -ah);
+            const double am = ah - gh, z = am - ah;
+            const double aml = ((ah - (am - z)) - (gh + z)) + (al - gl);
+            wild |= !(gh < 31.0) || !(gh >= 0.0) || !(fabs(am) < 63.0);
+            const int ex = int(double_bits(gh) >> 52) - 1022;  // gh < 2^ex
+            const int sh = ex < 1 ? 4 : ex > 5 ? 0 : 5 - ex;   // gamma 2^(57 + sh) = gh 2^(58 + sh) < 2^63
+            const double up = bits_double(uint64_t(1023 + 58 + sh) << 52);
+            uint64_t g = uint64_t(__double2ll_rn(gh * up) + __double2ll_rn(gl * up));
+            o[4] = __longlong_as_double(__double2ll_rn(am * 0x1p57) + __double2ll_rn(aml * 0x1p57));
+            o[5] = __longlong_as_double((long long)((g & ~uint64_t(7)) | uint64_t(sh)));
+        }
+    } else {
+        o[4] = dl;
+        o[5] = rs;
+    }
+    if (wild) {  // plain_step's layout: delta, dv
+        cls |= kWildBit | kSplitBit;
+        o[4] = dl;
+        o[5] = wv;
+    }
+    sg.on[s_rec] = on;
+    return cls;
+}
+
 // Record of sample s_abs of the chunk (relative to its first) into record s_rec.
 // Returns (packed form) the mask of the lines that take part, bit 31 set when some bin may need a split.
 template <class C>
@@ -808,6 +925,8 @@ __device__ __forceinline__ unsigned gen_sample(Stage<C> &sg, int s_abs, int s_re
 #pragma unroll
             for (int c = 0; c < 2 * NL; ++c) o[6 + c] = ce[c];
         }
+    } else if constexpr (C::kInt) {
+        return gen_sample_int<C>(sg, k, nv, j, s_rec, sign, dtau_max);
     } else {
         // the definition's layout: samples interpolated from the earlier point
         // along +r with t = i / nv, exact end points; ds between consecutive samples
@@ -1359,6 +1478,285 @@ __device__ __noinline__ int consume_chunk(Stage<C> &sg, Lane<C> &ln, const Solve
     return r0 < total ? r0 + s : total;
 }
 
+// ---- the double-precision second-order form on the integer pipes -------------
+
+// State of one bin: Y = D Fh and z of the scaled form above in homogeneous
+// coordinates, Y = N / Q and z = W / Q, in which a row is linear and needs no
+// reciprocal (dt the increment beyond the current sample, dtb its mean with the
+// one before, S the current sample's source function):
+//   N += dtb Q,  W += S dtb Q,  Q += dt N
+// (D = Q / Q', so N' / Q' = D (dtb + Y) and W' / Q' = D (z + dtb S)).  Every
+// term is positive (W's sign apart, which I_bdy may make negative), so nothing
+// cancels; Q grows like e^tau and is scaled back when it passes 2^300.
+struct IntSweep {
+    double N, Q, W, T, S, h;  // T, S: opacity and source function of the current sample; h: half the last increment
+};
+
+__device__ __forceinline__ void int_row(IntSweep &w, double S, double h) {
+    const double p = (w.h + h) * w.Q;
+    w.N += p;
+    w.W = fma(S, p, w.W);
+    w.Q = fma(h, __hiloint2double(__double2hiint(w.N) + 0x100000, __double2loint(w.N)), w.Q);  // h 2N
+    w.h = h;
+    if (__double2hiint(w.Q) > 0x52b00000) {  // 2^300
+        const double f = bits_double(uint64_t(2046 - (__double2hiint(w.Q) >> 20)) << 52);
+        w.N *= f;
+        w.Q *= f;
+        w.W *= f;
+    }
+}
+
+// Opacity and emissivity of record src for bin i of the lane, over the lines in `on`.
+template <class C>
+__device__ __forceinline__ void int_optics(const double *src, unsigned on, const Stage<C> &sg, const uint64_t *tab,
+                                           int i, uint64_t u, double &chi, double &eta) {
+    chi = src[2];
+    eta = src[3];
+    if constexpr (C::NL == 1) {
+        if (!on) return;
+        const uint64_t g = double_bits(src[5]);
+        int64_t a = __double_as_longlong(src[4]) + int64_t((mul_hi63(u, g) << 1) >> (g & 7));
+        a = a < 0 ? -a : a;
+        const double e = exp2_neg_sq(uint64_t(a), tab);
+        chi = fma(src[6], e, chi);
+        eta = fma(src[7], e, eta);
+    } else {
+        const int lane = threadIdx.x & 31;
+#pragma unroll 1
+        for (; on; on &= on - 1) {
+            const int l = __ffs(int(on)) - 1;
+            const double a = fabs(fma(sg.fB[l][i][lane], src[4], sg.fA[l][i][lane]) * src[5]);
+            const double e = a < 31.0 ? exp2_neg_sq(uint64_t(__double2ll_rn(a * 0x1p57)), tab) : 0.0;
+            chi = fma(src[6 + 2 * l], e, chi);
+            eta = fma(src[7 + 2 * l], e, eta);
+        }
+    }
+}
+
+// A sample of an interval on which some bin may need sub-intervals (Eq. 2).
+// The counts are the definition's: taken here where chi ds / dtau_max is
+// farther than its rounding from an integer, else left open (false is
+// returned, sg.fix marks the bins) and redone in the definition's own order.
+template <class C>
+__device__ __forceinline__ bool int_split_step(const double *src, unsigned on, bool fixed, Stage<C> &sg,
+                                               const SolveArgs &a, const uint64_t *tab,
+                                               const uint64_t (&u)[C::BPL], IntSweep (&w)[C::BPL]) {
+    const int lane = threadIdx.x & 31;
+    double chi[C::BPL], eta[C::BPL];
+    const double q = src[0];
+    bool split = false;
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) {
+        int_optics<C>(src, on, sg, tab, i, u[i], chi[i], eta[i]);
+        split |= !(fmax(w[i].T, chi[i]) * (4.0 * q) <= a.dtau_max * (1.0 - 0x1p-45));
+    }
+    int n[C::BPL];
+    if (__any_sync(kFull, split)) {
+        bool open = false;
+#pragma unroll
+        for (int i = 0; i < C::BPL; ++i) {
+            const double r = fmax(w[i].T, chi[i]) * (4.0 * q) / a.dtau_max;
+            const double c = ceil(r);
+            n[i] = c > double(kMaxSubdiv) ? kMaxSubdiv + 1 : c <= 1.0 ? 1 : int(c);
+            const bool near = fabs(r - rint(r)) <= r * 0x1p-45 && r > 0.5;
+            if (fixed && sg.fix[i][lane] > 0) {
+                n[i] = sg.fix[i][lane];
+            } else if (near) {
+                n[i] = -1;
+                open = true;
+            } else if (n[i] > kMaxSubdiv) {
+                dev_fail(a.status, kDevSubdivLimit);
+                n[i] = kMaxSubdiv;
+            }
+        }
+        if (__any_sync(kFull, open)) {
+#pragma unroll
+            for (int i = 0; i < C::BPL; ++i) sg.fix[i][lane] = n[i] < 0 ? -1 : 0;
+            __syncwarp();
+            return false;
+        }
+        if (a.counters) {
+            unsigned extra = 0;
+#pragma unroll
+            for (int i = 0; i < C::BPL; ++i)
+                if (lane_bin<C>(sg, i, lane) < sg.NB) extra += unsigned(n[i] - 1);
+            extra = __reduce_add_sync(kFull, extra);
+            if (lane == 0) sg.n_extra += extra;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < C::BPL; ++i) n[i] = 1;
+    }
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) {
+        const double S = div_pos(eta[i], chi[i]);
+        if (n[i] > 1) {  // chi and eta linear on the sub-intervals
+            const double rn = 1.0 / double(n[i]), qs = q * rn;
+            const double c0 = w[i].T, e0 = w[i].S * c0;
+            const double dc = (chi[i] - c0) * rn, de = (eta[i] - e0) * rn;
+            double cp = c0, Sp = w[i].S;
+#pragma unroll 1
+            for (int k = 1; k < n[i]; ++k) {
+                const double ck = fma(dc, double(k), c0), ek = fma(de, double(k), e0);
+                int_row(w[i], Sp, qs * (cp + ck));
+                cp = ck;
+                Sp = ek > 0.0 ? div_pos(ek, ck) : 0.0;
+            }
+            int_row(w[i], Sp, qs * (cp + chi[i]));
+        } else {
+            int_row(w[i], w[i].S, q * (w[i].T + chi[i]));
+        }
+        w[i].T = chi[i];
+        w[i].S = S;
+    }
+    return true;
+}
+
+// consume_chunk of the integer form.  Also returns at a sample that the
+// fixed-point arithmetic does not cover (sg.m_wild), for plain_step.
+template <class C>
+__device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, const uint64_t *tab, int total,
+                                        int nch, int sign, int pos, int pend, bool fresh) {
+    constexpr int kS = Stage<C>::kS, kCap = Stage<C>::kCap;
+    const int lane = threadIdx.x & 31;
+    IntSweep w[C::BPL];
+    uint64_t u[C::BPL];
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) {
+        w[i].N = ln.wp[0][i][lane];
+        w[i].Q = 1.0;
+        w[i].h = ln.wp[1][i][lane];
+        w[i].W = ln.wr[0][i][lane];
+        w[i].T = ln.wr[1][i][lane];
+        w[i].S = ln.wr[2][i][lane];
+        u[i] = C::NL == 1 ? sg.uk[i][lane] : 0;
+    }
+    int r0 = pos / kCap * kCap, s = pos - r0;
+#pragma unroll 1
+    for (; r0 < total; r0 += kCap, s = 0, fresh = true) {
+        const int nr = total - r0 < kCap ? total - r0 : kCap;
+        unsigned m_split, m_new, m_wild;
+        if (fresh) {
+            const unsigned cls = lane < nr ? gen_sample<C>(sg, r0 + lane, lane, nch, sign, a.dtau_max) : 0u;
+            const unsigned up = __shfl_up_sync(kFull, cls, 1);
+            m_split = __ballot_sync(kFull, cls & kSplitBit);
+            m_wild = __ballot_sync(kFull, cls & kWildBit);
+            m_new = __ballot_sync(kFull, ((cls ^ up) & kLineBits) != 0u);
+            if (lane == 0) {
+                sg.m_split = m_split;
+                sg.m_new = m_new;
+                sg.m_wild = m_wild;
+            }
+            __syncwarp();
+        } else {
+            m_split = sg.m_split;
+            m_new = sg.m_new;
+            m_wild = sg.m_wild;
+        }
+        while (s < nr) {
+            const double *src = sg.rec + s * kS;
+            const unsigned on = sg.on[s];
+            if ((m_split >> s) & 1u) {
+                if ((m_wild >> s) & 1u) break;
+                if (!int_split_step<C>(src, on, r0 + s == pend, sg, a, tab, u, w)) break;
+                ++s;
+                continue;
+            }
+            const unsigned next = (m_split | m_new) & (0xfffffffeu << s);
+            const int e = next ? min(__ffs(int(next)) - 1, nr) : nr;
+            const double *end = sg.rec + e * kS;
+            s = e;
+            if (on == 0u) {
+#pragma unroll 1
+                for (; src < end; src += kS) {
+#pragma unroll
+                    for (int i = 0; i < C::BPL; ++i) {
+                        int_row(w[i], w[i].S, src[0] * (w[i].T + src[2]));
+                        w[i].T = src[2];
+                        w[i].S = src[1];
+                    }
+                }
+            } else {
+#pragma unroll 1
+                for (; src < end; src += kS) {
+#pragma unroll
+                    for (int i = 0; i < C::BPL; ++i) {
+                        double chi, eta;
+                        int_optics<C>(src, on, sg, tab, i, u[i], chi, eta);
+                        int_row(w[i], w[i].S, src[0] * (w[i].T + chi));
+                        w[i].T = chi;
+                        w[i].S = div_pos(eta, chi);
+                    }
+                }
+            }
+        }
+        if (s < nr) break;
+        __syncwarp();
+    }
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) {
+        ln.wp[0][i][lane] = div_pos(w[i].N, w[i].Q);
+        ln.wp[1][i][lane] = w[i].h;
+        ln.wr[0][i][lane] = copysign(div_pos(fabs(w[i].W), w[i].Q), w[i].W);
+        ln.wr[1][i][lane] = w[i].T;
+        ln.wr[2][i][lane] = w[i].S;
+    }
+    __syncwarp();
+    return r0 < total ? r0 + s : total;
+}
+
+// One sample of the integer form outside what its fixed-point arithmetic
+// covers (profile arguments in steps of more than 31 per half-range, optical
+// depths beyond 1e60, continua below 1e-150): the plain double-precision step.
+template <class C>
+__device__ __noinline__ void plain_step(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, int s_abs) {
+    constexpr int NL = C::NL;
+    const int lane = threadIdx.x & 31;
+    const double *src = sg.rec + s_abs % Stage<C>::kCap * Stage<C>::kS;
+    const double hq = 2.0 * src[0], rdv = 1.0 / src[5];
+#pragma unroll 1
+    for (int i = 0; i < C::BPL; ++i) {
+        Bin<double, NL> f;
+        double ce[2 * NL], chi, eta;
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            f.A[l] = sg.fA[l][i][lane];
+            f.B[l] = sg.fB[l][i][lane];
+            ce[2 * l] = src[6 + 2 * l];
+            ce[2 * l + 1] = src[7 + 2 * l];
+        }
+        optics<double, NL>(src[4], rdv, src[2], src[3], ce, f, chi, eta);
+        Sweep<double> w;
+        w.Fh = ln.wp[0][i][lane];
+        w.Dm = 1.0;
+        w.dtp = ln.wp[1][i][lane];
+        w.zh = ln.wr[0][i][lane];
+        const double c0 = ln.wr[1][i][lane], e0 = ln.wr[2][i][lane] * c0;
+        const double r = ceil(fmax(c0, chi) * (hq + hq) / a.dtau_max);
+        int n = r > double(kMaxSubdiv) ? kMaxSubdiv + 1 : r <= 1.0 ? 1 : int(r);
+        if (n > kMaxSubdiv) {
+            dev_fail(a.status, kDevSubdivLimit);
+            n = kMaxSubdiv;
+        }
+        if (n > 1 && lane_bin<C>(sg, i, lane) < sg.NB) atomicAdd(&sg.n_extra, unsigned(n - 1));
+        const double rn = 1.0 / double(n), hh = hq * rn, dc = (chi - c0) * rn, de = (eta - e0) * rn;
+        double cp = c0, ep = e0;
+#pragma unroll 1
+        for (int k = 1; k <= n; ++k) {
+            const double ck = k == n ? chi : c0 + dc * double(k), ek = k == n ? eta : e0 + de * double(k);
+            row<2>(w, cp, ep, hh * (cp + ck), 0.0, 0.0);
+            cp = ck;
+            ep = ek;
+        }
+        ln.wp[0][i][lane] = w.Dm * w.Fh;
+        ln.wp[1][i][lane] = w.dtp;
+        ln.wr[0][i][lane] = w.zh;
+        ln.wr[1][i][lane] = chi;
+        ln.wr[2][i][lane] = eta / chi;
+    }
+    __syncwarp();
+}
+
 // Copy the point data of slot `from` into slot 0 (the next chunk's farther point).
 template <class C>
 __device__ __forceinline__ void carry_slot(Stage<C> &sg, int from) {
@@ -1428,7 +1826,7 @@ __device__ __noinline__ int stage_chunk(const DevMesh &m, const DevLines &Ln, co
 // and the last optical-depth increment in the lane's sweep state.
 template <class C>
 __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs &a, Stage<C> &sg, Lane<C> &ln,
-                           int sign) {
+                           int sign, const uint64_t *tab) {
     using R = typename C::R;
     using V = typename C::V;
     constexpr int NL = C::NL;
@@ -1469,7 +1867,7 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
                 R chi, eta;
                 optics<R, NL>(sg.d[1], rdv, sg.cc[1], sg.ec[1], ce, f, chi, eta);
                 vput(ln.wr[1][i / C::kIn][lane], i % C::kIn, chi);
-                vput(ln.wr[2][i / C::kIn][lane], i % C::kIn, eta);
+                vput(ln.wr[2][i / C::kIn][lane], i % C::kIn, C::kInt ? eta / chi : eta);
                 if constexpr (C::ORD == 4) ln.wr[4][i][lane] = Ar<R>::src(eta, chi);
             }
             __syncwarp();
@@ -1478,8 +1876,20 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
         bool fresh = true;
 #pragma unroll 1
         for (;;) {
-            pos = consume_chunk<C>(sg, ln, a, total, nch, sign, pos, pend, fresh);
-            if (pos >= total) break;
+            if constexpr (C::kInt) {
+                pos = consume_int<C>(sg, ln, a, tab, total, nch, sign, pos, pend, fresh);
+                if (pos >= total) break;
+                if ((sg.m_wild >> pos % Stage<C>::kCap) & 1u) {
+                    plain_step<C>(sg, ln, a, pos);
+                    ++pos;
+                    fresh = pos % Stage<C>::kCap == 0;
+                    if (pos >= total) break;
+                    continue;
+                }
+            } else {
+                pos = consume_chunk<C>(sg, ln, a, total, nch, sign, pos, pend, fresh);
+                if (pos >= total) break;
+            }
             resolve_n_inter<C>(sg, m, Ln, a, sign, pos);
             pend = pos;
             fresh = false;
@@ -1489,8 +1899,8 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
     }
 }
 
-// CTAs of 4 warps (2 in double precision, whose per-warp stage is twice as
-// large); the minimum resident CTAs per SM caps the registers
+// CTAs of 4 warps (2 in the double-precision Hermitian form, whose per-warp
+// stage is twice as large); the minimum resident CTAs per SM caps the registers
 // (65536 / (threads x CTAs)).  The packed form: 8 for one line (64 registers,
 // 25 KB of shared memory each; the 50 000-point step takes 92.6 ms with 7, 89.9
 // with 8, 91.4 with 9, where the loop spills), 7 and 6 for two and four lines,
@@ -1498,10 +1908,11 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
 template <class C>
 struct Occ {
     static constexpr int NL = C::NL;
-    static constexpr int kWarps = sizeof(typename C::R) == 8 ? 2 : 4;
+    static constexpr int kWarps = sizeof(typename C::R) == 8 && !C::kInt ? 2 : 4;
     static constexpr int kThreads = 32 * kWarps;
     static constexpr int kMinBlocks =
-        sizeof(typename C::R) == 8 ? 1
+        C::kInt ? (NL == 1 ? 4 : NL <= 2 ? 3 : 2)
+        : sizeof(typename C::R) == 8 ? 1
         : sizeof(typename C::P) == 8 ? (NL == 1 ? 4 : 2)
         : C::BPL == 4 ? 5
         : C::kPacked ? (NL == 1 ? 8 : NL == 2 ? 7 : NL <= 4 ? 6 : 4)
@@ -1512,7 +1923,7 @@ struct Occ {
 template <class C>
 __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln, const DevRays &Rs,
                                            const SolveArgs &a, int32_t oc, int32_t tile, Stage<C> &sg, Lane<C> &ln,
-                                           int lane) {
+                                           int lane, const uint64_t *tab) {
     using R = typename C::R;
     using P = typename C::P;
     constexpr int NL = C::NL, BPL = C::BPL, ORD = C::ORD;
@@ -1533,6 +1944,7 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         sg.vor[1] = Pts<R>::vy(m)[o];
         sg.vor[2] = Pts<R>::vz(m)[o];
         sg.n_smp = sg.n_extra = sg.n_redo = 0u;
+        sg.span = Ln.x_span * dvo;
     }
     // the origin's own optics give S_o
     R oce[2 * NL];
@@ -1553,6 +1965,16 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         const int32_t l = bb / F, k = bb % F;
         const double x = (F == 1) ? 0.0 : -Ln.x_span + 2.0 * Ln.x_span * double(k) / double(F - 1);
         const double ub = x * dvo;
+        if constexpr (C::kInt && NL == 1) {  // (ub / span + 1) / 2 in Q0.63, with the quotient's residual
+            const double G = Ln.x_span * dvo, G2 = 2.0 * G, t = ub + G, tl = ub - (t - G);
+            const double q = t / G2, r = (fma(-q, G2, t) + tl) / G2;
+            long long u = 1ll << 62;
+            if (G > 0.0) {
+                u = q >= 1.0 ? INT64_MAX : __double2ll_rn(q * 0x1p63) + __double2ll_rn(r * 0x1p63);
+                if (u < 0) u = 0;
+            }
+            sg.uk[i][lane] = uint64_t(u);
+        }
         Bin<R, NL> f;
 #pragma unroll
         for (int lp = 0; lp < NL; ++lp) {
@@ -1571,7 +1993,7 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         optics<R, NL>(R(0), rdvo, __ldg(Pts<R>::chic(Ln) + o), __ldg(Pts<R>::etac(Ln) + o), oce, f, chi_o, eta_o);
         So_[i] = eta_o / chi_o;
     }
-    if constexpr (sizeof(R) == 4) {
+    if constexpr (sizeof(R) == 4 || C::kInt) {
         // the ranges of A and B over the warp's bins (line_is_far) and the largest
         // |A|, |B| (the opacity bound of Eq. 2)
 #pragma unroll
@@ -1609,7 +2031,7 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         if (lane < 3) sg.r[lane] = Rs.dir[3 * (level_offset(lev) + (ray & 0x0FFFFFFFu)) + lane];
         if (lane == 0) sg.hl = half_list(a, hb);
         __syncwarp();
-        half_sweep<C>(m, Ln, a, sg, ln, -1);
+        half_sweep<C>(m, Ln, a, sg, ln, -1, tab);
 #pragma unroll
         for (int i = 0; i < BPL; ++i) {  // the backward half's coupling to the origin row
             const int v = i / C::kIn, c = i % C::kIn;
@@ -1623,7 +2045,7 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
         }
         if (lane == 0) sg.hl = half_list(a, hb + 1);
         __syncwarp();
-        half_sweep<C>(m, Ln, a, sg, ln, 1);
+        half_sweep<C>(m, Ln, a, sg, ln, 1, tab);
         const double w2 = a.w2[lev];
 #pragma unroll
         for (int i = 0; i < BPL; ++i) {
@@ -1684,6 +2106,21 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
     }
 }
 
+// 2^(j/1024) in shared memory, after the warps' staging (the integer form).
+__device__ const Exp2Table d_exp2_table{};
+
+template <class C>
+__device__ __forceinline__ const uint64_t *load_table(unsigned char *smem) {
+    if constexpr (C::kInt) {
+        uint64_t *tab = reinterpret_cast<uint64_t *>(smem + (sizeof(Stage<C>) + sizeof(Lane<C>)) * Occ<C>::kWarps);
+        for (int j = threadIdx.x; j < 1024; j += Occ<C>::kThreads) tab[j] = d_exp2_table.v[j];
+        __syncthreads();
+        return tab;
+    } else {
+        return nullptr;
+    }
+}
+
 // Grid-mapped launch: warp w of the grid solves item w = oc * n_tiles + tile.
 template <class C>
 __global__ void __launch_bounds__(Occ<C>::kThreads, (Occ<C>::kMinBlocks))
@@ -1692,12 +2129,13 @@ k_solve(const __grid_constant__ DevMesh m, const __grid_constant__ DevLines Ln, 
     extern __shared__ __align__(16) unsigned char smem[];
     Stage<C> *stage = reinterpret_cast<Stage<C> *>(smem);  // one per warp
     Lane<C> *lanes = reinterpret_cast<Lane<C> *>(smem + sizeof(Stage<C>) * Occ<C>::kWarps);
+    const uint64_t *tab = load_table<C>(smem);
     const int lane = threadIdx.x & 31;
     const int64_t item = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
     const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles;
     if (item >= n_items) return;
     solve_item<C>(m, Ln, Rs, a, int32_t(item / a.n_tiles), int32_t(item % a.n_tiles), stage[threadIdx.x >> 5],
-                  lanes[threadIdx.x >> 5], lane);
+                  lanes[threadIdx.x >> 5], lane, tab);
 }
 
 // Persistent launch over a work list of (model, origin, tile) items of many
@@ -1710,6 +2148,7 @@ k_solve_queue(const BatchSlot *__restrict__ slots, const uint2 *__restrict__ wor
     extern __shared__ __align__(16) unsigned char smem[];
     Stage<C> *stage = reinterpret_cast<Stage<C> *>(smem);
     Lane<C> *lanes = reinterpret_cast<Lane<C> *>(smem + sizeof(Stage<C>) * Occ<C>::kWarps);
+    const uint64_t *tab = load_table<C>(smem);
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long it = 0;
@@ -1719,7 +2158,7 @@ k_solve_queue(const BatchSlot *__restrict__ slots, const uint2 *__restrict__ wor
         const uint2 w = work[it];  // x = model << 16 | tile, y = origin
         const BatchSlot &s = slots[w.x >> 16];
         solve_item<C>(s.m, s.Ln, s.R, s.a, int32_t(w.y), int32_t(w.x & 0xffffu), stage[threadIdx.x >> 5],
-                      lanes[threadIdx.x >> 5], lane);
+                      lanes[threadIdx.x >> 5], lane, tab);
         __syncwarp();
     }
 }
@@ -1728,7 +2167,7 @@ k_solve_queue(const BatchSlot *__restrict__ slots, const uint2 *__restrict__ wor
 template <class C>
 constexpr size_t solve_smem() {
     static_assert(sizeof(Stage<C>) % 16 == 0 && sizeof(Lane<C>) % 16 == 0, "16-byte aligned records");
-    return (sizeof(Stage<C>) + sizeof(Lane<C>)) * Occ<C>::kWarps;
+    return (sizeof(Stage<C>) + sizeof(Lane<C>)) * Occ<C>::kWarps + (C::kInt ? sizeof(Exp2Table) : 0);
 }
 
 // Prefer the largest shared-memory carveout for a solve kernel (its resident
@@ -1790,7 +2229,8 @@ template <int ORD>
 void launch_solve_ord(const DevMesh &m, const DevLines &Ln, const DevRays &R, const SolveArgs &a, int precision,
                       cudaStream_t st) {
     const int bpl = solve_bins_per_lane(precision, ORD, Ln.L, Ln.L * Ln.F);
-    if (precision == MGX_FP64) launch_RB<double, 1, ORD>(m, Ln, R, a, st);
+    if (precision == MGX_FP64 && ORD == 2 && bpl == 2) launch_RB<double, ORD == 2 ? 2 : 1, ORD>(m, Ln, R, a, st);
+    else if (precision == MGX_FP64) launch_RB<double, 1, ORD>(m, Ln, R, a, st);
     else if (precision == MGX_FP32_DT64) launch_solve_dt64(m, Ln, R, a, bpl, st);
     else if (ORD == 2 && bpl == 4) launch_one<Form<float, 1, ORD == 2 ? 4 : 2, ORD>>(m, Ln, R, a, st);
     else if (bpl == 2) launch_RB<float, 2, ORD>(m, Ln, R, a, st);
@@ -1801,7 +2241,9 @@ template <int ORD>
 void launch_solve_queue_ord(int precision, int bins_per_lane, int max_lines, const BatchSlot *slots,
                             const uint2 *work, int64_t n_work, unsigned long long *next, cudaStream_t st) {
     if (n_work == 0) return;
-    if (precision == MGX_FP64) launch_queue_RB<double, 1, ORD>(max_lines, slots, work, n_work, next, st);
+    if (precision == MGX_FP64 && ORD == 2 && bins_per_lane == 2)
+        launch_queue_RB<double, ORD == 2 ? 2 : 1, ORD>(max_lines, slots, work, n_work, next, st);
+    else if (precision == MGX_FP64) launch_queue_RB<double, 1, ORD>(max_lines, slots, work, n_work, next, st);
     else if (precision == MGX_FP32_DT64)
         launch_solve_queue_dt64(bins_per_lane, max_lines, slots, work, n_work, next, st);
     else if (ORD == 2 && bins_per_lane == 4)

@@ -1,0 +1,78 @@
+"""The fixed-point exponential and division of the double-precision solve
+(csrc/f64_int.cuh), compiled for the host: against mpmath at 40 digits.  Bounds:
+* table: ten roots, each within two units (its own truncation and half its
+  predecessor's error), a product of at most ten with half a unit of rounding
+  each: below 32 units;
+* exponential: a^2 low by at most three units of its last place (2^-56 below
+  |a| = 8, 2^-52 above), times ln 2; the polynomial's 32-bit product below 2^-55
+  and the table's 32 units of 2^-62: 2^-53.8 below |a| = 8 and 2^-50.8 above,
+  plus half an ulp of rounding;
+* division: 2^-55 plus half an ulp.
+CPU only."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+mp = pytest.importorskip("mpmath")
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SRC = """
+#include "f64_int.cuh"
+static constexpr mgx::Exp2Table tab;
+extern "C" double t_exp(uint64_t A) { return mgx::exp2_neg_sq(A, tab.v); }
+extern "C" double t_div(double e, double t) { return mgx::div_pos(e, t); }
+extern "C" uint64_t t_tab(int j) { return tab.v[j]; }
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("f64")
+    (d / "t.cpp").write_text(SRC)
+    so = str(d / "t.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I",
+                    os.path.join(ROOT, "paper_2011_14998_gb300", "csrc"), str(d / "t.cpp"), "-o", so], check=True)
+    L = C.CDLL(so)
+    L.t_exp.restype, L.t_exp.argtypes = C.c_double, [C.c_uint64]
+    L.t_div.restype, L.t_div.argtypes = C.c_double, [C.c_double, C.c_double]
+    L.t_tab.restype, L.t_tab.argtypes = C.c_uint64, [C.c_int]
+    return L
+
+
+def test_table(lib):
+    mp.mp.dps = 40
+    for j in list(range(0, 1024, 37)) + [1, 511, 512, 1023]:
+        assert abs(mp.mpf(lib.t_tab(j)) - mp.mpf(2) ** (62 + mp.mpf(j) / 1024)) < 32
+
+
+@pytest.mark.parametrize("lo,hi,rel", [(0.0, 1e-3, 2.0 ** -53.8), (0.0, 1.0, 2.0 ** -53.8), (1.0, 8.0, 2.0 ** -53.8),
+                                       (8.0, 31.0, 2.0 ** -50.8)])
+def test_exponential(lib, lo, hi, rel):
+    mp.mp.dps = 40
+    rng = np.random.default_rng(int(hi * 10) + int(lo))
+    edges = [int(lo * 2 ** 57), int(hi * 2 ** 57) - 1]
+    for A in [int(x * 2.0 ** 57) for x in rng.uniform(lo, hi, 4000)] + edges:
+        a = mp.mpf(A) / mp.mpf(2) ** 57
+        ref = mp.mpf(2) ** (-a * a)
+        assert abs(mp.mpf(lib.t_exp(A)) - ref) <= (rel + 2.0 ** -53) * ref
+    assert lib.t_exp(0) == 1.0 and lib.t_exp(31 << 57) == 0.0 and lib.t_exp((1 << 64) - 1) == 0.0
+
+
+def test_division(lib):
+    mp.mp.dps = 40
+    rng = np.random.default_rng(9)
+    e = np.ldexp(rng.uniform(1, 2, 6000), rng.integers(-300, 300, 6000))
+    t = np.ldexp(rng.uniform(1, 2, 6000), rng.integers(-300, 300, 6000))
+    e[:200] = t[:200] * rng.integers(1, 9, 200)
+    t[200:260] = np.ldexp(1.0, rng.integers(-50, 50, 60))
+    t[260:320] = np.nextafter(np.ldexp(1.0, rng.integers(-50, 50, 60)), 0.0)
+    for x, y in zip(e, t):
+        ref = mp.mpf(float(x)) / mp.mpf(float(y))
+        assert abs(mp.mpf(lib.t_div(float(x), float(y))) - ref) <= (2.0 ** -55 + 2.0 ** -53) * ref
+    # outside the fixed-point range: the plain division
+    for x, y in [(0.0, 3.0), (1e-320, 3.0), (3.0, 1e-320), (1e300, 1e-300), (1e-300, 1e300)]:
+        with np.errstate(over="ignore", under="ignore"):
+            assert lib.t_div(x, y) == float(np.float64(x) / np.float64(y))

@@ -15,6 +15,48 @@ int solve_bins_per_lane(int precision, int order, int32_t n_lines, int32_t n_bin
     return n_bins > 32 ? 2 : 1;
 }
 
+// Warps per origin and tile.  A warp takes all pairs of an item one after the
+// other, which leaves the chip idle when there are few items, and its last wave
+// nearly empty when there are a few waves: with fewer than four waves of
+// resident warps (28 per SM in single precision, 16 in the forms with double)
+// the pairs of an item are dealt to several warps, which store u, and J is
+// summed from u in the same order (400 points, 33 pairs: 1.95 -> 0.34 ms;
+// 12 000 points, 96 pairs, Hermitian: 50.8 -> 48.2 ms; 4001 points in double
+// precision 194 -> 165 ms).  Not when u would take more than a GiB.
+int32_t solve_parts(int precision, int64_t n_items, int32_t npairs, size_t u_bytes) {
+    const int64_t want = int64_t(4) * 152 * (precision == MGX_FP32 ? 28 : 16);
+    if (n_items <= 0 || n_items >= want || u_bytes > (size_t(1) << 30)) return 1;
+    const int64_t parts = (want + n_items - 1) / n_items;
+    return int32_t(parts < npairs ? parts : npairs);
+}
+
+namespace {
+
+// J = sum of 2 w u over the pairs in ascending order, Neumaier's compensated sum.
+__global__ void k_sum_pairs(const __grid_constant__ DevRays R, const __grid_constant__ SolveArgs a, int32_t n_bins) {
+    const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    const int64_t oc = t / n_bins;
+    if (oc >= a.o_end - a.o_begin) return;
+    const int32_t b = int32_t(t - oc * n_bins);
+    const uint32_t *rays = R.rays + (a.o_begin + oc) * R.npairs;
+    const double *u = a.u_out + oc * R.npairs * n_bins + b;
+    double sum = 0.0, comp = 0.0;
+    for (int32_t p = 0; p < R.npairs; ++p) {
+        const double x = a.w2[rays[p] >> 28] * u[int64_t(p) * n_bins];
+        const double t2 = sum + x;
+        comp += fabs(sum) >= fabs(x) ? (sum - t2) + x : (x - t2) + sum;
+        sum = t2;
+    }
+    a.J[(a.o_begin + oc) * n_bins + b] = sum + comp;
+}
+
+}  // namespace
+
+void launch_sum_pairs(const DevRays &R, const SolveArgs &a, int32_t n_bins, cudaStream_t st) {
+    const int64_t n = int64_t(a.o_end - a.o_begin) * n_bins;
+    if (n > 0) k_sum_pairs<<<unsigned((n + 127) / 128), 128, 0, st>>>(R, a, n_bins);
+}
+
 template void launch_solve_ord<2>(const DevMesh &, const DevLines &, const DevRays &, const SolveArgs &, int,
                                   cudaStream_t);
 template void launch_solve_queue_ord<2>(int, int, int, const BatchSlot *, const uint2 *, int64_t,

@@ -1919,11 +1919,13 @@ struct Occ {
         : (NL == 1 ? 9 : NL == 2 ? 8 : NL <= 4 ? 6 : 3);
 };
 
-// J of origin a.o_begin + oc for the bins of frequency tile `tile`, by one warp.
+// J of origin a.o_begin + oc for the bins of frequency tile vt / a.parts, by one
+// warp (a.parts > 1: u of its share vt % a.parts of the pairs).
 template <class C>
 __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln, const DevRays &Rs,
-                                           const SolveArgs &a, int32_t oc, int32_t tile, Stage<C> &sg, Lane<C> &ln,
+                                           const SolveArgs &a, int32_t oc, int32_t vt, Stage<C> &sg, Lane<C> &ln,
                                            int lane, const uint64_t *tab) {
+    const int32_t tile = a.parts > 1 ? vt / a.parts : vt, part = vt - tile * a.parts;
     using R = typename C::R;
     using P = typename C::P;
     constexpr int NL = C::NL, BPL = C::BPL, ORD = C::ORD;
@@ -2024,7 +2026,9 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
 #pragma unroll
     for (int i = 0; i < BPL; ++i) js[i] = jc[i] = 0.0;
 #pragma unroll 1
-    for (int32_t p = 0; p < Rs.npairs; ++p) {
+    for (int32_t p = int32_t(int64_t(Rs.npairs) * part / a.parts),
+                 p1 = int32_t(int64_t(Rs.npairs) * (part + 1) / a.parts);
+         p < p1; ++p) {
         const uint32_t ray = __ldg(Rs.rays + int64_t(o) * Rs.npairs + p);
         const int lev = int(ray >> 28);
         const int64_t hb = h0 + 2 * int64_t(p);
@@ -2087,7 +2091,7 @@ __device__ __forceinline__ void solve_item(const DevMesh &m, const DevLines &Ln,
     for (int i = 0; i < BPL; ++i) {
         const int32_t b = lane_bin<C>(sg, i, lane);
         if (b < NB) {
-            a.J[int64_t(o) * NB + b] = js[i] + jc[i];
+            if (a.parts == 1) a.J[int64_t(o) * NB + b] = js[i] + jc[i];
             ++n_act;
         }
     }
@@ -2121,7 +2125,7 @@ __device__ __forceinline__ const uint64_t *load_table(unsigned char *smem) {
     }
 }
 
-// Grid-mapped launch: warp w of the grid solves item w = oc * n_tiles + tile.
+// Grid-mapped launch: warp w of the grid solves item w = (oc * n_tiles + tile) * parts + part.
 template <class C>
 __global__ void __launch_bounds__(Occ<C>::kThreads, (Occ<C>::kMinBlocks))
 k_solve(const __grid_constant__ DevMesh m, const __grid_constant__ DevLines Ln, const __grid_constant__ DevRays Rs,
@@ -2132,9 +2136,9 @@ k_solve(const __grid_constant__ DevMesh m, const __grid_constant__ DevLines Ln, 
     const uint64_t *tab = load_table<C>(smem);
     const int lane = threadIdx.x & 31;
     const int64_t item = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-    const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles;
-    if (item >= n_items) return;
-    solve_item<C>(m, Ln, Rs, a, int32_t(item / a.n_tiles), int32_t(item % a.n_tiles), stage[threadIdx.x >> 5],
+    const int64_t per = int64_t(a.n_tiles) * a.parts;
+    if (item >= (a.o_end - a.o_begin) * per) return;
+    solve_item<C>(m, Ln, Rs, a, int32_t(item / per), int32_t(item % per), stage[threadIdx.x >> 5],
                   lanes[threadIdx.x >> 5], lane, tab);
 }
 
@@ -2181,7 +2185,7 @@ void prefer_shared(K kernel) {
 
 template <class C>
 void launch_one(const DevMesh &m, const DevLines &Ln, const DevRays &R_, const SolveArgs &a, cudaStream_t st) {
-    const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles;
+    const int64_t n_items = int64_t(a.o_end - a.o_begin) * a.n_tiles * a.parts;
     if (n_items == 0) return;
     constexpr int tb = Occ<C>::kThreads;
     const unsigned grid = unsigned((n_items * 32 + tb - 1) / tb);

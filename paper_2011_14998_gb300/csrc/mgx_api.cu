@@ -63,6 +63,9 @@ struct BatchPlan {
     std::vector<double *> J;
     std::vector<double *> Jdev;   // device staging of an output in host memory (null: J[k] is device memory)
     std::vector<size_t> Jbytes;
+    std::vector<SolveArgs> args;  // of each model, as its slot holds them
+    double *u = nullptr;          // u of every model when the pairs of an origin are dealt to several warps
+    int32_t parts = 1;
     mgx_solve_params p{};
     int32_t flags = 0;
     int64_t total_half = 0, n_origins = 0, n_work = 0, tail_cap = 0, total_points = 0;
@@ -416,6 +419,8 @@ void free_plan(mgx_ctx *ctx, BatchPlan &pl) {
     for (double *&q : pl.Jdev) dfree(ctx, q);
     pl.Jdev.clear();
     pl.Jbytes.clear();
+    pl.args.clear();
+    dfree(ctx, pl.u);
     dfree(ctx, pl.lens);
     dfree(ctx, pl.excess);
     dfree(ctx, pl.offs);
@@ -503,6 +508,8 @@ mgx_status enqueue_batch_back(mgx_ctx *ctx, BatchPlan &pl, std::vector<Model *> 
         Timed t(ctx, MGX_K_SOLVE);
         launch_solve_queue(pl.p.precision, pl.p.order == 4 ? 4 : 2, pl.bpl, pl.max_lines, pl.slots, pl.work, pl.n_work,
                            pl.scratch + kScratchQueue, ctx->stream);
+        for (size_t k = 0; pl.parts > 1 && k < ms.size(); ++k)
+            launch_sum_pairs(rays_view(ctx, *ms[k]), pl.args[k], ms[k]->L * ms[k]->F, ctx->stream);
     }
     CK(cudaGetLastError());
     return MGX_OK;
@@ -973,11 +980,16 @@ mgx_status mgx_solve_J(mgx_ctx *ctx, int32_t model, const mgx_solve_params *p, v
         a.status = ctx->d_status;
         a.counters = ctx->prof ? ctx->d_counters : nullptr;
         fill_pair_weights(a);
+        const size_t n_u = size_t(o1 - o0) * size_t(np) * size_t(NB);
+        a.parts = solve_parts(p->precision, int64_t(o1 - o0) * a.n_tiles, np, n_u * sizeof(double));
+        if (a.parts > 1) CK(dalloc(ctx, &a.u_out, n_u));
         {
             Timed t(ctx, MGX_K_SOLVE);
             launch_solve(dm, dl, dr, a, p->precision, p->order == 4 ? 4 : 2, ctx->stream);
+            if (a.parts > 1) launch_sum_pairs(dr, a, int32_t(NB), ctx->stream);
         }
         CK(cudaGetLastError());
+        dfree(ctx, a.u_out);
     }
     if (!p->out_on_device)
         CK(cudaMemcpyAsync(J_out, J, size_t(n) * size_t(NB) * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1062,7 +1074,6 @@ mgx_status mgx_solve_u(mgx_ctx *ctx, int32_t model, const mgx_solve_params *p, i
     int32_t *aidx = nullptr;
     double *J = nullptr, *u = nullptr;
     CK(dalloc(ctx, &aidx, size_t(std::max<int64_t>(total, 1))));
-    CK(dalloc(ctx, &J, size_t(m->n) * size_t(NB)));  // the kernel indexes J by absolute origin
     if (p->out_on_device) u = u_out;
     else CK(dalloc(ctx, &u, n_u));
     const DevMesh dm = mesh_view(*m);
@@ -1081,8 +1092,10 @@ mgx_status mgx_solve_u(mgx_ctx *ctx, int32_t model, const mgx_solve_params *p, i
     a.offs = offs;
     a.base = 0;
     a.idx = aidx;
-    a.J = J;
     a.u_out = u;
+    a.parts = solve_parts(p->precision, int64_t(o1 - o0) * a.n_tiles, np, 0);
+    if (a.parts == 1) CK(dalloc(ctx, &J, size_t(m->n) * size_t(NB)));  // the kernel indexes J by absolute origin
+    a.J = J;
     a.status = ctx->d_status;
     a.counters = ctx->prof ? ctx->d_counters : nullptr;
     fill_pair_weights(a);
@@ -1235,12 +1248,25 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
     std::vector<BatchGeom> geo(static_cast<size_t>(n_models));
     std::vector<int64_t> obase(static_cast<size_t>(n_models));
     pl.total_half = pl.n_origins = pl.n_work = 0;
+    // few items: the pairs of an origin are dealt to several warps (solve_parts)
+    int64_t n_items = 0;
+    size_t n_u = 0;
+    int32_t min_pairs = INT32_MAX, max_tiles = 1;
+    for (const Model *m : ms) {
+        const int64_t nb = int64_t(m->L) * m->F, tiles = (nb + 32 * pl.bpl - 1) / (32 * pl.bpl);
+        n_items += m->n * tiles;
+        n_u += size_t(m->n) * size_t(m->npairs) * size_t(nb);
+        min_pairs = std::min(min_pairs, m->npairs);
+        max_tiles = std::max(max_tiles, int32_t(std::min<int64_t>(tiles, 65535)));
+    }
+    pl.parts = std::min(solve_parts(p->precision, n_items, min_pairs, n_u * sizeof(double)), 65535 / max_tiles);
+    if (pl.parts > 1) CK(dalloc(ctx, &pl.u, n_u));
     for (int32_t k = 0; k < n_models; ++k) {
         const Model &m = *ms[size_t(k)];
         const int64_t nb = int64_t(m.L) * m.F;
         geo[size_t(k)].half_base = pl.total_half;
         geo[size_t(k)].npairs2 = 2 * m.npairs;
-        geo[size_t(k)].n_tiles = int32_t((nb + 32 * pl.bpl - 1) / (32 * pl.bpl));
+        geo[size_t(k)].n_tiles = int32_t((nb + 32 * pl.bpl - 1) / (32 * pl.bpl)) * pl.parts;
         obase[size_t(k)] = pl.n_origins;
         pl.total_half += int64_t(m.n) * m.npairs * 2;
         pl.n_origins += m.n;
@@ -1330,6 +1356,7 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
     pl.total_points = int64_t(tot[kPadCandidates]);
     CK(dalloc(ctx, &pl.tail, size_t(std::max<int64_t>(pl.tail_cap, 1))));
     std::vector<BatchSlot> slots(static_cast<size_t>(n_models));
+    size_t u_off = 0;
     for (int32_t k = 0; k < n_models; ++k) {
         Model &m = *ms[size_t(k)];
         BatchSlot &b = slots[size_t(k)];
@@ -1342,7 +1369,10 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
         a.I_bdy = p->I_bdy;
         a.o_begin = 0;
         a.o_end = m.n;
-        a.n_tiles = geo[size_t(k)].n_tiles;
+        a.parts = pl.parts;
+        a.n_tiles = geo[size_t(k)].n_tiles / pl.parts;
+        if (pl.parts > 1) a.u_out = pl.u + u_off;
+        u_off += size_t(m.n) * size_t(m.npairs) * size_t(m.L) * size_t(m.F);
         a.offs = pl.offs + geo[size_t(k)].half_base;
         a.base = 0;
         a.idx = pl.rows + geo[size_t(k)].half_base * pl.pad;
@@ -1353,6 +1383,7 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
         a.status = ctx->d_status;
         a.counters = ctx->prof ? ctx->d_counters : nullptr;
         fill_pair_weights(a);
+        pl.args.push_back(a);
         ctx->solves += int64_t(m.n) * m.npairs * int64_t(m.L) * m.F;
     }
     ctx->trace_points += pl.total_points;

@@ -79,7 +79,8 @@ struct SolveArgs {
     const int64_t *lens = nullptr;  // padded: half-ray lengths
     const int32_t *tail = nullptr;  // padded: entries beyond the row
     double *u_out = nullptr;        // optional: u per (origin - o_begin, pair, bin)
-    double *J;                // [n][L*F]
+    int32_t parts = 1;        // > 1: an origin's pairs are dealt to that many warps per tile, which store u only
+    double *J;                // [n][L*F] (not written when parts > 1)
     int *status;
     unsigned long long *counters;  // nullable: [0] elimination updates, [1] optics samples,
                                    // [2] tracer steps, [3] tracer steps redone in double
@@ -173,6 +174,10 @@ void launch_excess_totals(const int64_t *lens, int64_t n, unsigned long long *ou
 // frequency bins per lane of the solve kernel; a chunk has
 // ceil(n_bins / (32 * bins_per_lane)) tiles per origin
 int solve_bins_per_lane(int precision, int order, int32_t n_lines, int32_t n_bins);
+// parts (SolveArgs::parts) for n_items (origin, tile) items of npairs pairs whose u takes u_bytes; 1: none
+int32_t solve_parts(int precision, int64_t n_items, int32_t npairs, size_t u_bytes);
+// J of origins [o_begin, o_end) from u (a solve with parts > 1)
+void launch_sum_pairs(const DevRays &R, const SolveArgs &a, int32_t n_bins, cudaStream_t st);
 // order: 2 (second-order scheme) or 4 (Hermitian scheme)
 void launch_solve(const DevMesh &m, const DevLines &Ln, const DevRays &R, const SolveArgs &a,
                   int precision, int order, cudaStream_t st);

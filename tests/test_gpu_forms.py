@@ -29,3 +29,33 @@ def test_forms_at_tile_edges(orc, lines, bins, precision, order, tol):
         ctx.close()
     Jo = orc.OracleModel(m, rays=rays).solve_J(orc.params(I_bdy=0.05, order=order))
     assert j_rel_err(J, Jo)[0] < tol
+
+
+@pytest.mark.parametrize("n,l_min,l_max", [(8, 0, 0), (27, 1, 1), (60, 0, 2), (300, 2, 2)])
+@pytest.mark.parametrize("precision", ["FP32", "FP64"])
+def test_pairs_dealt_to_several_warps(orc, n, l_min, l_max, precision):
+    """Few origins: the pairs of an origin are solved by several warps.  J of the per-model and
+    the batched call (alone and next to a larger model, which changes the share) is the same
+    bit for bit, and the sum of solve_u over the pairs."""
+    import paper_2011_14998_gb300 as mgx
+
+    prec = getattr(mgx, "MGX_" + precision)
+    m = synth.random_cloud(n, seed=n, n_lines=2, n_freq=20, l_min=l_min, l_max=l_max)
+    big = synth.wind_model(3000, seed=1, n_freq=20, level=1)
+    ctx = mgx.Context(0)
+    try:
+        mid, bid = ctx.load(m), ctx.load(big)
+        J = ctx.solve_J(mid, precision=prec)
+        alone = ctx.solve_J_batch([mid], precision=prec)[0].cpu().numpy()
+        both = ctx.solve_J_batch([bid, mid], precision=prec)
+        u = ctx.solve_u(mid, 0, n, precision=prec)
+        w = 2.0 / (12.0 * 4.0 ** (ctx.rays(mid) >> 28))
+        rays = ctx.rays(mid)
+        Jb = ctx.solve_J(bid, precision=prec)
+    finally:
+        ctx.close()
+    np.testing.assert_array_equal(J, alone)
+    np.testing.assert_array_equal(J, both[1].cpu().numpy())
+    np.testing.assert_array_equal(Jb, both[0].cpu().numpy())
+    np.testing.assert_allclose((w[:, :, None] * u).sum(1), J, rtol=1e-12)
+    assert j_rel_err(J, orc.OracleModel(m, rays=rays).solve_J(orc.params()))[0] < (1e-4 if precision == "FP32" else 1e-10)

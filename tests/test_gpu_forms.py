@@ -41,7 +41,8 @@ def test_pairs_dealt_to_several_warps(orc, n, l_min, l_max, precision):
 
     prec = getattr(mgx, "MGX_" + precision)
     m = synth.random_cloud(n, seed=n, n_lines=2, n_freq=20, l_min=l_min, l_max=l_max)
-    big = synth.wind_model(3000, seed=1, n_freq=20, level=1)
+    # as many lines and bins as m: another bin count would take another compiled form in the batch
+    big = synth.with_lines(synth.wind_model(3000, seed=1, n_freq=20, level=1), 2, 20)
     ctx = mgx.Context(0)
     try:
         mid, bid = ctx.load(m), ctx.load(big)

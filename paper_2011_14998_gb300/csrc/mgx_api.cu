@@ -1707,20 +1707,22 @@ mgx_status mgx_mlp_features(mgx_ctx *ctx, int32_t model, const double *rho, cons
             return fail(ctx, MGX_EINVAL, "mlp_features: rho and T must be positive and finite (point %lld)", (long long)i);
     DeviceGuard g(ctx->device);
     const size_t n = size_t(m->n);
-    double *rd = nullptr, *Td = nullptr;
+    double *rd = nullptr, *Td = nullptr, *lr = nullptr;
     float *Xd = nullptr;
     CK(dalloc(ctx, &rd, n));
+    CK(dalloc(ctx, &lr, n));
     CK(dalloc(ctx, &Td, n));
     CK(dalloc(ctx, &Xd, n * 8));
     CK(cudaMemcpyAsync(rd, rho, n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(Td, T, n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     {
         Timed t(ctx, MGX_K_OTHER);
-        launch_mlp_features(mesh_view(*m), m->chi0f, m->L, m->dvwf, rd, Td, Xd, ctx->stream);
+        launch_mlp_features(mesh_view(*m), m->chi0f, m->L, m->dvwf, rd, Td, lr, Xd, ctx->stream);
     }
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(X, Xd, n * 8 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     dfree(ctx, rd);
+    dfree(ctx, lr);
     dfree(ctx, Td);
     dfree(ctx, Xd);
     return sync_status(ctx);
@@ -1762,6 +1764,9 @@ mgx_status mgx_reduce_mesh_learned(mgx_ctx *ctx, int32_t model, const float *X, 
     return s;
 }
 
+// Newton steps of the weighted thinning between two looks of the host.
+constexpr int kThinSteps = 12;
+
 mgx_status mgx_reduce_mesh_learned_weighted(mgx_ctx *ctx, int32_t model, const float *X, double keep_fraction,
                                             double alpha, uint64_t seed, uint8_t *keep, int64_t *n_kept,
                                             double *scale) {
@@ -1776,7 +1781,7 @@ mgx_status mgx_reduce_mesh_learned_weighted(mgx_ctx *ctx, int32_t model, const f
     const int64_t n = m->n;
     const double target = keep_fraction * double(n);
     float *Xd = nullptr, *yd = nullptr, *wd = nullptr;
-    double *sd = nullptr;
+    ThinSolve *sd = nullptr;
     unsigned long long *cnt = nullptr;
     uint8_t *kd = nullptr;
     CK(dalloc(ctx, &Xd, size_t(n) * 8));
@@ -1792,18 +1797,18 @@ mgx_status mgx_reduce_mesh_learned_weighted(mgx_ctx *ctx, int32_t model, const f
         launch_mlp(false, Xd, nullptr, nullptr, n, ctx->mlp_W1b, ctx->mlp_W2b, ctx->mlp_theta, yd, nullptr, nullptr,
                    0.0f, ctx->stream);
         launch_thin_weights(yd, n, float(alpha), wd, ctx->stream);
-        // bisection on log2 c: the expected kept count grows with c
-        double lo = -400.0, hi = 400.0;
-        for (int it = 0; it < 80 && keep_fraction > 0.0 && keep_fraction < 1.0; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            double sum = 0.0;
-            launch_thin_expected(wd, n, std::exp2(mid), sd, ctx->stream);
-            CK(cudaMemcpyAsync(&sum, sd, sizeof sum, cudaMemcpyDeviceToHost, ctx->stream));
-            CK(cudaStreamSynchronize(ctx->stream));
-            if (sum < target) lo = mid;
-            else hi = mid;
+        c = keep_fraction <= 0.0 ? 0.0 : 1e300;
+        if (keep_fraction > 0.0 && keep_fraction < 1.0) {
+            ThinSolve h{};
+            CK(cudaMemsetAsync(sd, 0, sizeof h, ctx->stream));
+            // each step saturates at least one more point, so n + 2 steps always end it
+            for (int64_t it = 0; it < n + 2 && !h.done; it += kThinSteps) {
+                for (int k = 0; k < kThinSteps; ++k) launch_thin_newton(wd, n, target, sd, ctx->stream);
+                CK(cudaMemcpyAsync(&h, sd, sizeof h, cudaMemcpyDeviceToHost, ctx->stream));
+                CK(cudaStreamSynchronize(ctx->stream));
+            }
+            c = h.c;
         }
-        c = keep_fraction <= 0.0 ? 0.0 : keep_fraction >= 1.0 ? 1e300 : std::exp2(0.5 * (lo + hi));
         launch_thin_mark(wd, n, c, seed, kd, cnt, ctx->stream);
     }
     CK(cudaGetLastError());

@@ -217,10 +217,15 @@ void launch_size_map(int64_t n, const double *Gf, const unsigned long long *mm, 
                      double ell_max, uint64_t seed, double *ell, uint8_t *keep, unsigned long long *kept,
                      cudaStream_t st);
 
-// ---- score-weighted thinning (k_thin.cu): w = 10^(alpha y); expected kept
-// count for a scale c; the coin flips
+// ---- score-weighted thinning (k_thin.cu): w = 10^(alpha y); the scale at
+// which the expected kept count meets the target; the coin flips
+struct ThinSolve {  // zeroed before the first step (c = 0: no point saturated)
+    double c, sum;
+    unsigned long long sat, last;
+    unsigned int blocks, steps, done, pad;
+};
 void launch_thin_weights(const float *y, int64_t n, float alpha, float *w, cudaStream_t st);
-void launch_thin_expected(const float *w, int64_t n, double c, double *sum, cudaStream_t st);
+void launch_thin_newton(const float *w, int64_t n, double target, ThinSolve *s, cudaStream_t st);
 void launch_thin_mark(const float *w, int64_t n, double c, uint64_t seed, uint8_t *keep, unsigned long long *kept,
                       cudaStream_t st);
 
@@ -246,7 +251,7 @@ void launch_mlp(bool train, const float *X, const float *t, const int32_t *perm,
 void launch_mlp_adam(float *theta, float *m, float *v, float *grad, float lr, float b1, float b2, float eps, float c1,
                      float c2, void *W1b, void *W2b, cudaStream_t st);
 void launch_mlp_features(const DevMesh &m, const float *chi0, int32_t L, const float *dvw, const double *rho,
-                         const double *T, float *X, cudaStream_t st);
+                         const double *T, double *log_rho, float *X, cudaStream_t st);
 void launch_select_top(const float *score, int64_t n, int64_t k, int32_t *ids, float *score_sorted,
                        int32_t *ids_sorted, uint8_t *keep, cudaStream_t st);
 

@@ -45,6 +45,7 @@ struct Model {
     int32_t lmin = 0, lmax = 0, npairs = 0;
     uint32_t *rays = nullptr;
     int32_t *sample = nullptr;  // device copy of the ray-set sample (adaptive sets)
+    float4 *split = nullptr;    // its positions, split (working memory of the ray-set kernel)
     int64_t n_sample = 0;
     // half-ray offsets of every origin, [2 n npairs + 1] on the device, and
     // their values at origin boundaries, [n + 1] on the host: made by the first
@@ -366,6 +367,7 @@ void free_model(mgx_ctx *ctx, Model &m) {
     free_lines(ctx, m);
     dfree(ctx, m.rays);
     dfree(ctx, m.sample);
+    dfree(ctx, m.split);
     drop_offsets(ctx, m);
     m.has_rays = false;
     m.live = false;
@@ -451,7 +453,7 @@ void enqueue_rays(mgx_ctx *ctx, Model &m, bool timed = true) {
     if (m.lmin == m.lmax) {
         launch_rays_fixed(m.n, m.lmin, m.npairs, ctx->pair_lists_dev[size_t(m.lmin)], m.rays, ctx->stream);
     } else {
-        launch_rays_adaptive(mesh_view(m), m.lmin, m.lmax, m.npairs, m.n_sample, m.sample, ctx->anti,
+        launch_rays_adaptive(mesh_view(m), m.lmin, m.lmax, m.npairs, m.n_sample, m.sample, m.split, ctx->anti,
                              ctx->pair_lists_dev[size_t(m.lmin)], int32_t(ctx->pair_lists[size_t(m.lmin)].size()),
                              m.rays, ctx->d_status, ctx->stream);
     }
@@ -813,13 +815,15 @@ mgx_status mgx_set_rays(mgx_ctx *ctx, int32_t model, int32_t l_min, int32_t l_ma
         CK(cudaGetLastError());
     } else {
         dfree(ctx, m->sample);
+        dfree(ctx, m->split);
         CK(dalloc(ctx, &m->sample, size_t(n_sample)));
+        CK(dalloc(ctx, &m->split, size_t(n_sample) * 2));
         m->n_sample = n_sample;
         if (n_sample > 0)
             CK(cudaMemcpyAsync(m->sample, sample, size_t(n_sample) * sizeof(int32_t), cudaMemcpyHostToDevice,
                                ctx->stream));
         Timed t(ctx, MGX_K_RAYS);
-        launch_rays_adaptive(mesh_view(*m), l_min, l_max, m->npairs, n_sample, m->sample, ctx->anti,
+        launch_rays_adaptive(mesh_view(*m), l_min, l_max, m->npairs, n_sample, m->sample, m->split, ctx->anti,
                              ctx->pair_lists_dev[size_t(l_min)], int32_t(ctx->pair_lists[size_t(l_min)].size()),
                              m->rays, ctx->d_status, ctx->stream);
         CK(cudaGetLastError());

@@ -108,8 +108,9 @@ void launch_ingest_lines(int32_t n, int32_t L, const double *chi0, const double 
 // ---- ray sets (k_rays.cu)
 void launch_rays_fixed(int32_t n, int32_t level, int32_t npairs, const uint32_t *pairs,
                        uint32_t *rays, cudaStream_t st);
+// (split: 2 n_sample float4 of working memory)
 void launch_rays_adaptive(const DevMesh &m, int32_t lmin, int32_t lmax, int32_t npairs,
-                          int64_t n_sample, const int32_t *sample, const int32_t *anti,
+                          int64_t n_sample, const int32_t *sample, float4 *split, const int32_t *anti,
                           const uint32_t *pairs_lmin, int32_t n_pairs_lmin, uint32_t *rays,
                           int *status, cudaStream_t st);
 

@@ -130,4 +130,57 @@ __host__ __device__ __forceinline__ double div_pos(double e, double t) {
     return bits_double(((s2 + 256) >> 9) + (uint64_t(int64_t(1022 + ex - int(low))) << 52));
 }
 
+// x in [0, 2) in Q1.62, rounded down.
+__host__ __device__ __forceinline__ uint64_t to_q62(double x) {
+    const uint64_t b = double_bits(x);
+    const uint32_t s = 1023u - uint32_t(b >> 52);
+    const uint64_t m = ((b << 10) & ((uint64_t(1) << 62) - 1)) | (uint64_t(1) << 62);
+    return s < 64u ? m >> s : 0;
+}
+
+// v 2^-62 for v in [2^59, 2^62], to the nearest double (halves up).
+__host__ __device__ __forceinline__ double from_q62(uint64_t v) {
+#ifdef __CUDA_ARCH__
+    const int sh = __clzll((long long)v) - 1;
+#else
+    const int sh = __builtin_clzll(v) - 1;
+#endif
+    return bits_double((((v << sh) + 512) >> 10) + (uint64_t(1022 - sh) << 52));
+}
+
+// v 2^-61 for v below 2^63, to the nearest double (0 for 0).
+__host__ __device__ __forceinline__ double from_q61(uint64_t v) {
+#ifdef __CUDA_ARCH__
+    return __ull2double_rn(v) * 0x1p-61;
+#else
+    return double(v) * 0x1p-61;
+#endif
+}
+
+// One pivot of the scaled elimination in fixed point: with Y = D Fh of the row
+// before (Q2.61), the increment t < 1.01 (Q1.62) and b, its mean with the one
+// before (Q2.61):  Fh = b + Y,  D = 1 / (1 + t Fh) (returned, Q0.62),  Y = D Fh.
+// The scaled quantities are of order one (Y at most about 2), so 59 fraction
+// bits are more than a double's 53; the reciprocal is a single-precision one
+// with one correction and its square.
+__host__ __device__ __forceinline__ uint64_t pivot_q(uint64_t t, uint64_t b, uint64_t &Y) {
+    const uint64_t F = b + Y;
+    const uint64_t den = (uint64_t(1) << 59) + mul_hi63(t, F);  // Q4.59, in [1, 4)
+    const uint32_t top = uint32_t(den >> 30);                   // Q2.29
+#ifdef __CUDA_ARCH__
+    float x;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(float(top)));  // 2^-29 / den
+    const uint32_t X = __float2uint_rz(x * 1152920954851033088.0f);  // Q0.31, low by up to 2^-20
+#else
+    const uint32_t X = uint32_t(1.0f / float(top) * 1152920954851033088.0f);
+#endif
+    const uint64_t dx = uint64_t(uint32_t(den >> 32)) * X + mul_hi32(uint32_t(den), X);  // den X in Q.58
+    uint64_t d = (uint64_t(1) << 58) - dx;  // 1 - den X in [0, 2^-20.5)
+    const uint32_t dh = uint32_t((d + (1u << 21)) >> 22);
+    d += (dh * dh) >> 14;                   // its square (the cube is below 2^-61)
+    const uint64_t D = (uint64_t(X) << 31) + (mul_hi63(uint64_t(X) << 31, d << 23) >> 17);
+    Y = mul_hi63(F, D) << 2;
+    return D;
+}
+
 }  // namespace mgx

@@ -233,6 +233,7 @@ struct Sweep {
     R zh;
     R chi, eta;     // optics of the current (not yet eliminated) sample
     R Sp, Sc, hp, rh;  // Hermitian scheme only
+    uint64_t Y;        // double-precision pivots with R = float: D Fh in Q2.61 (Fh, Dm not kept)
 };
 
 // The second-order row below for two bins at once, operation for operation.
@@ -271,19 +272,29 @@ constexpr double kHermRatio = 64.0;
 
 template <int ORD, typename R, typename P>
 __device__ __forceinline__ void row(Sweep<R, P> &w, R chi, R eta, P dt, R Si, R Sn) {
-    if constexpr (ORD == 2) {
+    if constexpr (ORD == 2 && sizeof(P) != sizeof(R)) {
+        // pivots of double's precision: D = 1 / (1 + dt Fh) in fixed point (pivot_q; of the
+        // 22 FP64 instructions a row took, the reciprocal most, six are left); z in single
+        // precision from D and S = eta / chi
+        const P dtb = fma(dt, P(0.5), w.dtp);
+        P D;
+        if (dt < P(1)) {
+            const uint64_t t = to_q62(dt);
+            D = from_q62(pivot_q(t, to_q62(dtb) >> 1, w.Y));
+        } else {  // thick cells without optical-depth sampling (dtau_max > 1)
+            const P Fh = dtb + from_q61(w.Y);
+            D = P(1) / (P(1) + dt * Fh);
+            w.Y = to_q62(D * Fh) >> 1;
+        }
+        w.zh = R(D) * w.zh + R(dtb * D) * (eta * Ar<R>::rcp(chi));
+        w.dtp = dt * P(0.5);
+    } else if constexpr (ORD == 2) {
         const P dtb = fma(dt, P(0.5), w.dtp);
         w.Fh = dtb + w.Dm * w.Fh;
-        if constexpr (sizeof(P) == sizeof(R)) {
+        {
             const R rr = Ar<R>::rcp(chi * (R(1) + dt * w.Fh));
             w.Dm = chi * rr;
             w.zh = w.Dm * w.zh + dtb * (eta * rr);
-        } else {
-            // pivots in double precision: D = 1 / (1 + dt Fh); z in single
-            // precision from D and S = eta / chi
-            const P D = P(1) / (P(1) + dt * w.Fh);
-            w.Dm = D;
-            w.zh = R(D) * w.zh + R(dtb * D) * (eta * Ar<R>::rcp(chi));
         }
         w.dtp = dt * P(0.5);
     } else {
@@ -1310,6 +1321,7 @@ __device__ __forceinline__ void put_sweep(Lane<C> &ln, const Sweep<typename C::V
 #pragma unroll
     for (int i = 0; i < C::NV; ++i) {
         if constexpr (C::kPacked) ln.wp[0][i][lane] = vmul(w[i].Dm, w[i].Fh);
+        else if constexpr (sizeof(typename C::P) != sizeof(typename C::R)) ln.wp[0][i][lane] = from_q61(w[i].Y);
         else ln.wp[0][i][lane] = w[i].Dm * w[i].Fh;
         ln.wp[1][i][lane] = w[i].dtp;
         ln.wr[0][i][lane] = w[i].zh;
@@ -1330,6 +1342,7 @@ __device__ __forceinline__ void get_sweep(const Lane<C> &ln, Sweep<typename C::V
     using R = typename C::R;
 #pragma unroll
     for (int i = 0; i < C::NV; ++i) {
+        if constexpr (sizeof(typename C::P) != sizeof(typename C::R)) w[i].Y = to_q62(ln.wp[0][i][lane]) >> 1;
         w[i].Fh = ln.wp[0][i][lane];
         w[i].Dm = vset<typename C::W>(1.f);
         w[i].dtp = ln.wp[1][i][lane];
@@ -1841,6 +1854,7 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
             else w[i].zh = R(a.I_bdy);
             w[i].hp = vset<V>(-1.f);  // no row yet (Hermitian scheme)
             w[i].Sp = w[i].Sc = w[i].rh = w[i].chi = w[i].eta = vset<V>(0.f);
+            w[i].Y = uint64_t(1) << 61;
         }
         put_sweep<C>(ln, w, lane);
     }

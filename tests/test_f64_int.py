@@ -7,7 +7,9 @@
   |a| = 8, 2^-52 above), times ln 2; the polynomial's 32-bit product below 2^-55
   and the table's 32 units of 2^-62: 2^-53.8 below |a| = 8 and 2^-50.8 above,
   plus half an ulp of rounding;
-* division: 2^-55 plus half an ulp.
+* division: 2^-55 plus half an ulp;
+* pivot: operands and products to 2^-59, the reciprocal's square term to 2^-56:
+  D within 2^-55 (relative) plus half an ulp, Y within 2^-54.
 CPU only."""
 import ctypes as C
 import os
@@ -24,6 +26,9 @@ SRC = """
 static constexpr mgx::Exp2Table tab;
 extern "C" double t_exp(uint64_t A) { return mgx::exp2_neg_sq(A, tab.v); }
 extern "C" double t_div(double e, double t) { return mgx::div_pos(e, t); }
+extern "C" double t_piv(double t, double b, uint64_t *Y) {
+    return mgx::from_q62(mgx::pivot_q(mgx::to_q62(t), mgx::to_q62(b) >> 1, *Y));
+}
 extern "C" uint64_t t_tab(int j) { return tab.v[j]; }
 """
 
@@ -38,6 +43,7 @@ def lib(tmp_path_factory):
     L = C.CDLL(so)
     L.t_exp.restype, L.t_exp.argtypes = C.c_double, [C.c_uint64]
     L.t_div.restype, L.t_div.argtypes = C.c_double, [C.c_double, C.c_double]
+    L.t_piv.restype, L.t_piv.argtypes = C.c_double, [C.c_double, C.c_double, C.POINTER(C.c_uint64)]
     L.t_tab.restype, L.t_tab.argtypes = C.c_uint64, [C.c_int]
     return L
 
@@ -76,3 +82,20 @@ def test_division(lib):
     for x, y in [(0.0, 3.0), (1e-320, 3.0), (3.0, 1e-320), (1e300, 1e-300), (1e-300, 1e300)]:
         with np.errstate(over="ignore", under="ignore"):
             assert lib.t_div(x, y) == float(np.float64(x) / np.float64(y))
+
+
+def test_pivot(lib):
+    """Chains of fixed-point pivots against the recurrence in 40 digits, each step from its own Y."""
+    mp.mp.dps = 40
+    rng = np.random.default_rng(10)
+    for chain in range(60):
+        Y, tp = C.c_uint64(1 << 61), 0.0
+        for _ in range(60):
+            t = float(rng.uniform(0, 1) if chain % 3 == 0 else 10.0 ** rng.uniform(-14, 0))
+            b = 0.5 * t + tp
+            F = mp.mpf(b) + mp.mpf(Y.value) / mp.mpf(2) ** 61
+            D = 1 / (1 + mp.mpf(t) * F)
+            got = lib.t_piv(t, b, C.byref(Y))
+            assert abs(mp.mpf(got) - D) <= (2.0 ** -55 + 2.0 ** -53) * D
+            assert abs(mp.mpf(Y.value) / mp.mpf(2) ** 61 - D * F) <= 2.0 ** -54
+            tp = 0.5 * t

@@ -783,8 +783,9 @@ __device__ __forceinline__ bool line_is_far(double dl, double rdv, double cc, do
 }
 
 // Record of the integer form: a quarter of the distance to the previous sample,
-// eta_c / chi_c, chi_c, eta_c, the profile argument's two terms, then chi0 and
-// eta0 of each line.  One line: the argument of bin k is alpha + u_k gamma with
+// eta_c / chi_c, chi_c, eta_c, the profile argument's two terms (a sample on
+// which no line takes part: half the increment if it was so at the sample
+// before too, and its sum with the one before), then chi0 and eta0 of each line.  One line: the argument of bin k is alpha + u_k gamma with
 // u_k = (ub_k / span + 1) / 2 (the bin's velocity ub within its range +-span),
 // alpha in Q6.57 and gamma scaled by the largest power
 // of two that keeps it below 2^63 (the shift back in its lowest three bits),
@@ -1505,8 +1506,8 @@ struct IntSweep {
     double N, Q, W, T, S, h;  // T, S: opacity and source function of the current sample; h: half the last increment
 };
 
-__device__ __forceinline__ void int_row(IntSweep &w, double S, double h) {
-    const double p = (w.h + h) * w.Q;
+__device__ __forceinline__ void int_row(IntSweep &w, double S, double h, double b) {
+    const double p = b * w.Q;  // b: dtb = the sum of the last half increment and this one
     w.N += p;
     w.W = fma(S, p, w.W);
     w.Q = fma(h, __hiloint2double(__double2hiint(w.N) + 0x100000, __double2loint(w.N)), w.Q);  // h 2N
@@ -1607,17 +1608,20 @@ __device__ __forceinline__ bool int_split_step(const double *src, unsigned on, b
             const double rn = 1.0 / double(n[i]), qs = q * rn;
             const double c0 = w[i].T, e0 = w[i].S * c0;
             const double dc = (chi[i] - c0) * rn, de = (eta[i] - e0) * rn;
-            double cp = c0, Sp = w[i].S;
+            double cp = c0, Sp = w[i].S, h;
 #pragma unroll 1
             for (int k = 1; k < n[i]; ++k) {
                 const double ck = fma(dc, double(k), c0), ek = fma(de, double(k), e0);
-                int_row(w[i], Sp, qs * (cp + ck));
+                h = qs * (cp + ck);
+                int_row(w[i], Sp, h, w[i].h + h);
                 cp = ck;
                 Sp = ek > 0.0 ? div_pos(ek, ck) : 0.0;
             }
-            int_row(w[i], Sp, qs * (cp + chi[i]));
+            h = qs * (cp + chi[i]);
+            int_row(w[i], Sp, h, w[i].h + h);
         } else {
-            int_row(w[i], w[i].S, q * (w[i].T + chi[i]));
+            const double h = q * (w[i].T + chi[i]);
+            int_row(w[i], w[i].S, h, w[i].h + h);
         }
         w[i].T = chi[i];
         w[i].S = S;
@@ -1661,6 +1665,13 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
                 sg.m_wild = m_wild;
             }
             __syncwarp();
+            if (lane > 0 && lane < nr && cls == 0u) {
+                double *o = sg.rec + lane * kS;
+                const double h = o[0] * (o[2 - kS] + o[2]);
+                o[4] = h;
+                o[5] = lane > 1 ? o[-kS] * (o[2 - 2 * kS] + o[2 - kS]) + h : h;
+            }
+            __syncwarp();
         } else {
             m_split = sg.m_split;
             m_new = sg.m_new;
@@ -1680,11 +1691,15 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
             const double *end = sg.rec + e * kS;
             s = e;
             if (on == 0u) {
+                // the continuum: from the run's second sample on the increments are the same
+                // for every bin, from the third their means too, and come with the record
+                int k = 0;
 #pragma unroll 1
-                for (; src < end; src += kS) {
+                for (; src < end; src += kS, ++k) {
 #pragma unroll
                     for (int i = 0; i < C::BPL; ++i) {
-                        int_row(w[i], w[i].S, src[0] * (w[i].T + src[2]));
+                        const double h = k > 0 ? src[4] : src[0] * (w[i].T + src[2]);
+                        int_row(w[i], w[i].S, h, k > 1 ? src[5] : w[i].h + h);
                         w[i].T = src[2];
                         w[i].S = src[1];
                     }
@@ -1696,7 +1711,8 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
                     for (int i = 0; i < C::BPL; ++i) {
                         double chi, eta;
                         int_optics<C>(src, on, sg, tab, i, u[i], chi, eta);
-                        int_row(w[i], w[i].S, src[0] * (w[i].T + chi));
+                        const double h = src[0] * (w[i].T + chi);
+                        int_row(w[i], w[i].S, h, w[i].h + h);
                         w[i].T = chi;
                         w[i].S = div_pos(eta, chi);
                     }

@@ -430,6 +430,8 @@ struct Stage {
     double z[sizeof(R) == 8 ? 33 : 1];      // exact Z (single precision: the carried point's only)
     int id[33], nv[33], so[33];             // point (-1: the origin), velocity samples, their offset
     unsigned on[C::kInt ? kCap : 1];        // integer form: the lines that take part in each record
+    unsigned m_block;                       // records at which a block of kBlock continuum rows starts
+    double blk[C::kInt ? kCap / 8 : 1][6];  // and the blocks' maps (block of record s in blk[s / 8])
     double span;                            // integer form, one line: x_span dvw_o, the bins' half-range in km/s
     uint64_t uk[C::kInt && NL == 1 ? BPL : 1][32];  // and each lane's bins' place in it, (ub / span + 1) / 2, in Q0.63
     R Am[NL], Bm[NL];                       // largest |A|, |B| of each line over the warp's bins
@@ -1506,18 +1508,22 @@ struct IntSweep {
     double N, Q, W, T, S, h;  // T, S: opacity and source function of the current sample; h: half the last increment
 };
 
-__device__ __forceinline__ void int_row(IntSweep &w, double S, double h, double b) {
-    const double p = b * w.Q;  // b: dtb = the sum of the last half increment and this one
-    w.N += p;
-    w.W = fma(S, p, w.W);
-    w.Q = fma(h, __hiloint2double(__double2hiint(w.N) + 0x100000, __double2loint(w.N)), w.Q);  // h 2N
-    w.h = h;
+__device__ __forceinline__ void int_rescale(IntSweep &w) {
     if (__double2hiint(w.Q) > 0x52b00000) {  // 2^300
         const double f = bits_double(uint64_t(2046 - (__double2hiint(w.Q) >> 20)) << 52);
         w.N *= f;
         w.Q *= f;
         w.W *= f;
     }
+}
+
+__device__ __forceinline__ void int_row(IntSweep &w, double S, double h, double b) {
+    const double p = b * w.Q;  // b: dtb = the sum of the last half increment and this one
+    w.N += p;
+    w.W = fma(S, p, w.W);
+    w.Q = fma(h, __hiloint2double(__double2hiint(w.N) + 0x100000, __double2loint(w.N)), w.Q);  // h 2N
+    w.h = h;
+    int_rescale(w);
 }
 
 // Opacity and emissivity of record src for bin i of the lane, over the lines in `on`.
@@ -1629,6 +1635,61 @@ __device__ __forceinline__ bool int_split_step(const double *src, unsigned on, b
     return true;
 }
 
+// Rows on which no line takes part are the same linear map for every bin:
+//   (N, Q) -> ((1, b), (t, 1 + t b)) (N, Q),   W -> W + S b Q.
+// Eight consecutive ones are composed into one map, six operations a bin in
+// place of 32; the lanes hold one row each and compose them in three doubling
+// steps (36 operations a round of records).  A block starts at the third
+// record of a run (the first two rows still depend on the bin), or where the
+// last block ended.  Not where an increment is so large that the map's entries
+// could leave the range of the state.  bound: the records at which a run
+// begins.  Returns the records at which a block starts.
+constexpr int kBlock = 8;
+
+template <class C>
+__device__ __forceinline__ unsigned compose_blocks(Stage<C> &sg, int lane, int nr, unsigned bound, bool far) {
+    const double *o = sg.rec + lane * Stage<C>::kS;
+    const unsigned ok = __ballot_sync(kFull, far && o[4] < 1e3);
+    const int first = 31 - __clz(int(bound & (0xffffffffu >> (31 - lane))));  // of the lane's run (bit 0 is set)
+    const int idx = lane - first;
+    const unsigned need = 0xffu << lane;
+    const bool start = idx >= 2 && (idx - 2) % kBlock == 0 && lane + kBlock <= nr && (ok & need) == need &&
+                       (bound & (need & ~(1u << lane))) == 0u;
+    const unsigned starts = __ballot_sync(kFull, start);
+    if (starts == 0u) return 0u;
+    double m11 = 1.0, m12 = 0.0, m21 = 0.0, m22 = 1.0, al = 0.0, be = 0.0;
+    if (lane > 1 && ((ok >> lane) & 1u)) {
+        const double t = 2.0 * o[4];
+        m12 = o[5];
+        m21 = t;
+        m22 = fma(t, m12, 1.0);
+        be = o[1 - Stage<C>::kS] * m12;
+    }
+#pragma unroll
+    for (int d = 1; d < kBlock; d <<= 1) {
+        const double s11 = __shfl_down_sync(kFull, m11, d), s12 = __shfl_down_sync(kFull, m12, d);
+        const double s21 = __shfl_down_sync(kFull, m21, d), s22 = __shfl_down_sync(kFull, m22, d);
+        const double sa = __shfl_down_sync(kFull, al, d), sb = __shfl_down_sync(kFull, be, d);
+        al = fma(sa, m11, fma(sb, m21, al));
+        be = fma(sa, m12, fma(sb, m22, be));
+        const double n11 = fma(s11, m11, s12 * m21), n12 = fma(s11, m12, s12 * m22);
+        m21 = fma(s21, m11, s22 * m21);
+        m22 = fma(s21, m12, s22 * m22);
+        m11 = n11;
+        m12 = n12;
+    }
+    if (start) {
+        double *b = sg.blk[lane / kBlock];
+        b[0] = m11;
+        b[1] = m12;
+        b[2] = m21;
+        b[3] = m22;
+        b[4] = al;
+        b[5] = be;
+    }
+    return starts;
+}
+
 // consume_chunk of the integer form.  Also returns at a sample that the
 // fixed-point arithmetic does not cover (sg.m_wild), for plain_step.
 template <class C>
@@ -1652,7 +1713,7 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
 #pragma unroll 1
     for (; r0 < total; r0 += kCap, s = 0, fresh = true) {
         const int nr = total - r0 < kCap ? total - r0 : kCap;
-        unsigned m_split, m_new, m_wild;
+        unsigned m_split, m_new, m_wild, m_block;
         if (fresh) {
             const unsigned cls = lane < nr ? gen_sample<C>(sg, r0 + lane, lane, nch, sign, a.dtau_max) : 0u;
             const unsigned up = __shfl_up_sync(kFull, cls, 1);
@@ -1672,10 +1733,15 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
                 o[5] = lane > 1 ? o[-kS] * (o[2 - 2 * kS] + o[2 - kS]) + h : h;
             }
             __syncwarp();
+            m_block = compose_blocks<C>(sg, lane, nr, m_split | m_split << 1 | m_new | 1u,
+                                        lane > 0 && lane < nr && cls == 0u);
+            if (lane == 0) sg.m_block = m_block;
+            __syncwarp();
         } else {
             m_split = sg.m_split;
             m_new = sg.m_new;
             m_wild = sg.m_wild;
+            m_block = sg.m_block;
         }
         while (s < nr) {
             const double *src = sg.rec + s * kS;
@@ -1689,6 +1755,8 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
             const unsigned next = (m_split | m_new) & (0xfffffffeu << s);
             const int e = next ? min(__ffs(int(next)) - 1, nr) : nr;
             const double *end = sg.rec + e * kS;
+            const unsigned blocks = m_block >> s;
+            const int s0 = s;
             s = e;
             if (on == 0u) {
                 // the continuum: from the run's second sample on the increments are the same
@@ -1696,6 +1764,23 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
                 int k = 0;
 #pragma unroll 1
                 for (; src < end; src += kS, ++k) {
+                    if ((blocks >> k) & 1u) {
+                        const double *b = sg.blk[(s0 + k) / kBlock];
+                        src += (kBlock - 1) * kS;  // to the block's last record
+                        k += kBlock - 1;
+#pragma unroll
+                        for (int i = 0; i < C::BPL; ++i) {
+                            const double N = w[i].N, Q = w[i].Q;
+                            w[i].W = fma(b[4], N, fma(b[5], Q, w[i].W));
+                            w[i].N = fma(b[0], N, b[1] * Q);
+                            w[i].Q = fma(b[2], N, b[3] * Q);
+                            w[i].h = src[4];
+                            w[i].T = src[2];
+                            w[i].S = src[1];
+                            int_rescale(w[i]);
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int i = 0; i < C::BPL; ++i) {
                         const double h = k > 0 ? src[4] : src[0] * (w[i].T + src[2]);

@@ -157,6 +157,43 @@ __host__ __device__ __forceinline__ double from_q61(uint64_t v) {
 #endif
 }
 
+// Conversions and a halving that the FP64 pipe would take 77 cycles for: a
+// non-negative float as a double, half a non-negative double, and D in Q0.62
+// as the nearest float.
+__host__ __device__ __forceinline__ double widen(float x) {
+#ifdef __CUDA_ARCH__
+    const uint32_t b = __float_as_uint(x);
+    return b >= 0x00800000u ? __hiloint2double(int((b >> 3) + 0x38000000u), int(b << 29)) : double(x);
+#else
+    return double(x);
+#endif
+}
+
+__host__ __device__ __forceinline__ double halve(double x) {
+    const uint64_t b = double_bits(x);
+    return b >= (uint64_t(2) << 52) ? bits_double(b - (uint64_t(1) << 52)) : x * 0.5;
+}
+
+__host__ __device__ __forceinline__ float narrow_q62(uint64_t D) {
+    const uint32_t top = uint32_t(D >> 31) | uint32_t((D & 0x7fffffffu) != 0);  // Q.31, sticky
+    return float(top) * 4.656612873077393e-10f;                                // 2^-31
+}
+
+// b D as the nearest float, D in Q0.62, b a double in [0, 2).
+__host__ __device__ __forceinline__ float narrow_product(double b, uint64_t D) {
+    const uint64_t bits = double_bits(b);
+    const uint32_t e = uint32_t(bits >> 52);
+    if (e < 930u) return float(b * from_q62(D));  // below 2^-93, where the scale below is no normal float
+    const uint64_t m = ((bits << 10) & ((uint64_t(1) << 62) - 1)) | (uint64_t(1) << 62);
+    const uint64_t p = mul_hi63(m, D);            // b D 2^(1023 - e) in Q.60, at least 2^58
+    const uint32_t top = uint32_t(p >> 29) | uint32_t((p & 0x1fffffffu) != 0);  // Q.31, sticky
+#ifdef __CUDA_ARCH__
+    return float(top) * __uint_as_float((e - 927u) << 23);  // 2^(e - 1023 - 31)
+#else
+    return float(double(top) * bits_double(uint64_t(e - 31u) << 52));
+#endif
+}
+
 // One pivot of the scaled elimination in fixed point: with Y = D Fh of the row
 // before (Q2.61), the increment t < 1.01 (Q1.62) and b, its mean with the one
 // before (Q2.61):  Fh = b + Y,  D = 1 / (1 + t Fh) (returned, Q0.62),  Y = D Fh.

@@ -270,24 +270,34 @@ __device__ __forceinline__ void row2(Sweep<float2> &w, float2 chi, float2 eta, f
 //   Fh = (1 + h/2) / (1 - h^2/6),  zh = D (h S_i / 3 + h S_{i+1} / 6 + I) / (1 - h^2/6).
 constexpr double kHermRatio = 64.0;
 
+// A non-negative value of the form in the pivots' precision.
+template <typename P, typename R>
+__device__ __forceinline__ P wide(R x) {
+    if constexpr (sizeof(P) != sizeof(R)) return widen(x);
+    else return x;
+}
+
 template <int ORD, typename R, typename P>
 __device__ __forceinline__ void row(Sweep<R, P> &w, R chi, R eta, P dt, R Si, R Sn) {
     if constexpr (ORD == 2 && sizeof(P) != sizeof(R)) {
         // pivots of double's precision: D = 1 / (1 + dt Fh) in fixed point (pivot_q; of the
-        // 22 FP64 instructions a row took, the reciprocal most, six are left); z in single
+        // 22 FP64 instructions a row took, the reciprocal most, three are left); z in single
         // precision from D and S = eta / chi
-        const P dtb = fma(dt, P(0.5), w.dtp);
-        P D;
-        if (dt < P(1)) {
-            const uint64_t t = to_q62(dt);
-            D = from_q62(pivot_q(t, to_q62(dtb) >> 1, w.Y));
+        const P half = halve(dt), dtb = half + w.dtp;
+        R Dr, bD;  // D and dtb D in single precision
+        if (__double2hiint(dt) < 0x3ff00000 && __double2hiint(dtb) < 0x3ff00000) {  // below 1 (not negative)
+            const uint64_t q = pivot_q(to_q62(dt), to_q62(dtb) >> 1, w.Y);
+            Dr = narrow_q62(q);
+            bD = narrow_product(dtb, q);
         } else {  // thick cells without optical-depth sampling (dtau_max > 1)
             const P Fh = dtb + from_q61(w.Y);
-            D = P(1) / (P(1) + dt * Fh);
+            const P D = P(1) / (P(1) + dt * Fh);
+            Dr = R(D);
+            bD = R(dtb * D);
             w.Y = to_q62(D * Fh) >> 1;
         }
-        w.zh = R(D) * w.zh + R(dtb * D) * (eta * Ar<R>::rcp(chi));
-        w.dtp = dt * P(0.5);
+        w.zh = Dr * w.zh + bD * (eta * Ar<R>::rcp(chi));
+        w.dtp = half;
     } else if constexpr (ORD == 2) {
         const P dtb = fma(dt, P(0.5), w.dtp);
         w.Fh = dtb + w.Dm * w.Fh;
@@ -1279,7 +1289,7 @@ __device__ __forceinline__ bool sample_step(const typename C::V (&v)[Stage<C>::k
         for (int i = 0; i < BPL; ++i) {
             R Sq = R(0);
             if constexpr (ORD == 4) Sq = Ar<R>::src(eta_q[i], chi_q[i]);
-            row<ORD>(w[i], w[i].chi, w[i].eta, P(hq) * (P(w[i].chi) + P(chi_q[i])), w[i].Sc, Sq);
+            row<ORD>(w[i], w[i].chi, w[i].eta, wide<P>(hq) * (wide<P>(w[i].chi) + wide<P>(chi_q[i])), w[i].Sc, Sq);
             w[i].chi = chi_q[i];
             w[i].eta = eta_q[i];
             w[i].Sc = Sq;
@@ -1301,14 +1311,14 @@ __device__ __forceinline__ bool sample_step(const typename C::V (&v)[Stage<C>::k
             const R ck = c0 + dchi * R(k), ek = e0 + deta * R(k);
             R Sk = R(0);
             if constexpr (ORD == 4) Sk = Ar<R>::src(ek, ck);
-            row<ORD>(w[i], cprev, eprev, P(hh) * (P(cprev) + P(ck)), Sprev, Sk);
+            row<ORD>(w[i], cprev, eprev, wide<P>(hh) * (wide<P>(cprev) + wide<P>(ck)), Sprev, Sk);
             cprev = ck;
             eprev = ek;
             Sprev = Sk;
         }
         R Sq = R(0);
         if constexpr (ORD == 4) Sq = Ar<R>::src(eta_q[i], chi_q[i]);
-        row<ORD>(w[i], cprev, eprev, P(hh) * (P(cprev) + P(chi_q[i])), Sprev, Sq);
+        row<ORD>(w[i], cprev, eprev, wide<P>(hh) * (wide<P>(cprev) + wide<P>(chi_q[i])), Sprev, Sq);
         w[i].chi = chi_q[i];
         w[i].eta = eta_q[i];
         w[i].Sc = Sq;

@@ -29,6 +29,8 @@ extern "C" double t_div(double e, double t) { return mgx::div_pos(e, t); }
 extern "C" double t_piv(double t, double b, uint64_t *Y) {
     return mgx::from_q62(mgx::pivot_q(mgx::to_q62(t), mgx::to_q62(b) >> 1, *Y));
 }
+extern "C" float t_prod(double b, uint64_t D) { return mgx::narrow_product(b, D); }
+extern "C" float t_narrow(uint64_t D) { return mgx::narrow_q62(D); }
 extern "C" uint64_t t_tab(int j) { return tab.v[j]; }
 """
 
@@ -44,6 +46,8 @@ def lib(tmp_path_factory):
     L.t_exp.restype, L.t_exp.argtypes = C.c_double, [C.c_uint64]
     L.t_div.restype, L.t_div.argtypes = C.c_double, [C.c_double, C.c_double]
     L.t_piv.restype, L.t_piv.argtypes = C.c_double, [C.c_double, C.c_double, C.POINTER(C.c_uint64)]
+    L.t_prod.restype, L.t_prod.argtypes = C.c_float, [C.c_double, C.c_uint64]
+    L.t_narrow.restype, L.t_narrow.argtypes = C.c_float, [C.c_uint64]
     L.t_tab.restype, L.t_tab.argtypes = C.c_uint64, [C.c_int]
     return L
 
@@ -99,3 +103,20 @@ def test_pivot(lib):
             assert abs(mp.mpf(got) - D) <= (2.0 ** -55 + 2.0 ** -53) * D
             assert abs(mp.mpf(Y.value) / mp.mpf(2) ** 61 - D * F) <= 2.0 ** -54
             tp = 0.5 * t
+
+
+def test_single_precision_results(lib):
+    """D and dtb D come out as the nearest floats of the fixed-point D's exact multiples."""
+    from fractions import Fraction
+
+    rng = np.random.default_rng(12)
+    D = [int(x) for x in rng.integers(1 << 60, 1 << 62, 4000)] + [1 << 62, (1 << 62) - 1, 3 << 60, (1 << 61) + (1 << 37)]
+    b = [float(x) for x in 10.0 ** rng.uniform(-40, 0, len(D))]
+    for d, x in zip(D, b):
+        for got, exact in ((lib.t_narrow(d), Fraction(d, 1 << 62)), (lib.t_prod(x, d), Fraction(x) * Fraction(d, 1 << 62))):
+            f = np.float32(got)
+            lo, hi = np.nextafter(f, np.float32(0)), np.nextafter(f, np.float32(2))
+            err = abs(Fraction(float(f)) - exact)
+            # nearest, but for products within 2^-34 of a tie (the high product's error)
+            slack = Fraction(float(hi) - float(f)) / (1 << 34)
+            assert err <= abs(Fraction(float(lo)) - exact) + slack and err <= abs(Fraction(float(hi)) - exact) + slack

@@ -631,17 +631,31 @@ __device__ __forceinline__ void stage_point(const DevMesh &m, const DevLines &Ln
     int32_t id = sg.o;
     double z = 0.0;
     R d = R(0), de = R(0);
+    // the traced ids stream through once: evict-first, so that they do not push the
+    // mesh and the spilled item state out of L2
     if (q < cnt) {
         const int32_t k = cnt - 1 - q;
-        // the traced ids stream through once: evict-first, so that they do not push the
-        // mesh and the spilled item state out of L2
         id = k < hl.n_main ? __ldcs(hl.main + k) : __ldcs(hl.tail + (hl.tail_off + k));
-        z = exact_Z(m, id, sg.xo[0], sg.xo[1], sg.xo[2], e0, e1, e2);
+    }
+    float4 p0, p1, p2, p3;  // single precision: the point's record
+    if constexpr (sizeof(R) == 4) {
+        const float4 *rec = Ln.pt + 4 * int64_t(id);
+        p0 = __ldg(rec);
+        p1 = __ldg(rec + 1);
+        p2 = __ldg(rec + 2);
+        p3 = __ldg(rec + 3);
+    }
+    if (q < cnt) {
         if constexpr (sizeof(R) == 8) {
+            z = exact_Z(m, id, sg.xo[0], sg.xo[1], sg.xo[2], e0, e1, e2);
             d = proj64(m, id, sg.vo, e0, e1, e2);
         } else {
+            const double dx = __dsub_rn(__hiloint2double(__float_as_int(p0.y), __float_as_int(p0.x)), sg.xo[0]);
+            const double dy = __dsub_rn(__hiloint2double(__float_as_int(p0.w), __float_as_int(p0.z)), sg.xo[1]);
+            const double dz = __dsub_rn(__hiloint2double(__float_as_int(p1.y), __float_as_int(p1.x)), sg.xo[2]);
+            z = __dadd_rn(__dadd_rn(__dmul_rn(dx, e0), __dmul_rn(dy, e1)), __dmul_rn(dz, e2));  // as exact_Z
             const float f0 = float(e0), f1 = float(e1), f2 = float(e2);
-            const float vx = __ldg(Pts<R>::vx(m) + id), vy = __ldg(Pts<R>::vy(m) + id), vz = __ldg(Pts<R>::vz(m) + id);
+            const float vx = p1.z, vy = p1.w, vz = p2.x;
             const float ux = vx - sg.vor[0], uy = vy - sg.vor[1], uz = vz - sg.vor[2];
             d = fmaf(uz, f2, fmaf(uy, f1, ux * f0));
             de = delta_bound<C>(sg, vx, vy, vz, f0, f1, f2);
@@ -652,11 +666,24 @@ __device__ __forceinline__ void stage_point(const DevMesh &m, const DevLines &Ln
     zq = z;
     deq = de;
     sg.d[slot] = d;
-    sg.w[slot] = __ldg(Pts<R>::dvw(Ln) + id);
-    sg.cc[slot] = __ldg(Pts<R>::chic(Ln) + id);
-    sg.ec[slot] = __ldg(Pts<R>::etac(Ln) + id);
+    constexpr int kIn = sizeof(R) == 4 ? (NL < 2 ? NL : 2) : 0;  // lines in the record
+    if constexpr (sizeof(R) == 4) {
+        sg.w[slot] = p2.y;
+        sg.cc[slot] = p2.z;
+        sg.ec[slot] = p2.w;
+        sg.ce[0][slot] = p3.x;
+        sg.ce[1][slot] = p3.y;
+        if constexpr (NL > 1) {
+            sg.ce[2][slot] = p3.z;
+            sg.ce[3][slot] = p3.w;
+        }
+    } else {
+        sg.w[slot] = __ldg(Pts<R>::dvw(Ln) + id);
+        sg.cc[slot] = __ldg(Pts<R>::chic(Ln) + id);
+        sg.ec[slot] = __ldg(Pts<R>::etac(Ln) + id);
+    }
 #pragma unroll
-    for (int l = 0; l < NL; ++l) {
+    for (int l = kIn; l < NL; ++l) {
         sg.ce[2 * l][slot] = l < L ? __ldg(Pts<R>::chi0(Ln) + int64_t(id) * L + l) : R(0);
         sg.ce[2 * l + 1][slot] = l < L ? __ldg(Pts<R>::eta0(Ln) + int64_t(id) * L + l) : R(0);
     }

@@ -40,6 +40,7 @@ struct Model {
     double nu0[MGX_MAX_LINES] = {};
     double *chi0 = nullptr, *eta0 = nullptr, *dvw = nullptr, *chic = nullptr, *etac = nullptr;
     float *chi0f = nullptr, *eta0f = nullptr, *dvwf = nullptr, *chicf = nullptr, *etacf = nullptr;
+    float4 *pt = nullptr;
     // rays
     bool has_rays = false;
     int32_t lmin = 0, lmax = 0, npairs = 0;
@@ -275,6 +276,7 @@ DevLines lines_view(const Model &m) {
         for (int lp = 0; lp < m.L; ++lp) d.ratio[l * MGX_MAX_LINES + lp] = m.nu0[l] / m.nu0[lp];
     d.chi0 = m.chi0; d.eta0 = m.eta0; d.dvw = m.dvw; d.chic = m.chic; d.etac = m.etac;
     d.chi0f = m.chi0f; d.eta0f = m.eta0f; d.dvwf = m.dvwf; d.chicf = m.chicf; d.etacf = m.etacf;
+    d.pt = m.pt;
     return d;
 }
 
@@ -349,6 +351,7 @@ mgx_status ensure_tables(mgx_ctx *ctx, int level) {
 void free_lines(mgx_ctx *ctx, Model &m) {
     dfree(ctx, m.chi0); dfree(ctx, m.eta0); dfree(ctx, m.dvw); dfree(ctx, m.chic); dfree(ctx, m.etac);
     dfree(ctx, m.chi0f); dfree(ctx, m.eta0f); dfree(ctx, m.dvwf); dfree(ctx, m.chicf); dfree(ctx, m.etacf);
+    dfree(ctx, m.pt);
     m.has_lines = false;
 }
 
@@ -759,6 +762,7 @@ mgx_status mgx_set_lines(mgx_ctx *ctx, int32_t model, int32_t n_lines, const dou
     CK(dalloc(ctx, &m->dvw, n)); CK(dalloc(ctx, &m->chic, n)); CK(dalloc(ctx, &m->etac, n));
     CK(dalloc(ctx, &m->chi0f, nl)); CK(dalloc(ctx, &m->eta0f, nl));
     CK(dalloc(ctx, &m->dvwf, n)); CK(dalloc(ctx, &m->chicf, n)); CK(dalloc(ctx, &m->etacf, n));
+    CK(dalloc(ctx, &m->pt, 4 * n));
     CK(cudaMemcpyAsync(m->chi0, chi0, nl * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(m->eta0, eta0, nl * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(m->dvw, dvw, n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
@@ -768,9 +772,10 @@ mgx_status mgx_set_lines(mgx_ctx *ctx, int32_t model, int32_t n_lines, const dou
         Timed t(ctx, MGX_K_OTHER);
         launch_ingest_lines(m->n, n_lines, m->chi0, m->eta0, m->dvw, m->chic, m->etac, m->chi0f, m->eta0f,
                             m->dvwf, m->chicf, m->etacf, ctx->d_status, ctx->stream);
+        m->L = n_lines;
+        launch_pack_points(mesh_view(*m), lines_view(*m), m->pt, ctx->stream);
     }
     CK(cudaGetLastError());
-    m->L = n_lines;
     m->F = n_freq;
     m->x_span = x_span;
     for (int l = 0; l < n_lines; ++l) m->nu0[l] = nu0[l];

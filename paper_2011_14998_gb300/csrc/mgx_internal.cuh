@@ -55,6 +55,8 @@ struct DevLines {
     const double *dvw, *chic, *etac;
     const float *chi0f, *eta0f;
     const float *dvwf, *chicf, *etacf;
+    const float4 *pt;  // [n][4] what the single-precision solve stages of a point, 64 bytes together:
+                       // x, y, z (double); velocity, Doppler width, continuum and the first two lines (float)
 };
 
 struct DevRays {
@@ -104,6 +106,7 @@ void launch_ingest_lines(int32_t n, int32_t L, const double *chi0, const double 
                          const double *dvw, const double *chic, const double *etac, float *chi0f,
                          float *eta0f, float *dvwf, float *chicf, float *etacf, int *status,
                          cudaStream_t st);
+void launch_pack_points(const DevMesh &m, const DevLines &Ln, float4 *pt, cudaStream_t st);
 
 // ---- ray sets (k_rays.cu)
 void launch_rays_fixed(int32_t n, int32_t level, int32_t npairs, const uint32_t *pairs,

@@ -441,9 +441,9 @@ struct Stage {
     int id[33], nv[33], so[33];             // point (-1: the origin), velocity samples, their offset
     unsigned on[C::kInt ? kCap : 1];        // integer form: the lines that take part in each record
     unsigned m_block;                       // records at which a block of kBlock continuum rows starts
-    double blk[C::kInt ? kCap / 8 : 1][6];  // and the blocks' maps (block of record s in blk[s / 8])
+    double blk[C::kInt ? kCap / 8 : 1][C::kInt ? 6 : 1];  // and the blocks' maps (block of record s in blk[s / 8])
     double span;                            // integer form, one line: x_span dvw_o, the bins' half-range in km/s
-    uint64_t uk[C::kInt && NL == 1 ? BPL : 1][32];  // and each lane's bins' place in it, (ub / span + 1) / 2, in Q0.63
+    uint64_t uk[C::kInt && NL == 1 ? BPL : 1][C::kInt && NL == 1 ? 32 : 1];  // and each lane's bins' place in it, (ub / span + 1) / 2, in Q0.63
     R Am[NL], Bm[NL];                       // largest |A|, |B| of each line over the warp's bins
     double r[3], xo[3], vo[3];              // pair direction, origin position and velocity (double)
     R vor[3];                               // origin velocity in the form's precision
@@ -453,7 +453,7 @@ struct Stage {
     int fix[BPL][32];                       // Eq. 2 counts of a sample whose single-precision decision was left
                                             // open (0: not open; negative: to resolve, the bits of -chi)
     float wA[NL][2], wB[NL][2];             // single precision: smallest and largest A, B over the warp's bins
-    unsigned m_split, m_new, m_wild;        // packed and integer forms: the round's records that may split; whose lines differ
+    unsigned m_split, m_new, m_wild;        // single-precision and integer forms: the round's records that may split; whose lines differ
                                             // from the record's before
 };
 
@@ -909,7 +909,7 @@ __device__ __forceinline__ unsigned gen_sample_int(Stage<C> &sg, int k, int nv, 
 }
 
 // Record of sample s_abs of the chunk (relative to its first) into record s_rec.
-// Returns (packed form) the mask of the lines that take part, bit 31 set when some bin may need a split.
+// Returns (single precision) the mask of the lines that take part, bit 31 set when some bin may need a split.
 template <class C>
 __device__ __forceinline__ unsigned gen_sample(Stage<C> &sg, int s_abs, int s_rec, int nch, int sign,
                                                double dtau_max) {
@@ -975,6 +975,7 @@ __device__ __forceinline__ unsigned gen_sample(Stage<C> &sg, int s_abs, int s_re
             o[5] = thr;
 #pragma unroll
             for (int c = 0; c < 2 * NL; ++c) o[6 + c] = ce[c];
+            return on | (thr != INFINITY ? 0x80000000u : 0u);
         }
     } else if constexpr (C::kInt) {
         return gen_sample_int<C>(sg, k, nv, j, s_rec, sign, dtau_max);
@@ -1507,6 +1508,73 @@ __device__ __noinline__ int consume_chunk(Stage<C> &sg, Lane<C> &ln, const Solve
                     for (; src < end; src += kS) {
                         all_lines<C>(src, on, sg, chi_q, eta_q);
                         rows_to<C>(src[4], chi_q, eta_q, w);
+                    }
+                }
+            }
+        } else if constexpr (sizeof(typename C::R) == 4 && sizeof(typename C::P) == 4) {
+            // the scalar single-precision forms in runs too: records on which no bin can split,
+            // with the continuum alone or with lines (12 000 points, Hermitian: 48.6 -> 42.9 ms;
+            // with FP64 pivots, whose row is long, the one loop below is faster: 142 against 151)
+            using R = typename C::R;
+            static_assert(kCap == 32, "one record per lane");
+            unsigned m_split, m_new;
+            if (fresh) {
+                const unsigned cls = lane < nr ? gen_sample<C>(sg, r0 + lane, lane, nch, sign, a.dtau_max) : 0u;
+                const unsigned any = __ballot_sync(kFull, (cls & 0x7fffffffu) != 0u);
+                m_split = __ballot_sync(kFull, cls >> 31);
+                m_new = any ^ (any << 1);
+                if (lane == 0) {
+                    sg.m_split = m_split;
+                    sg.m_new = m_new;
+                    sg.m_wild = any;
+                }
+                __syncwarp();
+            } else {
+                m_split = sg.m_split;
+                m_new = sg.m_new;
+            }
+            while (s < nr) {
+                R v[kS];
+                if ((m_split >> s) & 1u) {
+                    load_rec<C>(sg.rec + s * kS, v);
+                    if (!sample_step<C>(v, r0 + s, r0 + s == pend, sg, a, f, w)) break;
+                    ++s;
+                    continue;
+                }
+                const unsigned next = (m_split | m_new) & (0xfffffffeu << s);
+                const int e = next ? min(__ffs(int(next)) - 1, nr) : nr;
+                const bool lines = ((sg.m_wild >> s) & 1u) != 0u;
+                auto rows = [&](const R (&chi_q)[C::BPL], const R (&eta_q)[C::BPL]) {
+#pragma unroll
+                    for (int i = 0; i < C::BPL; ++i) {
+                        R Sq = R(0);
+                        if constexpr (C::ORD == 4) Sq = Ar<R>::src(eta_q[i], chi_q[i]);
+                        row<C::ORD>(w[i], w[i].chi, w[i].eta, v[4] * (w[i].chi + chi_q[i]), w[i].Sc, Sq);
+                        w[i].chi = chi_q[i];
+                        w[i].eta = eta_q[i];
+                        w[i].Sc = Sq;
+                    }
+                };
+                R chi_q[C::BPL], eta_q[C::BPL];
+                if (lines) {
+#pragma unroll 2
+                    for (; s < e; ++s) {
+                        load_rec<C>(sg.rec + s * kS, v);
+#pragma unroll
+                        for (int i = 0; i < C::BPL; ++i)
+                            optics<R, C::NL>(v[0], v[1], v[2], v[3], v + 6, f[i], chi_q[i], eta_q[i]);
+                        rows(chi_q, eta_q);
+                    }
+                } else {
+#pragma unroll 2
+                    for (; s < e; ++s) {
+                        load_rec<C>(sg.rec + s * kS, v);
+#pragma unroll
+                        for (int i = 0; i < C::BPL; ++i) {
+                            chi_q[i] = v[2];
+                            eta_q[i] = v[3];
+                        }
+                        rows(chi_q, eta_q);
                     }
                 }
             }

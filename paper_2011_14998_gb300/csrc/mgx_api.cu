@@ -991,7 +991,11 @@ mgx_status mgx_solve_J(mgx_ctx *ctx, int32_t model, const mgx_solve_params *p, v
         fill_pair_weights(a);
         const size_t n_u = size_t(o1 - o0) * size_t(np) * size_t(NB);
         a.parts = solve_parts(p->precision, int64_t(o1 - o0) * a.n_tiles, np, n_u * sizeof(double));
-        if (a.parts > 1) CK(dalloc(ctx, &a.u_out, n_u));
+        if (a.parts > 1 && dalloc(ctx, &a.u_out, n_u) != cudaSuccess) {  // no room for u: one warp per item
+            cudaGetLastError();
+            a.u_out = nullptr;
+            a.parts = 1;
+        }
         {
             Timed t(ctx, MGX_K_SOLVE);
             launch_solve(dm, dl, dr, a, p->precision, p->order == 4 ? 4 : 2, ctx->stream);
@@ -1269,7 +1273,11 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
         max_tiles = std::max(max_tiles, int32_t(std::min<int64_t>(tiles, 65535)));
     }
     pl.parts = std::min(solve_parts(p->precision, n_items, min_pairs, n_u * sizeof(double)), 65535 / max_tiles);
-    if (pl.parts > 1) CK(dalloc(ctx, &pl.u, n_u));
+    if (pl.parts > 1 && dalloc(ctx, &pl.u, n_u) != cudaSuccess) {  // no room for u: one warp per item
+        cudaGetLastError();
+        pl.u = nullptr;
+        pl.parts = 1;
+    }
     for (int32_t k = 0; k < n_models; ++k) {
         const Model &m = *ms[size_t(k)];
         const int64_t nb = int64_t(m.L) * m.F;

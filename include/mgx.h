@@ -57,10 +57,11 @@ enum {
                      the double-precision definition's: taken in single precision
                      under a rigorous error bound, redone in double precision
                      where the bound leaves the integer open                        */
-    MGX_FP32_DT64 = 2 /* MGX_FP32 with the optical-depth increments and the pivot
-                     recurrence of the elimination (Fh and D of the scaled 1+B form)
-                     also in double precision, z and S in single precision; second-
-                     order scheme only (order 4 gives MGX_EINVAL)                    */
+    MGX_FP32_DT64 = 2 /* MGX_FP32 with the optical-depth increments in double precision
+                     and the pivot recurrence of the elimination (Fh and D of the
+                     scaled 1+B form) in 59 fraction bits or double precision, z and
+                     S in single precision; second-order scheme only (order 4 gives
+                     MGX_EINVAL)                                                     */
 };
 
 /* Limits. */
@@ -217,8 +218,8 @@ mgx_status mgx_solve_u(mgx_ctx *ctx, int32_t model, const mgx_solve_params *para
  * prediction for the features X [n][8] (as in mgx_reduce_mesh_learned), point i
  * is kept when u_i < min(1, c 10^(alpha y_i)), u_i the SplitMix64 uniform of
  * (seed, i) as in mgx_reduce_mesh, and c the scale at which the expected kept
- * count sum_i min(1, c 10^(alpha y_i)) equals keep_fraction * n (bisection on
- * log2 c).  alpha = 0 is uniform thinning.  keep [n] host; *n_kept and *scale
+ * count sum_i min(1, c 10^(alpha y_i)) equals keep_fraction * n (its root, by
+ * Newton steps).  alpha = 0 is uniform thinning.  keep [n] host; *n_kept and *scale
  * (c) may be NULL.  Requires 0 <= keep_fraction <= 1, alpha finite and >= 0,
  * and parameters set (mgx_mlp_set_params) else MGX_ESTATE. */
 mgx_status mgx_reduce_mesh_learned_weighted(mgx_ctx *ctx, int32_t model, const float *X, double keep_fraction,
@@ -288,7 +289,8 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
  * whose J may differ from the other's in its rounding (about 1e-8 relative:
  * the compilers' fused multiply-adds differ), never beyond that. */
 typedef struct {
-    int32_t bins_per_lane;     /* single-precision frequency bins per lane: 0 automatic (2 above 32 bins), 1, 2 */
+    int32_t bins_per_lane;     /* single-precision frequency bins per lane: 0 automatic (2 above 32 bins, 4 for one
+                                  line where that takes no more bin slots), 1, 2 */
     int32_t trace_ctas_per_sm; /* resident tracer CTAs of 128 threads per SM: 0 = 7, else 1..32 (capped at
                                   what fits) */
     int32_t tail_permille;     /* row width of the traced lists: the narrowest power of two leaving at most this

@@ -195,11 +195,12 @@ __host__ __device__ __forceinline__ float narrow_product(double b, uint64_t D) {
 }
 
 // One pivot of the scaled elimination in fixed point: with Y = D Fh of the row
-// before (Q2.61), the increment t < 1.01 (Q1.62) and b, its mean with the one
+// before (Q2.61), the increment t < 1 (Q1.62) and b < 1, its mean with the one
 // before (Q2.61):  Fh = b + Y,  D = 1 / (1 + t Fh) (returned, Q0.62),  Y = D Fh.
-// The scaled quantities are of order one (Y at most about 2), so 59 fraction
-// bits are more than a double's 53; the reciprocal is a single-precision one
-// with one correction and its square.
+// For Y < 2 on entry Fh is below 3 and 1 + t Fh below 4, which is what the
+// formats hold.  The scaled quantities are of order one, so 59 fraction bits are
+// more than a double's 53; the reciprocal is a single-precision one with one
+// correction and its square.
 __host__ __device__ __forceinline__ uint64_t pivot_q(uint64_t t, uint64_t b, uint64_t &Y) {
     const uint64_t F = b + Y;
     const uint64_t den = (uint64_t(1) << 59) + mul_hi63(t, F);  // Q4.59, in [1, 4)
@@ -218,6 +219,37 @@ __host__ __device__ __forceinline__ uint64_t pivot_q(uint64_t t, uint64_t b, uin
     const uint64_t D = (uint64_t(X) << 31) + (mul_hi63(uint64_t(X) << 31, d << 23) >> 17);
     Y = mul_hi63(F, D) << 2;
     return D;
+}
+
+// Y of the pivots as they carry it: Q2.61 below 2, else the double's own bits
+// with the sign bit set.  With increments up to 1 alone Y stays below 1.12
+// (Y + t / 2 does not pass sqrt(1 + t^2 / 4) for the largest t); a thick cell
+// followed by a thin one leaves half the thick one's increment.
+__host__ __device__ __forceinline__ uint64_t hold_y(double y) {
+    const uint64_t b = double_bits(y);
+    return b < (uint64_t(1024) << 52) ? to_q62(y) >> 1 : b | (uint64_t(1) << 63);
+}
+
+__host__ __device__ __forceinline__ double held_y(uint64_t Y) {
+    return Y >> 63 ? bits_double(Y & ~(uint64_t(1) << 63)) : from_q61(Y);
+}
+
+// One pivot for any increment dt >= 0 and mean increment dtb: D and dtb D as the
+// nearest floats, Y updated.  In fixed point where its formats hold the operands;
+// else (cells thicker than dtau_max <= 1 lets through, and the thin ones behind
+// them) in double precision.
+__host__ __device__ __forceinline__ void pivot(double dt, double dtb, uint64_t &Y, float &D, float &bD) {
+    constexpr uint32_t kOne = 0x3ff00000u;
+    if (uint32_t(double_bits(dt) >> 32) < kOne && uint32_t(double_bits(dtb) >> 32) < kOne && Y < (uint64_t(1) << 62)) {
+        const uint64_t q = pivot_q(to_q62(dt), to_q62(dtb) >> 1, Y);
+        D = narrow_q62(q);
+        bD = narrow_product(dtb, q);
+    } else {
+        const double F = dtb + held_y(Y), d = div_pos(1.0, 1.0 + dt * F);
+        D = float(d);
+        bD = float(dtb * d);
+        Y = hold_y(d * F);
+    }
 }
 
 }  // namespace mgx

@@ -233,7 +233,7 @@ struct Sweep {
     R zh;
     R chi, eta;     // optics of the current (not yet eliminated) sample
     R Sp, Sc, hp, rh;  // Hermitian scheme only
-    uint64_t Y;        // double-precision pivots with R = float: D Fh in Q2.61 (Fh, Dm not kept)
+    uint64_t Y;        // double-precision pivots with R = float: D Fh as hold_y has it (Fh, Dm not kept)
 };
 
 // The second-order row below for two bins at once, operation for operation.
@@ -280,22 +280,12 @@ __device__ __forceinline__ P wide(R x) {
 template <int ORD, typename R, typename P>
 __device__ __forceinline__ void row(Sweep<R, P> &w, R chi, R eta, P dt, R Si, R Sn) {
     if constexpr (ORD == 2 && sizeof(P) != sizeof(R)) {
-        // pivots of double's precision: D = 1 / (1 + dt Fh) in fixed point (pivot_q; of the
+        // pivots of double's precision: D = 1 / (1 + dt Fh) in fixed point (pivot; of the
         // 22 FP64 instructions a row took, the reciprocal most, three are left); z in single
         // precision from D and S = eta / chi
         const P half = halve(dt), dtb = half + w.dtp;
         R Dr, bD;  // D and dtb D in single precision
-        if (__double2hiint(dt) < 0x3ff00000 && __double2hiint(dtb) < 0x3ff00000) {  // below 1 (not negative)
-            const uint64_t q = pivot_q(to_q62(dt), to_q62(dtb) >> 1, w.Y);
-            Dr = narrow_q62(q);
-            bD = narrow_product(dtb, q);
-        } else {  // thick cells without optical-depth sampling (dtau_max > 1)
-            const P Fh = dtb + from_q61(w.Y);
-            const P D = P(1) / (P(1) + dt * Fh);
-            Dr = R(D);
-            bD = R(dtb * D);
-            w.Y = to_q62(D * Fh) >> 1;
-        }
+        pivot(dt, dtb, w.Y, Dr, bD);
         w.zh = Dr * w.zh + bD * (eta * Ar<R>::rcp(chi));
         w.dtp = half;
     } else if constexpr (ORD == 2) {
@@ -1362,7 +1352,7 @@ __device__ __forceinline__ void put_sweep(Lane<C> &ln, const Sweep<typename C::V
 #pragma unroll
     for (int i = 0; i < C::NV; ++i) {
         if constexpr (C::kPacked) ln.wp[0][i][lane] = vmul(w[i].Dm, w[i].Fh);
-        else if constexpr (sizeof(typename C::P) != sizeof(typename C::R)) ln.wp[0][i][lane] = from_q61(w[i].Y);
+        else if constexpr (sizeof(typename C::P) != sizeof(typename C::R)) ln.wp[0][i][lane] = held_y(w[i].Y);
         else ln.wp[0][i][lane] = w[i].Dm * w[i].Fh;
         ln.wp[1][i][lane] = w[i].dtp;
         ln.wr[0][i][lane] = w[i].zh;
@@ -1383,7 +1373,7 @@ __device__ __forceinline__ void get_sweep(const Lane<C> &ln, Sweep<typename C::V
     using R = typename C::R;
 #pragma unroll
     for (int i = 0; i < C::NV; ++i) {
-        if constexpr (sizeof(typename C::P) != sizeof(typename C::R)) w[i].Y = to_q62(ln.wp[0][i][lane]) >> 1;
+        if constexpr (sizeof(typename C::P) != sizeof(typename C::R)) w[i].Y = hold_y(ln.wp[0][i][lane]);
         w[i].Fh = ln.wp[0][i][lane];
         w[i].Dm = vset<typename C::W>(1.f);
         w[i].dtp = ln.wp[1][i][lane];
@@ -2060,7 +2050,7 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
             else w[i].zh = R(a.I_bdy);
             w[i].hp = vset<V>(-1.f);  // no row yet (Hermitian scheme)
             w[i].Sp = w[i].Sc = w[i].rh = w[i].chi = w[i].eta = vset<V>(0.f);
-            w[i].Y = uint64_t(1) << 61;
+            w[i].Y = hold_y(1.0);
         }
         put_sweep<C>(ln, w, lane);
     }

@@ -29,6 +29,9 @@ extern "C" double t_div(double e, double t) { return mgx::div_pos(e, t); }
 extern "C" double t_piv(double t, double b, uint64_t *Y) {
     return mgx::from_q62(mgx::pivot_q(mgx::to_q62(t), mgx::to_q62(b) >> 1, *Y));
 }
+extern "C" void t_pivot(double dt, double dtb, uint64_t *Y, float *D, float *bD) { mgx::pivot(dt, dtb, *Y, *D, *bD); }
+extern "C" double t_held(uint64_t Y) { return mgx::held_y(Y); }
+extern "C" uint64_t t_hold(double y) { return mgx::hold_y(y); }
 extern "C" float t_prod(double b, uint64_t D) { return mgx::narrow_product(b, D); }
 extern "C" float t_narrow(uint64_t D) { return mgx::narrow_q62(D); }
 extern "C" uint64_t t_tab(int j) { return tab.v[j]; }
@@ -46,6 +49,9 @@ def lib(tmp_path_factory):
     L.t_exp.restype, L.t_exp.argtypes = C.c_double, [C.c_uint64]
     L.t_div.restype, L.t_div.argtypes = C.c_double, [C.c_double, C.c_double]
     L.t_piv.restype, L.t_piv.argtypes = C.c_double, [C.c_double, C.c_double, C.POINTER(C.c_uint64)]
+    L.t_pivot.restype, L.t_pivot.argtypes = None, [C.c_double, C.c_double, C.POINTER(C.c_uint64)] + [C.POINTER(C.c_float)] * 2
+    L.t_held.restype, L.t_held.argtypes = C.c_double, [C.c_uint64]
+    L.t_hold.restype, L.t_hold.argtypes = C.c_uint64, [C.c_double]
     L.t_prod.restype, L.t_prod.argtypes = C.c_float, [C.c_double, C.c_uint64]
     L.t_narrow.restype, L.t_narrow.argtypes = C.c_float, [C.c_uint64]
     L.t_tab.restype, L.t_tab.argtypes = C.c_uint64, [C.c_int]
@@ -103,6 +109,43 @@ def test_pivot(lib):
             assert abs(mp.mpf(got) - D) <= (2.0 ** -55 + 2.0 ** -53) * D
             assert abs(mp.mpf(Y.value) / mp.mpf(2) ** 61 - D * F) <= 2.0 ** -54
             tp = 0.5 * t
+
+
+def increments(rng, kind, n):
+    if kind == "any":
+        return 10.0 ** rng.uniform(-12, 6, n)
+    if kind == "thick_thin":  # a thick cell, then thin ones
+        return np.where(rng.random(n) < 0.3, 10.0 ** rng.uniform(0, 6, n), 10.0 ** rng.uniform(-12, -1, n))
+    return np.where(np.arange(n) % 2 == 0, 10.0 ** rng.uniform(-0.1, 0.7), 1e-3)  # around the formats' ends
+
+
+@pytest.mark.parametrize("kind", ["any", "thick_thin", "ends"])
+def test_pivot_of_any_increment(lib, kind):
+    """The pivot over chains of increments from 1e-12 to 1e6, Y carried over as between two chunks,
+    against the recurrence in 40 digits: D within six roundings of a double and its own to a float;
+    Y = D F within eight, or within 2^-53 in fixed point (below 3); over a whole chain the pivot
+    F = dtb + Y within eight roundings a row, since dln(D F) / dlnF is at most 1."""
+    mp.mp.dps = 40
+    rng = np.random.default_rng(14)
+    wide = 0
+    for _ in range(60):
+        Y, tp, ref = C.c_uint64(lib.t_hold(1.0)), 0.0, mp.mpf(1)
+        D, bD = C.c_float(), C.c_float()
+        for row, t in enumerate(float(x) for x in increments(rng, kind, 60)):
+            b = 0.5 * t + tp
+            Y.value = lib.t_hold(lib.t_held(Y))  # as put_sweep and get_sweep hand it over
+            F = mp.mpf(b) + mp.mpf(lib.t_held(Y))
+            d = 1 / (1 + mp.mpf(t) * F)
+            lib.t_pivot(t, b, C.byref(Y), C.byref(D), C.byref(bD))
+            assert abs(mp.mpf(D.value) - d) <= (6 * 2.0 ** -53 + 2.0 ** -24) * d
+            assert abs(mp.mpf(bD.value) - mp.mpf(b) * d) <= (7 * 2.0 ** -53 + 2.0 ** -24 * (1 + 2.0 ** -9)) * mp.mpf(b) * d
+            got = mp.mpf(lib.t_held(Y))
+            assert abs(got - d * F) <= (8 * 2.0 ** -53) * d * F + (2.0 ** -53 if Y.value < 3 << 61 else 0)
+            wide += Y.value >> 63
+            ref = 1 / (1 / (mp.mpf(b) + ref) + mp.mpf(t))
+            assert abs(got - ref) <= 8 * (row + 1) * 2.0 ** -53 * (0.5 * t + ref)
+            tp = 0.5 * t
+    assert wide > 100  # the double form was reached
 
 
 def test_single_precision_results(lib):

@@ -60,3 +60,30 @@ def test_pairs_dealt_to_several_warps(orc, n, l_min, l_max, precision):
     np.testing.assert_array_equal(Jb, both[0].cpu().numpy())
     np.testing.assert_allclose((w[:, :, None] * u).sum(1), J, rtol=1e-12)
     assert j_rel_err(J, orc.OracleModel(m, rays=rays).solve_J(orc.params()))[0] < (1e-4 if precision == "FP32" else 1e-10)
+
+
+@pytest.mark.parametrize("dtau_max", [1.0, 2.0, 3.5, 10.0, 1e3, 1e6])
+@pytest.mark.parametrize("lines,bins", [(1, 20), (2, 33)])
+def test_double_pivots_over_thick_and_thin_cells(orc, lines, bins, dtau_max):
+    """MGX_FP32_DT64 where thick cells (increments to some hundreds, which a large dtau_max leaves
+    whole) stand next to thin ones: J and the sum of u against the oracle, within twice the
+    form's stated error of 4.8e-6."""
+    import paper_2011_14998_gb300 as mgx
+
+    m = synth.random_cloud(90, seed=5 + lines, n_lines=lines, n_freq=bins, x_span=4.0, l_min=1, l_max=1)
+    f = 10.0 ** np.random.default_rng(5 + lines).uniform(-3, 2.5, 90)
+    m = dict(m, chi0=m["chi0"] * f[:, None], eta0=m["eta0"] * f[:, None], chi_c=m["chi_c"] * f, eta_c=m["eta_c"] * f)
+    ctx = mgx.Context(0)
+    try:
+        mid = ctx.load(m)
+        rays = ctx.rays(mid)
+        kw = dict(precision=mgx.MGX_FP32_DT64, I_bdy=0.05, dtau_max=dtau_max)
+        J = ctx.solve_J(mid, **kw)
+        batch = ctx.solve_J_batch([mid], **kw)[0].cpu().numpy()
+        u = ctx.solve_u(mid, 0, 90, **kw)
+    finally:
+        ctx.close()
+    Jo = orc.OracleModel(m, rays=rays).solve_J(orc.params(I_bdy=0.05, dtau_max=dtau_max))
+    w = 2.0 / (12.0 * 4.0 ** (rays >> 28))
+    for got in (J, batch, (w[:, :, None] * u).sum(1)):
+        assert j_rel_err(got, Jo)[0] < 9.6e-6

@@ -10,6 +10,7 @@
 // low halves' product is dropped: an error below two units of the result).
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -98,6 +99,32 @@ __host__ __device__ __forceinline__ double exp2_neg_sq(uint64_t A, const uint64_
     const uint64_t s = (mul_hi63(R, q) >> 11) + 6393154322601327830ull;        // Q0.63
     const uint64_t m = T + (mul_hi63(T, mul_hi63(R, s)) >> 8);  // Q1.62
     return bits_double(((m + 512) >> 10) + (uint64_t(1021 - n) << 52));
+}
+
+// log2 x for x >= 0 from its exponent and first 20 fraction bits, low by less
+// than 2^-18 for a normal x; an upper bound for a subnormal one and for 0.
+__host__ __device__ __forceinline__ float log2_bits(double x) {
+    const uint32_t hi = uint32_t(double_bits(x) >> 32), mb = 0x3f800000u | (hi & 0xfffffu) << 3;
+#ifdef __CUDA_ARCH__
+    const float f = __log2f(__uint_as_float(mb));
+#else
+    float m;
+    memcpy(&m, &mb, 4);
+    const float f = log2f(m);
+#endif
+    return float(int(hi >> 20) - 1023) + f;
+}
+
+// The |a| from which a line (centre values c0, e0) leaves the continuum's cc and
+// ec as they are, bit for bit: a product below half an ulp, at least 2^-54 of
+// them, rounds away, and 2^(-a^2) is taken as 0 from |a| = 31 on.  From exponents,
+// so that the values' units do not matter.
+__host__ __device__ __forceinline__ float far_profile(double cc, double ec, double c0, double e0) {
+    constexpr uint64_t kNormal = uint64_t(1) << 52;
+    if (double_bits(cc) < kNormal || (e0 > 0.0 && double_bits(ec) < kNormal)) return 31.f;
+    float x = log2_bits(c0) - log2_bits(cc);
+    if (e0 > 0.0) x = fmaxf(x, log2_bits(e0) - log2_bits(ec));
+    return fminf(sqrtf(fmaxf(54.1f + x, 0.f)) * 1.0001f + 1e-3f, 31.f);
 }
 
 // e / t for finite e >= 0, t > 0: the mantissas' quotient from a

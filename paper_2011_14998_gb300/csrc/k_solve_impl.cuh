@@ -793,21 +793,16 @@ __device__ __forceinline__ int slot_of(const Stage<C> &sg, int s_abs, int nch) {
     return lo;
 }
 
-// The same for the double-precision integer form, where a product below half
-// an ulp is below 2^-54 of chi and the profile is taken as 0 from |a| = 31 on.
-// Evaluated in single precision; the margin on |a| covers its rounding.
+// The same for the double-precision integer form (far_profile).  The argument's
+// range is formed in single precision; the margin on |a| covers its rounding.
 __device__ __forceinline__ bool line_is_far(double dl, double rdv, double cc, double ec, double c0, double e0,
                                             const float *wA, const float *wB) {
     if (c0 == 0.0 && e0 == 0.0) return true;
-    const float d = float(dl), rd = float(rdv), fc = float(cc), fe = float(ec), f0 = float(c0), g0 = float(e0);
+    const float d = float(dl), rd = float(rdv);
     const float lo = fmaf(d >= 0.f ? wB[0] : wB[1], d, wA[0]) * rd;
     const float hi = fmaf(d >= 0.f ? wB[1] : wB[0], d, wA[1]) * rd;
     const float mar = 1e-6f * (fmaxf(fabsf(wA[0]), fabsf(wA[1])) + fmaxf(fabsf(wB[0]), fabsf(wB[1])) * fabsf(d)) * rd;
-    float t = 31.f;
-    if (fc > 1e-30f && f0 < 1e30f && (g0 == 0.f || (fe > 1e-30f && g0 < 1e30f))) {
-        const float x = fmaxf(fmaxf(f0 * Ar<float>::rcp(fc), g0 > 0.f ? g0 * Ar<float>::rcp(fe) : 0.f), 1e-30f);
-        t = fminf(sqrtf(fmaxf(54.1f + __log2f(x), 0.f)) * 1.0001f + 1e-3f, 31.f);
-    }
+    const float t = far_profile(cc, ec, c0, e0);
     return lo - mar >= t || hi + mar <= -t;
 }
 

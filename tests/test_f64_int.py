@@ -14,6 +14,7 @@ CPU only."""
 import ctypes as C
 import os
 import subprocess
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -32,6 +33,7 @@ extern "C" double t_piv(double t, double b, uint64_t *Y) {
 extern "C" void t_pivot(double dt, double dtb, uint64_t *Y, float *D, float *bD) { mgx::pivot(dt, dtb, *Y, *D, *bD); }
 extern "C" double t_held(uint64_t Y) { return mgx::held_y(Y); }
 extern "C" uint64_t t_hold(double y) { return mgx::hold_y(y); }
+extern "C" float t_far(double cc, double ec, double c0, double e0) { return mgx::far_profile(cc, ec, c0, e0); }
 extern "C" float t_prod(double b, uint64_t D) { return mgx::narrow_product(b, D); }
 extern "C" float t_narrow(uint64_t D) { return mgx::narrow_q62(D); }
 extern "C" uint64_t t_tab(int j) { return tab.v[j]; }
@@ -52,6 +54,7 @@ def lib(tmp_path_factory):
     L.t_pivot.restype, L.t_pivot.argtypes = None, [C.c_double, C.c_double, C.POINTER(C.c_uint64)] + [C.POINTER(C.c_float)] * 2
     L.t_held.restype, L.t_held.argtypes = C.c_double, [C.c_uint64]
     L.t_hold.restype, L.t_hold.argtypes = C.c_uint64, [C.c_double]
+    L.t_far.restype, L.t_far.argtypes = C.c_float, [C.c_double] * 4
     L.t_prod.restype, L.t_prod.argtypes = C.c_float, [C.c_double, C.c_uint64]
     L.t_narrow.restype, L.t_narrow.argtypes = C.c_float, [C.c_uint64]
     L.t_tab.restype, L.t_tab.argtypes = C.c_uint64, [C.c_int]
@@ -150,8 +153,6 @@ def test_pivot_of_any_increment(lib, kind):
 
 def test_single_precision_results(lib):
     """D and dtb D come out as the nearest floats of the fixed-point D's exact multiples."""
-    from fractions import Fraction
-
     rng = np.random.default_rng(12)
     D = [int(x) for x in rng.integers(1 << 60, 1 << 62, 4000)] + [1 << 62, (1 << 62) - 1, 3 << 60, (1 << 61) + (1 << 37)]
     b = [float(x) for x in 10.0 ** rng.uniform(-40, 0, len(D))]
@@ -163,3 +164,28 @@ def test_single_precision_results(lib):
             # nearest, but for products within 2^-34 of a tie (the high product's error)
             slack = Fraction(float(hi) - float(f)) / (1 << 34)
             assert err <= abs(Fraction(float(lo)) - exact) + slack and err <= abs(Fraction(float(hi)) - exact) + slack
+
+
+def test_far_lines_leave_the_continuum(lib):
+    """From far_profile on a line adds nothing to chi or eta, whatever the values' units (opacities
+    and emissivities from 1e-320 to 1e300), and not much nearer it still does."""
+    rng = np.random.default_rng(15)
+    add = lambda c, x, a: float(Fraction(c) + Fraction(x) * Fraction(2.0 ** -(a * a)))  # fused
+    near = 0
+    for _ in range(20000):
+        cc, ec = (float(10.0 ** rng.uniform(*r)) for r in ((-300, 300), (-320, 300)))
+        c0, e0 = float(cc * 10.0 ** rng.uniform(-30, 10)), float(ec * 10.0 ** rng.uniform(-30, 300))
+        if rng.random() < 0.2:
+            ec = 0.0
+        if rng.random() < 0.2:
+            c0 = 0.0
+        if not (c0 < 1e300 and e0 < 1e300):
+            continue
+        t = float(np.nextafter(np.float32(lib.t_far(cc, ec, c0, e0)), np.float32(0)))
+        if t < 30.9:
+            assert add(cc, c0, t) == cc and add(ec, e0, t) == ec
+            if t > 1.0:
+                near += int(add(cc, c0, t - 0.5) != cc or add(ec, e0, t - 0.5) != ec)
+    assert near > 5000
+    # an emissivity that is 0 in single precision, beside no continuum emissivity
+    assert lib.t_far(1.0, 0.0, 1e-20, 1e-50) == 31.0

@@ -87,3 +87,29 @@ def test_double_pivots_over_thick_and_thin_cells(orc, lines, bins, dtau_max):
     w = 2.0 / (12.0 * 4.0 ** (rays >> 28))
     for got in (J, batch, (w[:, :, None] * u).sum(1)):
         assert j_rel_err(got, Jo)[0] < 9.6e-6
+
+
+def emissivity_units(mgx, lines, bins, exponent, floor):
+    """J in FP64 of a patchy cloud with emissivities (and I_bdy) in units 2^-exponent of the
+    plain ones, in plain units; `floor`: the continuum's emissivity, of its plain one."""
+    m = synth.random_cloud(90, seed=5 + lines, n_lines=lines, n_freq=bins, x_span=4.0, l_min=1, l_max=1)
+    f = 10.0 ** np.random.default_rng(5 + lines).uniform(1, 3, 90)
+    s = 2.0 ** exponent
+    m = dict(m, chi0=m["chi0"] * f[:, None] * (1e-6 if floor == 0.0 else 1.0), eta0=m["eta0"] * f[:, None] * s,
+             chi_c=m["chi_c"] * f, eta_c=m["eta_c"] * f * s * floor)
+    ctx = mgx.Context(0)
+    try:
+        return ctx.solve_J(ctx.load(m), precision=mgx.MGX_FP64, I_bdy=0.05 * s * floor) / s
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("lines,bins", [(1, 20), (2, 33)])
+@pytest.mark.parametrize("exponent", [-155, -300])
+def test_small_emissivities(lines, bins, exponent):
+    """Line emissivities that single precision does not hold, over no continuum emissivity: powers of
+    two in the units change nothing but the exponents (1e-14: some roundings all the same)."""
+    import paper_2011_14998_gb300 as mgx
+
+    np.testing.assert_allclose(emissivity_units(mgx, lines, bins, exponent, 0.0), emissivity_units(mgx, lines, bins, 0, 0.0),
+                               rtol=1e-14)

@@ -707,10 +707,17 @@ __device__ __forceinline__ int stage_interval(const DevMesh &m, const DevLines &
             nv = kMaxSubdiv;
         }
         if constexpr (C::kInt) {
-            // the largest opacity any sample of the interval can reach
+            // the largest opacity any sample of the interval can reach; infinite, for plain_step,
+            // where a source function may pass 2^291: with Q to 2^301, increments to 1e60 and eight
+            // composed rows below 1e3 each (2^187), S Q times them stays below 2^1000
             R cb = fmax(sg.cc[pa], sg.cc[slot]);
+            int top = max(__double2hiint(sg.ec[pa]), __double2hiint(sg.ec[slot]));
 #pragma unroll
-            for (int l = 0; l < NL; ++l) cb += fmax(sg.ce[2 * l][pa], sg.ce[2 * l][slot]);
+            for (int l = 0; l < NL; ++l) {
+                cb += fmax(sg.ce[2 * l][pa], sg.ce[2 * l][slot]);
+                top = max(top, max(__double2hiint(sg.ce[2 * l + 1][pa]), __double2hiint(sg.ce[2 * l + 1][slot])));
+            }
+            if (top - min(__double2hiint(sg.cc[pa]), __double2hiint(sg.cc[slot])) > (290 << 20)) cb = INFINITY;
             sg.hq[slot] = cb * (1.0 + 0x1p-40);
         }
         return nv;
@@ -1911,7 +1918,8 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
 
 // One sample of the integer form outside what its fixed-point arithmetic
 // covers (profile arguments in steps of more than 31 per half-range, optical
-// depths beyond 1e60, continua below 1e-150): the plain double-precision step.
+// depths beyond 1e60, continua below 1e-150, source functions beyond 2^290): the
+// plain double-precision step.
 template <class C>
 __device__ __noinline__ void plain_step(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, int s_abs) {
     constexpr int NL = C::NL;

@@ -113,3 +113,14 @@ def test_small_emissivities(lines, bins, exponent):
 
     np.testing.assert_allclose(emissivity_units(mgx, lines, bins, exponent, 0.0), emissivity_units(mgx, lines, bins, 0, 0.0),
                                rtol=1e-14)
+
+
+@pytest.mark.parametrize("lines,bins", [(1, 20), (2, 33)])
+@pytest.mark.parametrize("exponent", [280, 300, 600, 800, 900])
+def test_large_emissivities(lines, bins, exponent):
+    """Source functions to 2^900 over optical depths of hundreds, which the homogeneous rows would
+    carry past the range: J in plain units within 64 rows of four roundings each."""
+    import paper_2011_14998_gb300 as mgx
+
+    np.testing.assert_allclose(emissivity_units(mgx, lines, bins, exponent, 1.0), emissivity_units(mgx, lines, bins, 0, 1.0),
+                               rtol=256 * 2.0 ** -53)

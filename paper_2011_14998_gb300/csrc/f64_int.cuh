@@ -101,6 +101,15 @@ __host__ __device__ __forceinline__ double exp2_neg_sq(uint64_t A, const uint64_
     return bits_double(((m + 512) >> 10) + (uint64_t(1021 - n) << 52));
 }
 
+// |alpha + u gamma| in Q7.57: alpha in Q6.57, gamma < 62 as gamma 2^(57 + sh) with
+// sh in its lowest three bits, u in Q0.63.  For alpha in (-63, 33) the sum is below
+// 95; from 64 on it is taken for a negative one of magnitude 128 less it, above 33,
+// where the profile is 0 all the same (exp2_neg_sq).
+__host__ __device__ __forceinline__ uint64_t arg_magnitude(uint64_t alpha, uint64_t g, uint64_t u) {
+    const uint64_t v = alpha + ((mul_hi63(u, g) << 1) >> (g & 7));
+    return v >> 63 ? 0 - v : v;
+}
+
 // log2 x for x >= 0 from its exponent and first 20 fraction bits, low by less
 // than 2^-18 for a normal x; an upper bound for a subnormal one and for 0.
 __host__ __device__ __forceinline__ float log2_bits(double x) {

@@ -879,12 +879,12 @@ __device__ __forceinline__ unsigned gen_sample_int(Stage<C> &sg, int k, int nv, 
             const double ah = dl * rs, al = fma(dl, rs, -ah);
             const double am = ah - gh, z = am - ah;
             const double aml = ((ah - (am - z)) - (gh + z)) + (al - gl);
-            wild |= !(gh < 31.0) || !(gh >= 0.0) || !(fabs(am) < 63.0);
+            wild |= !(gh < 31.0) || !(gh >= 0.0) || !(am > -63.0 && am < 33.0);
             const int ex = int(double_bits(gh) >> 52) - 1022;  // gh < 2^ex
             const int sh = ex < 1 ? 4 : ex > 5 ? 0 : 5 - ex;   // gamma 2^(57 + sh) = gh 2^(58 + sh) < 2^63
             const double up = bits_double(uint64_t(1023 + 58 + sh) << 52);
             uint64_t g = uint64_t(__double2ll_rn(gh * up) + __double2ll_rn(gl * up));
-            o[4] = __longlong_as_double(__double2ll_rn(am * 0x1p57) + __double2ll_rn(aml * 0x1p57));
+            o[4] = bits_double(uint64_t(__double2ll_rn(am * 0x1p57)) + uint64_t(__double2ll_rn(aml * 0x1p57)));
             o[5] = __longlong_as_double((long long)((g & ~uint64_t(7)) | uint64_t(sh)));
         }
     } else {
@@ -1631,10 +1631,7 @@ __device__ __forceinline__ void int_optics(const double *src, unsigned on, const
     eta = src[3];
     if constexpr (C::NL == 1) {
         if (!on) return;
-        const uint64_t g = double_bits(src[5]);
-        int64_t a = __double_as_longlong(src[4]) + int64_t((mul_hi63(u, g) << 1) >> (g & 7));
-        a = a < 0 ? -a : a;
-        const double e = exp2_neg_sq(uint64_t(a), tab);
+        const double e = exp2_neg_sq(arg_magnitude(double_bits(src[4]), double_bits(src[5]), u), tab);
         chi = fma(src[6], e, chi);
         eta = fma(src[7], e, eta);
     } else {

@@ -33,6 +33,7 @@ extern "C" double t_piv(double t, double b, uint64_t *Y) {
 extern "C" void t_pivot(double dt, double dtb, uint64_t *Y, float *D, float *bD) { mgx::pivot(dt, dtb, *Y, *D, *bD); }
 extern "C" double t_held(uint64_t Y) { return mgx::held_y(Y); }
 extern "C" uint64_t t_hold(double y) { return mgx::hold_y(y); }
+extern "C" uint64_t t_arg(uint64_t alpha, uint64_t g, uint64_t u) { return mgx::arg_magnitude(alpha, g, u); }
 extern "C" float t_far(double cc, double ec, double c0, double e0) { return mgx::far_profile(cc, ec, c0, e0); }
 extern "C" float t_prod(double b, uint64_t D) { return mgx::narrow_product(b, D); }
 extern "C" float t_narrow(uint64_t D) { return mgx::narrow_q62(D); }
@@ -54,6 +55,7 @@ def lib(tmp_path_factory):
     L.t_pivot.restype, L.t_pivot.argtypes = None, [C.c_double, C.c_double, C.POINTER(C.c_uint64)] + [C.POINTER(C.c_float)] * 2
     L.t_held.restype, L.t_held.argtypes = C.c_double, [C.c_uint64]
     L.t_hold.restype, L.t_hold.argtypes = C.c_uint64, [C.c_double]
+    L.t_arg.restype, L.t_arg.argtypes = C.c_uint64, [C.c_uint64] * 3
     L.t_far.restype, L.t_far.argtypes = C.c_float, [C.c_double] * 4
     L.t_prod.restype, L.t_prod.argtypes = C.c_float, [C.c_double, C.c_uint64]
     L.t_narrow.restype, L.t_narrow.argtypes = C.c_float, [C.c_uint64]
@@ -189,3 +191,23 @@ def test_far_lines_leave_the_continuum(lib):
     assert near > 5000
     # an emissivity that is 0 in single precision, beside no continuum emissivity
     assert lib.t_far(1.0, 0.0, 1e-20, 1e-50) == 31.0
+
+
+def test_profile_argument(lib):
+    """|alpha + u gamma| over the whole range the records have, its ends included: exact to three
+    units (the product's high half and the shift), or where it passes 31, past 31 as well."""
+    rng = np.random.default_rng(16)
+    span = [(-63.0, 33.0), (32.5, 33.0), (-63.0, -62.0)]
+    for k in range(30000):
+        alpha = int(rng.uniform(*span[k % 3]) * 2.0 ** 57)
+        gamma = float(rng.uniform(0, 62) if k % 5 else rng.uniform(61, 62)) if k % 2 else float(10.0 ** rng.uniform(-6, 0))
+        sh = max(0, min(4, 5 - (int(np.frexp(gamma / 2)[1]))))
+        g = int(gamma * 2.0 ** 57) << sh & ~7 | sh
+        u = int(rng.integers(0, 1 << 63)) if k % 7 else (1 << 63) - 1
+        assert g < 1 << 63
+        got = lib.t_arg(alpha & ((1 << 64) - 1), g, u)
+        exact = abs(alpha + (u * (g & ~7) >> 63 >> sh))
+        if exact >= 31 << 57:
+            assert got >= 31 << 57
+        else:
+            assert abs(got - exact) <= 3

@@ -821,11 +821,14 @@ __device__ __forceinline__ bool line_is_far(double dl, double rdv, double cc, do
 // alpha in Q6.57 and gamma scaled by the largest power
 // of two that keeps it below 2^63 (the shift back in its lowest three bits),
 // both from double products with their residuals, so that the cancellation
-// between them costs nothing.  More lines: delta and sqrt(log2 e) / dv.
+// between them costs nothing.  More lines, and one line where the origin's bins
+// span 31 widths of the sample or the argument starts beyond what Q6.57 holds
+// (kWide in `on`): delta and sqrt(log2 e) / dv.
 // Returns the mask of the lines that take part, bit 31 set when some bin may
-// need a split, bit 30 when the sample is outside what the fixed-point
-// arithmetic covers (plain_step takes it).
+// need a split, bit 30 when the sample is outside what consume_int's arithmetic
+// covers (consume_wide takes it, or plain_step).
 constexpr unsigned kSplitBit = 0x80000000u, kWildBit = 0x40000000u, kLineBits = 0x3fffffffu;
+constexpr unsigned kWide = 0x100u, kWideSplit = 0x200u;  // in `on`; kWideSplit: some bin may need a split
 
 template <class C>
 __device__ __forceinline__ unsigned gen_sample_int(Stage<C> &sg, int k, int nv, int j, int s_rec, int sign,
@@ -869,7 +872,7 @@ __device__ __forceinline__ unsigned gen_sample_int(Stage<C> &sg, int k, int nv, 
     const double top = sg.hq[k];  // bound of chi on the interval
     unsigned cls = on;
     if (!(top * ds <= dtau_max * (1.0 - 0x1p-38))) cls |= kSplitBit;
-    bool wild = !(top * ds < 1e60) || !(cc > 1e-150);
+    const bool wild = !(top * ds < 1e60) || !(cc > 1e-150);
     if constexpr (NL == 1) {
         if (on) {
             // gamma = 2 span (1 + delta/c) rs, alpha = delta rs - gamma / 2
@@ -879,13 +882,18 @@ __device__ __forceinline__ unsigned gen_sample_int(Stage<C> &sg, int k, int nv, 
             const double ah = dl * rs, al = fma(dl, rs, -ah);
             const double am = ah - gh, z = am - ah;
             const double aml = ((ah - (am - z)) - (gh + z)) + (al - gl);
-            wild |= !(gh < 31.0) || !(gh >= 0.0) || !(am > -63.0 && am < 33.0);
             const int ex = int(double_bits(gh) >> 52) - 1022;  // gh < 2^ex
             const int sh = ex < 1 ? 4 : ex > 5 ? 0 : 5 - ex;   // gamma 2^(57 + sh) = gh 2^(58 + sh) < 2^63
             const double up = bits_double(uint64_t(1023 + 58 + sh) << 52);
-            uint64_t g = uint64_t(__double2ll_rn(gh * up) + __double2ll_rn(gl * up));
+            const uint64_t g = uint64_t(__double2ll_rn(gh * up)) + uint64_t(__double2ll_rn(gl * up));
             o[4] = bits_double(uint64_t(__double2ll_rn(am * 0x1p57)) + uint64_t(__double2ll_rn(aml * 0x1p57)));
-            o[5] = __longlong_as_double((long long)((g & ~uint64_t(7)) | uint64_t(sh)));
+            o[5] = bits_double((g & ~uint64_t(7)) | uint64_t(sh));
+            if (!(gh < 31.0 && gh >= 0.0 && am > -63.0 && am < 33.0) && !wild) {
+                on |= cls & kSplitBit ? kWide | kWideSplit : kWide;
+                cls |= kWildBit | kSplitBit;
+                o[4] = dl;
+                o[5] = rs;
+            }
         }
     } else {
         o[4] = dl;
@@ -1623,13 +1631,14 @@ __device__ __forceinline__ void int_row(IntSweep &w, double S, double h, double 
     int_rescale(w);
 }
 
-// Opacity and emissivity of record src for bin i of the lane, over the lines in `on`.
-template <class C>
+// Opacity and emissivity of record src for bin i of the lane, over the lines in
+// `on`; kDouble: the argument in double precision (more lines, or kWide).
+template <class C, bool kDouble>
 __device__ __forceinline__ void int_optics(const double *src, unsigned on, const Stage<C> &sg, const uint64_t *tab,
                                            int i, uint64_t u, double &chi, double &eta) {
     chi = src[2];
     eta = src[3];
-    if constexpr (C::NL == 1) {
+    if constexpr (!kDouble) {
         if (!on) return;
         const double e = exp2_neg_sq(arg_magnitude(double_bits(src[4]), double_bits(src[5]), u), tab);
         chi = fma(src[6], e, chi);
@@ -1638,7 +1647,7 @@ __device__ __forceinline__ void int_optics(const double *src, unsigned on, const
         const int lane = threadIdx.x & 31;
 #pragma unroll 1
         for (; on; on &= on - 1) {
-            const int l = __ffs(int(on)) - 1;
+            const int l = C::NL == 1 ? 0 : __ffs(int(on)) - 1;
             const double a = fabs(fma(sg.fB[l][i][lane], src[4], sg.fA[l][i][lane]) * src[5]);
             const double e = a < 31.0 ? exp2_neg_sq(uint64_t(__double2ll_rn(a * 0x1p57)), tab) : 0.0;
             chi = fma(src[6 + 2 * l], e, chi);
@@ -1651,7 +1660,7 @@ __device__ __forceinline__ void int_optics(const double *src, unsigned on, const
 // The counts are the definition's: taken here where chi ds / dtau_max is
 // farther than its rounding from an integer, else left open (false is
 // returned, sg.fix marks the bins) and redone in the definition's own order.
-template <class C>
+template <class C, bool kDouble>
 __device__ __forceinline__ bool int_split_step(const double *src, unsigned on, bool fixed, Stage<C> &sg,
                                                const SolveArgs &a, const uint64_t *tab,
                                                const uint64_t (&u)[C::BPL], IntSweep (&w)[C::BPL]) {
@@ -1661,7 +1670,7 @@ __device__ __forceinline__ bool int_split_step(const double *src, unsigned on, b
     bool split = false;
 #pragma unroll
     for (int i = 0; i < C::BPL; ++i) {
-        int_optics<C>(src, on, sg, tab, i, u[i], chi[i], eta[i]);
+        int_optics<C, kDouble>(src, on, sg, tab, i, u[i], chi[i], eta[i]);
         split |= !(fmax(w[i].T, chi[i]) * (4.0 * q) <= a.dtau_max * (1.0 - 0x1p-45));
     }
     int n[C::BPL];
@@ -1784,15 +1793,9 @@ __device__ __forceinline__ unsigned compose_blocks(Stage<C> &sg, int lane, int n
     return starts;
 }
 
-// consume_chunk of the integer form.  Also returns at a sample that the
-// fixed-point arithmetic does not cover (sg.m_wild), for plain_step.
+// The lane's state of the integer form to and from shared memory.
 template <class C>
-__device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, const uint64_t *tab, int total,
-                                        int nch, int sign, int pos, int pend, bool fresh) {
-    constexpr int kS = Stage<C>::kS, kCap = Stage<C>::kCap;
-    const int lane = threadIdx.x & 31;
-    IntSweep w[C::BPL];
-    uint64_t u[C::BPL];
+__device__ __forceinline__ void get_int(const Lane<C> &ln, IntSweep (&w)[C::BPL], int lane) {
 #pragma unroll
     for (int i = 0; i < C::BPL; ++i) {
         w[i].N = ln.wp[0][i][lane];
@@ -1801,8 +1804,33 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
         w[i].W = ln.wr[0][i][lane];
         w[i].T = ln.wr[1][i][lane];
         w[i].S = ln.wr[2][i][lane];
-        u[i] = C::NL == 1 ? sg.uk[i][lane] : 0;
     }
+}
+
+template <class C>
+__device__ __forceinline__ void put_int(Lane<C> &ln, const IntSweep (&w)[C::BPL], int lane) {
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) {
+        ln.wp[0][i][lane] = div_pos(w[i].N, w[i].Q);
+        ln.wp[1][i][lane] = w[i].h;
+        ln.wr[0][i][lane] = copysign(div_pos(fabs(w[i].W), w[i].Q), w[i].W);
+        ln.wr[1][i][lane] = w[i].T;
+        ln.wr[2][i][lane] = w[i].S;
+    }
+}
+
+// consume_chunk of the integer form.  Also returns at a sample that its
+// arithmetic does not cover (sg.m_wild), for consume_wide or plain_step.
+template <class C>
+__device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, const uint64_t *tab, int total,
+                                        int nch, int sign, int pos, int pend, bool fresh) {
+    constexpr int kS = Stage<C>::kS, kCap = Stage<C>::kCap;
+    const int lane = threadIdx.x & 31;
+    IntSweep w[C::BPL];
+    uint64_t u[C::BPL];
+    get_int<C>(ln, w, lane);
+#pragma unroll
+    for (int i = 0; i < C::BPL; ++i) u[i] = C::NL == 1 ? sg.uk[i][lane] : 0;
     int r0 = pos / kCap * kCap, s = pos - r0;
 #pragma unroll 1
     for (; r0 < total; r0 += kCap, s = 0, fresh = true) {
@@ -1842,7 +1870,7 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
             const unsigned on = sg.on[s];
             if ((m_split >> s) & 1u) {
                 if ((m_wild >> s) & 1u) break;
-                if (!int_split_step<C>(src, on, r0 + s == pend, sg, a, tab, u, w)) break;
+                if (!int_split_step<C, (C::NL > 1)>(src, on, r0 + s == pend, sg, a, tab, u, w)) break;
                 ++s;
                 continue;
             }
@@ -1889,7 +1917,7 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
 #pragma unroll
                     for (int i = 0; i < C::BPL; ++i) {
                         double chi, eta;
-                        int_optics<C>(src, on, sg, tab, i, u[i], chi, eta);
+                        int_optics<C, (C::NL > 1)>(src, on, sg, tab, i, u[i], chi, eta);
                         const double h = src[0] * (w[i].T + chi);
                         int_row(w[i], w[i].S, h, w[i].h + h);
                         w[i].T = chi;
@@ -1901,22 +1929,55 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
         if (s < nr) break;
         __syncwarp();
     }
-#pragma unroll
-    for (int i = 0; i < C::BPL; ++i) {
-        ln.wp[0][i][lane] = div_pos(w[i].N, w[i].Q);
-        ln.wp[1][i][lane] = w[i].h;
-        ln.wr[0][i][lane] = copysign(div_pos(fabs(w[i].W), w[i].Q), w[i].W);
-        ln.wr[1][i][lane] = w[i].T;
-        ln.wr[2][i][lane] = w[i].S;
-    }
+    put_int<C>(ln, w, lane);
     __syncwarp();
     return r0 < total ? r0 + s : total;
 }
 
+// Of one line: the kWide samples from `pos` on that follow one another in the
+// round, the profile argument in double precision.  Returns the sample after
+// them, or the complement of one whose count was left open (int_split_step).  A
+// function of its own: in consume_int's loop the choice cost every other sample
+// (4001-point wind 101.3 -> 102.2 ms).  A slow wind of 4001 points, widths spread
+// by 10 either way, bins to 4 and 16 widths: 67 -> 47 and 107 -> 52 ms against the
+// plain step for every such sample.
+template <class C>
+__device__ __noinline__ int consume_wide(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, const uint64_t *tab, int total,
+                                         int pos, int pend) {
+    constexpr int kS = Stage<C>::kS, kCap = Stage<C>::kCap;
+    const int lane = threadIdx.x & 31;
+    IntSweep w[C::BPL];
+    get_int<C>(ln, w, lane);
+    const uint64_t none[C::BPL] = {};
+    const int r0 = pos / kCap * kCap, nr = total - r0 < kCap ? total - r0 : kCap;
+    int s = pos - r0;
+    bool open = false;
+#pragma unroll 1
+    for (; s < nr && (sg.on[s] & kWide) != 0u; ++s) {
+        const double *src = sg.rec + s * kS;
+        if (sg.on[s] & kWideSplit) {
+            open = !int_split_step<C, true>(src, 1u, r0 + s == pend, sg, a, tab, none, w);
+            if (open) break;
+            continue;
+        }
+#pragma unroll
+        for (int i = 0; i < C::BPL; ++i) {
+            double chi, eta;
+            int_optics<C, true>(src, 1u, sg, tab, i, 0, chi, eta);
+            const double h = src[0] * (w[i].T + chi);
+            int_row(w[i], w[i].S, h, w[i].h + h);
+            w[i].T = chi;
+            w[i].S = div_pos(eta, chi);
+        }
+    }
+    put_int<C>(ln, w, lane);
+    __syncwarp();
+    return open ? ~(r0 + s) : r0 + s;
+}
+
 // One sample of the integer form outside what its fixed-point arithmetic
-// covers (profile arguments in steps of more than 31 per half-range, optical
-// depths beyond 1e60, continua below 1e-150, source functions beyond 2^290): the
-// plain double-precision step.
+// covers (optical depths beyond 1e60, continua below 1e-150, source functions
+// beyond 2^290): the plain double-precision step.
 template <class C>
 __device__ __noinline__ void plain_step(Stage<C> &sg, Lane<C> &ln, const SolveArgs &a, int s_abs) {
     constexpr int NL = C::NL;
@@ -2090,11 +2151,18 @@ __device__ void half_sweep(const DevMesh &m, const DevLines &Ln, const SolveArgs
                 pos = consume_int<C>(sg, ln, a, tab, total, nch, sign, pos, pend, fresh);
                 if (pos >= total) break;
                 if ((sg.m_wild >> pos % Stage<C>::kCap) & 1u) {
-                    plain_step<C>(sg, ln, a, pos);
-                    ++pos;
-                    fresh = pos % Stage<C>::kCap == 0;
+                    int next = pos + 1;  // the complement of a sample left open
+                    if (NL == 1 && (sg.on[pos % Stage<C>::kCap] & kWide) != 0u) {
+                        if constexpr (NL == 1) next = consume_wide<C>(sg, ln, a, tab, total, pos, pend);
+                    } else {
+                        plain_step<C>(sg, ln, a, pos);
+                    }
+                    pos = next < 0 ? ~next : next;
                     if (pos >= total) break;
-                    continue;
+                    if (next >= 0) {
+                        fresh = pos % Stage<C>::kCap == 0;
+                        continue;
+                    }
                 }
             } else {
                 pos = consume_chunk<C>(sg, ln, a, total, nch, sign, pos, pend, fresh);

@@ -124,3 +124,56 @@ def test_large_emissivities(lines, bins, exponent):
 
     np.testing.assert_allclose(emissivity_units(mgx, lines, bins, exponent, 1.0), emissivity_units(mgx, lines, bins, 0, 1.0),
                                rtol=256 * 2.0 ** -53)
+
+
+def fp64_error(orc, m, **kw):
+    import paper_2011_14998_gb300 as mgx
+
+    ctx = mgx.Context(0)
+    try:
+        mid = ctx.load(m)
+        rays = ctx.rays(mid)
+        J = ctx.solve_J(mid, precision=mgx.MGX_FP64, I_bdy=0.05, **kw)
+    finally:
+        ctx.close()
+    return j_rel_err(J, orc.OracleModel(m, rays=rays).solve_J(orc.params(I_bdy=0.05, **kw)))[0]
+
+
+@pytest.mark.parametrize("bins", [1, 20, 64, 100])
+@pytest.mark.parametrize("x_span,ratio", [(4.0, 20.0), (16.0, 10.0), (16.0, 1.0), (13.0, 1.0), (64.0, 3.0)])
+def test_fp64_wide_arguments(orc, bins, x_span, ratio):
+    """One line whose profile arguments span 31 widths and more on some samples and fewer on others
+    (the argument's two forms).  The argument carries five roundings, so an opacity 72 times that
+    in its wings (|a| to 6) and J some ten times more: 1e-12 covers both sides."""
+    m = synth.random_cloud(120, seed=bins, n_lines=1, n_freq=bins, x_span=x_span, l_min=1, l_max=1)
+    m = dict(m, dvw=m["dvw"] * ratio ** np.random.default_rng(bins).uniform(-1, 1, 120))
+    assert fp64_error(orc, m) < 1e-12
+
+
+def test_fp64_plain_samples_between_others(orc):
+    """Continua below 1e-150 at a third of the points: samples the fixed-point form leaves to the plain
+    step, single and in a row, at any place of a round of records."""
+    rng = np.random.default_rng(3)
+    m = synth.random_cloud(200, seed=3, n_lines=1, n_freq=40, x_span=4.0, l_min=1, l_max=1)
+    tiny = np.where(rng.random(200) < 0.3, 1e-160, 1.0)
+    assert fp64_error(orc, dict(m, chi_c=m["chi_c"] * tiny, eta_c=m["eta_c"] * tiny)) < 1e-12
+
+
+@pytest.mark.parametrize("lines", [1, 2, 5])
+def test_fp64_composed_rows(orc, lines):
+    """A long static bar, most of it without line opacity, so that its rows are composed by eight, with
+    thick cells (split, or too thick to compose) and cells with lines between them.  Some 200 rows of six
+    roundings each, on both sides: 3e-13."""
+    rng = np.random.default_rng(lines)
+    g = np.stack(np.meshgrid(np.arange(60.0), np.arange(3.0), np.arange(3.0), indexing="ij"), -1).reshape(-1, 3)
+    pos = g + rng.uniform(-0.2, 0.2, g.shape)
+    off, nbr = synth.delaunay_csr(pos)
+    n = len(pos)
+    m = synth.random_cloud(n, seed=lines, n_lines=lines, n_freq=40, l_min=1, l_max=1)
+    on = (rng.random(n) < 0.04)[:, None]
+    thick = np.where(rng.random(n) < 0.03, 10.0 ** rng.uniform(1, 4, n), 1.0)
+    chi_c = 10.0 ** rng.uniform(-2, -0.5, n) * thick
+    m = dict(m, pos=pos, vel=np.zeros((n, 3)), nbr_off=off, nbr_idx=nbr, chi0=m["chi0"] * on, eta0=m["eta0"] * on,
+             chi_c=chi_c, eta_c=chi_c * rng.uniform(0.2, 1.5, n))
+    for dtau_max in (0.5, 1e5):
+        assert fp64_error(orc, m, dtau_max=dtau_max) < 3e-13

@@ -164,36 +164,72 @@ __device__ bool vec2pix_nest_f(int l, float a, float b, float c, int32_t &pix) {
     return true;
 }
 
-// The direction between two points from their positions split into two floats
-// each (hi = fl(x), lo = fl(x - hi)): a double subtraction takes the FP64 pipe
-// 77 cycles a warp.  X bounds |x|_1 over the mesh.  Each component carries the
-// roundings of the two differences and their sum, 2.01u of itself, and
-// 2^-45.5 X from the split and the cancellation; false (the double path decides)
-// unless the largest component is at least 2^-17 X, so that the latter is below
-// 0.05u of it, the horizontal part at least 1/16 of it, and its square far from
-// the ends of the float range.
+// The power of two that brings the mesh's X, which bounds |x|_1, to [1, 2), and X
+// so scaled: the screen then sees the same numbers in any unit of length.
+__device__ __forceinline__ double mesh_scale(const DevMesh &m, float &X) {
+    const uint32_t b = __float_as_uint(m.g0 * 8796093022208.0f);  // g0 >= 2^-43 max |x|_1, and 1e-37
+    X = __uint_as_float((b & 0x7fffffu) | 0x3f800000u);
+    return __longlong_as_double((long long)(1150u - (b >> 23)) << 52);
+}
+
+// A position's coordinate, scaled, as two floats.
+__device__ __forceinline__ void split_coordinate(double x, double scale, float &hi, float &lo) {
+    x = __dmul_rn(x, scale);
+    hi = __double2float_rn(x);
+    lo = __double2float_rn(__dsub_rn(x, double(hi)));
+}
+
+// The direction between two points from their scaled positions split into two
+// floats each (hi = fl(x), lo = fl(x - hi)): a double subtraction takes the FP64
+// pipe 77 cycles a warp.  Each component carries the roundings of the two
+// differences and their sum, 2.01u of itself, and 2^-45.5 X from the split and the
+// cancellation; false (scaled_direction takes it) unless the largest component is
+// at least 2^-17 X, so that the latter is below 0.05u of it, and the horizontal
+// part at least 1/16 of it.
 __device__ __forceinline__ bool split_direction(const float4 &h, const float4 &l, const float4 &oh, const float4 &ol,
                                                 float X, float &a, float &b, float &c) {
     a = (h.x - oh.x) + (l.x - ol.x);
     b = (h.y - oh.y) + (l.y - ol.y);
     c = (h.z - oh.z) + (l.z - ol.z);
     const float hor = fmaxf(fabsf(a), fabsf(b)), M = fmaxf(hor, fabsf(c));
-    return M >= 7.62939453125e-6f * X && hor >= 0.0625f * M && M > 1e-15f && M < 1e15f;
+    return M >= 7.62939453125e-6f * X && hor >= 0.0625f * M;
 }
 
-// The sample's positions split (x, y, z of sp[2s] and sp[2s + 1]), the point's
-// index in sp[2s].w (-1: out of range).
+// The direction in single precision from the double differences, scaled by the
+// power of two of the largest: each component within u of itself (2^-99 of the
+// largest where it is left out).  False when all are 0 or next to the end of the range.
+__device__ __forceinline__ bool scaled_direction(double dx, double dy, double dz, float &a, float &b, float &c) {
+    auto field = [](double d) { return (__double2hiint(d) >> 20) & 0x7ff; };
+    const int top = max(field(dx), max(field(dy), field(dz)));
+    if (top <= 100) return false;
+    auto part = [&](double d) {
+        if (field(d) + 100 < top) return 0.0f;
+        return __double2float_rn(__hiloint2double(__double2hiint(d) + (1023 - top) * (1 << 20), __double2loint(d)));
+    };
+    a = part(dx);
+    b = part(dy);
+    c = part(dz);
+    return true;
+}
+
+// The sample's positions scaled and split (x, y, z of sp[2s] and sp[2s + 1]), the
+// point's index in sp[2s].w (-1: out of range).
 __global__ void k_split_sample(DevMesh m, int64_t n_sample, const int32_t *__restrict__ sample,
                                float4 *__restrict__ sp) {
     const int64_t s = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (s >= n_sample) return;
     const int32_t j = sample[s];
     const bool ok = j >= 0 && j < m.n;
-    const double x = ok ? m.x[j] : 0.0, y = ok ? m.y[j] : 0.0, z = ok ? m.z[j] : 0.0;
-    const float hx = __double2float_rn(x), hy = __double2float_rn(y), hz = __double2float_rn(z);
-    sp[2 * s] = make_float4(hx, hy, hz, __int_as_float(ok ? j : -1));
-    sp[2 * s + 1] = make_float4(__double2float_rn(__dsub_rn(x, double(hx))), __double2float_rn(__dsub_rn(y, double(hy))),
-                                __double2float_rn(__dsub_rn(z, double(hz))), 0.0f);
+    float X;
+    const double scale = mesh_scale(m, X);
+    float4 h = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(ok ? j : -1)), l = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (ok) {
+        split_coordinate(m.x[j], scale, h.x, l.x);
+        split_coordinate(m.y[j], scale, h.y, l.y);
+        split_coordinate(m.z[j], scale, h.z, l.z);
+    }
+    sp[2 * s] = h;
+    sp[2 * s + 1] = l;
 }
 
 // atan2f as the single-precision ray-set screen evaluates it (for the tests of kAtanErr).
@@ -236,50 +272,82 @@ k_rays_adaptive(DevMesh m, int32_t lmin, int32_t lmax, int32_t npairs, int64_t n
     if (tid == 0) nout = 0;
     __syncthreads();
     const double xo = m.x[o], yo = m.y[o], zo = m.z[o];
-    // Single precision where the screen certifies the pixel.  The directions it leaves
-    // open (below a per cent) wait in a list of the warp and take the double path 32 at
-    // a time: taken at once, by one lane, they cost the whole warp the double path's
-    // 100-odd FP64 instructions (77 cycles each) in a third of its steps.  30 000 points
-    // with 10 000 directions each: 19.4 ms so, 9.7 with the list, 5.3 with the split
-    // positions and 32-bit indices in place of FP64 differences and 64-bit ones.
+    // Single precision where the screen certifies the pixel, from the split positions or,
+    // where they do not carry the direction (a distance below 2^-17 of the mesh's farthest
+    // point from the coordinate origin; next to the z axis), from the double differences.
+    // The directions that need either (`far`) or that the screen leaves open (`open`, below
+    // a per cent) wait in lists of the warp and are taken 32 at a time: taken at once, by one
+    // lane, they cost the whole warp the double path's 100-odd FP64 instructions (77 cycles
+    // each) in a third of its steps.  30 000 points with 10 000 directions each: 19.4 ms so,
+    // 9.7 with the list, 5.2 with the split positions and 32-bit indices in place of FP64
+    // differences and 64-bit ones, 3.7 with the second list; 3.7 in any unit of length, 5.4 and
+    // 4.9 when the mesh (of 100) is moved by 1e6 and 1e9 (with one list 57 in units of 1e16 or
+    // when moved by 1e9, 31 when moved by 1e6).
     constexpr int kList = 64;
-    __shared__ int32_t list[256 / 32][kList];
+    __shared__ int32_t lists[256 / 32][2][kList];
     const int lane = tid & 31;
-    int32_t *mine = list[tid >> 5];
-    int waiting = 0;
+    int32_t *far = lists[tid >> 5][0], *open = lists[tid >> 5][1];
+    int n_far = 0, n_open = 0;
+    auto push = [&](int32_t *list, int &n, bool on, int32_t j) {  // returns whether 32 are waiting
+        const unsigned mask = __ballot_sync(0xffffffffu, on);
+        if (on) list[n + __popc(mask & ((1u << lane) - 1u))] = j;
+        n += __popc(mask);
+        __syncwarp();
+        return n >= 32;
+    };
     auto exact = [&](int32_t j) {
         const double dx = __dsub_rn(m.x[j], xo), dy = __dsub_rn(m.y[j], yo), dz = __dsub_rn(m.z[j], zo);
         if (dx == 0.0 && dy == 0.0 && dz == 0.0) return;  // a coincident point has no direction
         atomicAdd(&hist[lmax][vec2pix_nest(lmax, dx, dy, dz)], 1u);
     };
-    const float4 oh = make_float4(__double2float_rn(xo), __double2float_rn(yo), __double2float_rn(zo), 0.0f);
-    const float4 ol = make_float4(__double2float_rn(__dsub_rn(xo, double(oh.x))), __double2float_rn(__dsub_rn(yo, double(oh.y))),
-                                  __double2float_rn(__dsub_rn(zo, double(oh.z))), 0.0f);
-    const float X = m.g0 * 8796093022208.0f;  // g0 >= 2^-43 max |x|_1
+    auto take_open = [&]() {
+        n_open -= 32;
+        exact(open[n_open + lane]);
+        __syncwarp();
+    };
+    auto take_far = [&](bool on, int32_t j) {
+        float a, b, c;
+        int32_t pix;
+        bool left = false;
+        if (on) {
+            left = !scaled_direction(__dsub_rn(m.x[j], xo), __dsub_rn(m.y[j], yo), __dsub_rn(m.z[j], zo), a, b, c) ||
+                   !vec2pix_nest_f(lmax, a, b, c, pix);
+            if (!left) atomicAdd(&hist[lmax][pix], 1u);
+        }
+        if (push(open, n_open, left, j)) take_open();
+    };
+    float X;
+    const double scale = mesh_scale(m, X);
+    float4 oh, ol;
+    split_coordinate(xo, scale, oh.x, ol.x);
+    split_coordinate(yo, scale, oh.y, ol.y);
+    split_coordinate(zo, scale, oh.z, ol.z);
     for (int64_t s0 = tid - lane; s0 < n_sample; s0 += nt) {
         int32_t j = -1;
-        bool open = false;
+        bool is_far = false, is_open = false;
         if (s0 + lane < n_sample) {
             const float4 h = __ldg(sp + 2 * (s0 + lane)), l = __ldg(sp + 2 * (s0 + lane) + 1);
             j = __float_as_int(h.w);
             if (j >= 0 && j != o) {
                 float a, b, c;
                 int32_t pix;
-                open = !split_direction(h, l, oh, ol, X, a, b, c) || !vec2pix_nest_f(lmax, a, b, c, pix);
-                if (!open) atomicAdd(&hist[lmax][pix], 1u);
+                is_far = !split_direction(h, l, oh, ol, X, a, b, c);
+                if (!is_far) {
+                    is_open = !vec2pix_nest_f(lmax, a, b, c, pix);
+                    if (!is_open) atomicAdd(&hist[lmax][pix], 1u);
+                }
             }
         }
-        const unsigned mask = __ballot_sync(0xffffffffu, open);
-        if (open) mine[waiting + __popc(mask & ((1u << lane) - 1u))] = j;
-        waiting += __popc(mask);
-        __syncwarp();
-        if (waiting >= 32) {
-            waiting -= 32;
-            exact(mine[waiting + lane]);
+        if (push(open, n_open, is_open, j)) take_open();
+        if (push(far, n_far, is_far, j)) {
+            n_far -= 32;
+            const int32_t q = far[n_far + lane];
             __syncwarp();
+            take_far(true, q);
         }
     }
-    if (lane < waiting) exact(mine[lane]);
+    take_far(lane < n_far, lane < n_far ? far[lane] : 0);
+    if (lane < n_open) exact(open[lane]);
     __syncthreads();
     for (int l = lmax - 1; l >= lmin; --l) {
         const int32_t np = int32_t(int64_t(12) << (2 * l));

@@ -94,3 +94,28 @@ def test_reduction_sweep_speedup_grows(ctx):
         c = np.asarray(r["cdf"])
         assert len(c) == 1000 and np.all(np.diff(c) >= 0) and abs(c[-1] - 1.0) < 1e-12
         assert np.isfinite(r["mean_rel_err"])
+
+
+@pytest.mark.parametrize("unit", [0, 53, 66, -53, -75, -97])
+@pytest.mark.parametrize("kind", ["cloud", "clump", "lattice", "far", "farther"])
+def test_adaptive_ray_sets_in_any_unit(ctx, orc, kind, unit):
+    """Ray sets where the single-precision screen gets its directions by each of its ways: near and far
+    from the coordinate origin, between points that all but coincide, along the axes, in units from
+    2^-97 to 2^66; the oracle's, bit for bit."""
+    import synth
+
+    m = synth.random_cloud(300, seed=9, l_min=0, l_max=3)
+    pos = m["pos"].copy()
+    if kind == "clump":
+        pos[150:] = pos[:150] + 1e-7 * (pos[150:] - 0.5)
+    elif kind == "lattice":
+        pos = np.stack(np.meshgrid(*[np.arange(7.0)] * 3, indexing="ij"), -1).reshape(-1, 3)[:300]
+    elif kind == "far":
+        pos += 2.0 ** 12
+    elif kind == "farther":
+        pos += 2.0 ** 30
+    pos = pos * 2.0 ** unit
+    mid = ctx.load(dict(m, pos=pos))
+    rays = ctx.rays(mid)
+    ctx.free(mid)
+    np.testing.assert_array_equal(rays, orc.rayset(pos, 0, 3, m["sample"]))

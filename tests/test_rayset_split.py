@@ -66,3 +66,45 @@ def test_without_the_limit_the_bounds_fail():
     ok &= ~(x == o).all(1)
     _, _, ephi = errors(d[ok], x[ok], o[ok])
     assert (ephi > 3.3 * U).any()
+
+
+def scaled(x, o):
+    """Positions times the power of two that brings the largest |x|_1 to [1, 2), and that largest value."""
+    X = max(np.abs(x).sum(1).max(), np.abs(o).sum(1).max())
+    s = 2.0 ** -np.floor(np.log2(float(f32(X))))
+    return x * s, o * s, f32(X * s)
+
+
+def scaled_direction(e):
+    """From the double differences, by the largest component's power of two (components below 2^-100 of it 0)."""
+    top = np.frexp(np.abs(e).max(1))[1][:, None]
+    d = np.ldexp(e, 1 - top)
+    return np.where(np.abs(d) < 2.0 ** -99, 0.0, d).astype(f32)
+
+
+def test_any_unit_of_length():
+    """Scaled positions: as many directions as in plain units, within the same bounds, whatever the unit."""
+    counts = set()
+    x, o = pairs(np.random.default_rng(21), 40000, 1.0)
+    for k in (-97, -53, -20, 0, 20, 53, 90):
+        xs, os_, X = scaled(x * 2.0 ** k, o * 2.0 ** k)
+        d, ok = direction(xs, os_, X)
+        assert not ok[(x == o).all(1)].any()
+        ez, z, ephi = errors(d[ok], x[ok], o[ok])
+        assert (ez <= 6.5 * U * z + 0.1 * U).all() and (ephi <= 3.3 * U).all()
+        counts.add(int(ok.sum()))
+    X = f32(max(np.abs(x).sum(1).max(), np.abs(o).sum(1).max()))
+    assert counts == {int(direction(x, o, X)[1].sum())}
+
+
+def test_directions_from_double_differences():
+    """Where the split positions do not carry it: within the bounds for every direction, near points of a far
+    mesh and directions along the axis included."""
+    rng = np.random.default_rng(22)
+    for scale in (1e-28, 1.0, 1e28):
+        x, o = pairs(rng, 40000, scale)
+        x[:2000] = o[:2000] + np.stack([np.zeros(2000), np.zeros(2000), rng.normal(size=2000) * scale], 1)
+        use = ~(x == o).all(1)
+        d = scaled_direction((x - o)[use])
+        ez, z, ephi = errors(d, x[use], o[use])
+        assert (ez <= 6.5 * U * z + 0.1 * U).all() and (ephi <= 3.3 * U).all()

@@ -279,6 +279,9 @@ enum {
  *           tuning replay the graph without host work.  A replay whose traced
  *           lists no longer fit the planned layout fails with MGX_ERANGE and
  *           drops the plan.  Freeing a model drops the plan.
+ * A batch of few items deals the pairs of an origin to several warps; its plan
+ * then also holds every pair's u (8 n_k pairs_k n_lines_k n_freq_k bytes, at most
+ * 1 GiB in all), unless there is no room for it.
  * The call synchronises the stream before returning. */
 mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_models, const mgx_solve_params *params,
                              double *const *J_out, int32_t flags);

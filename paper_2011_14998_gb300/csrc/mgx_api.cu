@@ -1273,11 +1273,6 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
         max_tiles = std::max(max_tiles, int32_t(std::min<int64_t>(tiles, 65535)));
     }
     pl.parts = std::min(solve_parts(p->precision, n_items, min_pairs, n_u * sizeof(double)), 65535 / max_tiles);
-    if (pl.parts > 1 && dalloc(ctx, &pl.u, n_u) != cudaSuccess) {  // no room for u: one warp per item
-        cudaGetLastError();
-        pl.u = nullptr;
-        pl.parts = 1;
-    }
     for (int32_t k = 0; k < n_models; ++k) {
         const Model &m = *ms[size_t(k)];
         const int64_t nb = int64_t(m.L) * m.F;
@@ -1372,6 +1367,19 @@ mgx_status mgx_solve_J_batch(mgx_ctx *ctx, const int32_t *models, int32_t n_mode
     pl.tail_cap = int64_t(tot[j]);
     pl.total_points = int64_t(tot[kPadCandidates]);
     CK(dalloc(ctx, &pl.tail, size_t(std::max<int64_t>(pl.tail_cap, 1))));
+    // u last, after what the step cannot do without: no room for it, one warp per item
+    if (pl.parts > 1 && dalloc(ctx, &pl.u, n_u) != cudaSuccess) {
+        cudaGetLastError();
+        pl.u = nullptr;
+        pl.n_work = 0;
+        for (int32_t k = 0; k < n_models; ++k) {
+            geo[size_t(k)].n_tiles /= pl.parts;
+            geo[size_t(k)].work_base = pl.n_work;
+            pl.n_work += int64_t(ms[size_t(k)]->n) * geo[size_t(k)].n_tiles;
+        }
+        pl.parts = 1;
+        CK(cudaMemcpyAsync(pl.geo, geo.data(), geo.size() * sizeof(BatchGeom), cudaMemcpyHostToDevice, ctx->stream));
+    }
     std::vector<BatchSlot> slots(static_cast<size_t>(n_models));
     size_t u_off = 0;
     for (int32_t k = 0; k < n_models; ++k) {

@@ -145,3 +145,66 @@ def test_autotune_keeps_fastest_candidate(setup):
     for o, r in zip(outs, ref):
         assert j_rel_err(o.cpu().numpy(), r)[0] < 1e-5
     ctx.set_tuning(None)
+
+
+class LimitedPool:
+    """The device's current memory pool replaced by one of at most `limit` bytes (0: no limit)."""
+
+    def __init__(self, limit):
+        import ctypes as C
+
+        class Props(C.Structure):
+            _fields_ = [("alloc_type", C.c_int), ("handle_types", C.c_int), ("location_type", C.c_int),
+                        ("location_id", C.c_int), ("security", C.c_void_p), ("max_size", C.c_size_t),
+                        ("usage", C.c_ushort), ("reserved", C.c_ubyte * 54)]
+
+        self.C, self.cu = C, C.CDLL("libcuda.so.1")
+        self.props = Props(alloc_type=1, location_type=1, max_size=limit)  # pinned, on device 0
+        self.pool, self.before = C.c_void_p(), C.c_void_p()
+
+    def __enter__(self):
+        assert self.cu.cuDeviceGetMemPool(self.C.byref(self.before), 0) == 0
+        assert self.cu.cuMemPoolCreate(self.C.byref(self.pool), self.C.byref(self.props)) == 0
+        assert self.cu.cuDeviceSetMemPool(0, self.pool) == 0
+        return self
+
+    def used_high(self):
+        v = self.C.c_uint64()
+        assert self.cu.cuMemPoolGetAttribute(self.pool, 8, self.C.byref(v)) == 0  # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+        return v.value
+
+    def __exit__(self, *_):
+        assert self.cu.cuDeviceSetMemPool(0, self.before) == 0
+        assert self.cu.cuMemPoolDestroy(self.pool) == 0
+
+
+@pytest.mark.parametrize("batch", [True, False])
+def test_without_room_for_u(batch):
+    """Few items: u of every pair takes half of the call's memory.  Where there is room for it or for the
+    rest, but not for both, the call goes on with one warp per item, and J is the same bit for bit."""
+    import torch
+
+    import synth
+
+    import paper_2011_14998_gb300 as mgx
+
+    torch.zeros(1, device="cuda")
+    m = synth.random_cloud(400, seed=2, n_lines=1, n_freq=20, l_min=4, l_max=4)
+    u_bytes = 400 * 1536 * 20 * 8
+
+    def call(limit):
+        with LimitedPool(limit) as pool:
+            ctx = mgx.Context(0)
+            try:
+                mid = ctx.load(m)
+                J = (ctx.solve_J_batch([mid], precision=mgx.MGX_FP32)[0].cpu().numpy() if batch
+                     else ctx.solve_J(mid, precision=mgx.MGX_FP32))
+                return J, pool.used_high()
+            finally:
+                ctx.close()
+                torch.cuda.synchronize()
+
+    J, high = call(0)
+    assert high > u_bytes  # u was held
+    rest = high - u_bytes
+    np.testing.assert_array_equal(call(high - min(u_bytes, rest) // 2)[0], J)

@@ -807,6 +807,7 @@ mgx_status mgx_set_rays(mgx_ctx *ctx, int32_t model, int32_t l_min, int32_t l_ma
     mgx_status s = ensure_tables(ctx, l_max);
     if (s != MGX_OK) return s;
     drop_offsets(ctx, *m);
+    m->has_rays = false;  // until the new set is complete: an allocation may fail on the way
     if (!m->rays || m->npairs != np) {
         dfree(ctx, m->rays);
         CK(dalloc(ctx, &m->rays, size_t(m->n) * size_t(np)));

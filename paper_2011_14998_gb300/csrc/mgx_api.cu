@@ -450,6 +450,13 @@ void free_plan(mgx_ctx *ctx, BatchPlan &pl) {
     pl.valid = false;
 }
 
+// Drop the plan when `model` is in it: its slots and its graph hold the arrays'
+// addresses, and its layout goes with the lines' and the rays' numbers.
+void drop_plan_of(mgx_ctx *ctx, int32_t model) {
+    BatchPlan &pl = ctx->plan;
+    if (std::find(pl.models.begin(), pl.models.end(), model) != pl.models.end()) free_plan(ctx, pl);
+}
+
 // Rebuild the ray set of a model with its current levels and sample (enqueue only).
 void enqueue_rays(mgx_ctx *ctx, Model &m, bool timed = true) {
     Timed t(ctx, timed ? MGX_K_RAYS : -1);
@@ -756,6 +763,7 @@ mgx_status mgx_set_lines(mgx_ctx *ctx, int32_t model, int32_t n_lines, const dou
     for (int l = 0; l < n_lines; ++l)
         if (!std::isfinite(nu0[l]) || !(nu0[l] > 0.0)) return fail(ctx, MGX_EINVAL, "set_lines: nu0[%d] must be > 0", l);
     DeviceGuard g(ctx->device);
+    drop_plan_of(ctx, model);
     free_lines(ctx, *m);
     const size_t n = size_t(m->n), nl = n * size_t(n_lines);
     CK(dalloc(ctx, &m->chi0, nl)); CK(dalloc(ctx, &m->eta0, nl));
@@ -804,6 +812,8 @@ mgx_status mgx_set_rays(mgx_ctx *ctx, int32_t model, int32_t l_min, int32_t l_ma
             if (sample[s] < 0 || sample[s] >= m->n) return fail(ctx, MGX_EINVAL, "set_rays: sample[%lld] out of range", (long long)s);
     }
     DeviceGuard g(ctx->device);
+    if (l_max > ctx->tab_level) free_plan(ctx, ctx->plan);  // its models' directions are replaced
+    else drop_plan_of(ctx, model);
     mgx_status s = ensure_tables(ctx, l_max);
     if (s != MGX_OK) return s;
     drop_offsets(ctx, *m);

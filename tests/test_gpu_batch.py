@@ -237,3 +237,44 @@ def test_failed_set_rays_leaves_no_ray_set():
         np.testing.assert_array_equal(ctx.solve_J(mid, I_bdy=0.5), J)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("what", ["lines", "rays", "deeper tables"])
+def test_changed_model_is_planned_anew(what):
+    """A captured step whose model is given other lines or another ray set, or whose direction tables are
+    replaced for another model's finer rays, another model having taken the freed memory: the next call
+    gives what a new context gives."""
+    import synth
+
+    import paper_2011_14998_gb300 as mgx
+
+    a = synth.random_cloud(300, seed=4, n_lines=1, n_freq=20, l_min=0, l_max=1)
+    b = synth.random_cloud(300, seed=5, n_lines=1, n_freq=20, l_min=0, l_max=1)
+    flags = mgx.MGX_BATCH_GRAPH | mgx.MGX_BATCH_RAYS
+
+    def set_lines(ctx, mid, m):
+        mgx.mgx_set_lines(ctx.ptr, mid, m["nu0"], m["chi0"], m["eta0"], m["dvw"], m["chi_c"], m["eta_c"], 20, 4.0)
+
+    changed = dict(a, x_span=4.0, chi0=0.1 * a["chi0"], eta0=0.2 * a["eta0"])
+    half = a["sample"][::2].copy()
+    ctx = mgx.Context(0)
+    try:
+        mid = ctx.load(dict(a, x_span=4.0))
+        outs = ctx.solve_J_batch([mid], flags=flags)
+        if what == "lines":
+            set_lines(ctx, mid, changed)
+        elif what == "rays":
+            ctx.set_rays(mid, 0, 1, half)
+        ctx.load(b, l_min=0 if what != "deeper tables" else 2, l_max=1 if what != "deeper tables" else 2)
+        J = ctx.solve_J_batch([mid], outs=outs, flags=flags)[0].cpu().numpy()
+        again = ctx.solve_J_batch([mid], outs=outs, flags=flags)[0].cpu().numpy()
+    finally:
+        ctx.close()
+    ctx = mgx.Context(0)
+    try:
+        mid = ctx.load(changed if what == "lines" else dict(a, x_span=4.0), sample=half if what == "rays" else None)
+        ref = ctx.solve_J_batch([mid], flags=flags)[0].cpu().numpy()
+    finally:
+        ctx.close()
+    np.testing.assert_array_equal(J, ref)
+    np.testing.assert_array_equal(again, ref)

@@ -1742,7 +1742,10 @@ __device__ __forceinline__ bool int_split_step(const double *src, unsigned on, b
 //   (N, Q) -> ((1, b), (t, 1 + t b)) (N, Q),   W -> W + S b Q.
 // Eight consecutive ones are composed into one map, six operations a bin in
 // place of 32; the lanes hold one row each and compose them in three doubling
-// steps (36 operations a round of records).  A block starts at the third
+// steps (47 operations a round of records).  The map is held less the identity:
+// an interval of many samples repeats one map, and its rounding, 2^-53 of 1, would
+// add up block by block (-2e-14 of J over thousands of samples), where the sums
+// with N and Q round differently each time.  A block starts at the third
 // record of a run (the first two rows still depend on the bin), or where the
 // last block ended.  Not where an increment is so large that the map's entries
 // could leave the range of the state.  bound: the records at which a run
@@ -1760,24 +1763,34 @@ __device__ __forceinline__ unsigned compose_blocks(Stage<C> &sg, int lane, int n
                        (bound & (need & ~(1u << lane))) == 0u;
     const unsigned starts = __ballot_sync(kFull, start);
     if (starts == 0u) return 0u;
-    double m11 = 1.0, m12 = 0.0, m21 = 0.0, m22 = 1.0, al = 0.0, be = 0.0;
+    double m11, m12 = 0.0, m21 = 0.0, m22 = 0.0, al, be = 0.0;
     if (lane > 1 && ((ok >> lane) & 1u)) {
-        const double t = 2.0 * o[4];
         m12 = o[5];
-        m21 = t;
-        m22 = fma(t, m12, 1.0);
+        m21 = 2.0 * o[4];
+        m22 = m21 * m12;
         be = o[1 - Stage<C>::kS] * m12;
     }
+    {  // of single rows m11 and al are 0
+        const double s12 = __shfl_down_sync(kFull, m12, 1), s21 = __shfl_down_sync(kFull, m21, 1);
+        const double s22 = __shfl_down_sync(kFull, m22, 1), sb = __shfl_down_sync(kFull, be, 1);
+        al = sb * m21;
+        be = fma(sb, m22, sb + be);
+        m11 = s12 * m21;
+        const double n12 = fma(s12, m22, s12 + m12);
+        m21 = fma(s22, m21, s21 + m21);
+        m22 = fma(s21, m12, fma(s22, m22, s22 + m22));
+        m12 = n12;
+    }
 #pragma unroll
-    for (int d = 1; d < kBlock; d <<= 1) {
+    for (int d = 2; d < kBlock; d <<= 1) {
         const double s11 = __shfl_down_sync(kFull, m11, d), s12 = __shfl_down_sync(kFull, m12, d);
         const double s21 = __shfl_down_sync(kFull, m21, d), s22 = __shfl_down_sync(kFull, m22, d);
         const double sa = __shfl_down_sync(kFull, al, d), sb = __shfl_down_sync(kFull, be, d);
-        al = fma(sa, m11, fma(sb, m21, al));
-        be = fma(sa, m12, fma(sb, m22, be));
-        const double n11 = fma(s11, m11, s12 * m21), n12 = fma(s11, m12, s12 * m22);
-        m21 = fma(s21, m11, s22 * m21);
-        m22 = fma(s21, m12, s22 * m22);
+        al = fma(sa, m11, fma(sb, m21, sa + al));
+        be = fma(sa, m12, fma(sb, m22, sb + be));
+        const double n11 = fma(s11, m11, fma(s12, m21, s11 + m11)), n12 = fma(s11, m12, fma(s12, m22, s12 + m12));
+        m21 = fma(s21, m11, fma(s22, m21, s21 + m21));
+        m22 = fma(s21, m12, fma(s22, m22, s22 + m22));
         m11 = n11;
         m12 = n12;
     }
@@ -1894,8 +1907,8 @@ __device__ __noinline__ int consume_int(Stage<C> &sg, Lane<C> &ln, const SolveAr
                         for (int i = 0; i < C::BPL; ++i) {
                             const double N = w[i].N, Q = w[i].Q;
                             w[i].W = fma(b[4], N, fma(b[5], Q, w[i].W));
-                            w[i].N = fma(b[0], N, b[1] * Q);
-                            w[i].Q = fma(b[2], N, b[3] * Q);
+                            w[i].N = fma(b[0], N, fma(b[1], Q, N));
+                            w[i].Q = fma(b[2], N, fma(b[3], Q, Q));
                             w[i].h = src[4];
                             w[i].T = src[2];
                             w[i].S = src[1];

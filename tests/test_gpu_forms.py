@@ -177,3 +177,27 @@ def test_fp64_composed_rows(orc, lines):
              chi_c=chi_c, eta_c=chi_c * rng.uniform(0.2, 1.5, n))
     for dtau_max in (0.5, 1e5):
         assert fp64_error(orc, m, dtau_max=dtau_max) < 3e-13
+
+
+def test_fp64_rows_of_equal_increments(orc):
+    """Intervals of some hundred velocity samples, most without a line: their rows repeat one map, whose
+    rounding must not add up.  Over the origins of a thin cloud the roundings of J (some 1e-15 each, for
+    lines of some thousand rows) average out: the mean relative difference from the oracle stays below 2e-15."""
+    import paper_2011_14998_gb300 as mgx
+
+    m = synth.random_cloud(60, seed=8, n_lines=1, n_freq=20, x_span=4.0, l_min=1, l_max=1, v_rms=2.0)
+    for dvw, chi in ((0.02, 1.0), (0.02, 1e-2), (0.01, 10.0)):
+        q = dict(m, dvw=dvw * m["dvw"], chi0=chi * m["chi0"], eta0=chi * m["eta0"], chi_c=chi * m["chi_c"],
+                 eta_c=chi * m["eta_c"])
+        ctx = mgx.Context(0)
+        try:
+            mid = ctx.load(q)
+            rays = ctx.rays(mid)
+            J = ctx.solve_J(mid, precision=mgx.MGX_FP64, I_bdy=0.05)
+        finally:
+            ctx.close()
+        o = np.arange(0, 60, 4)
+        Jo = orc.OracleModel(q, rays=rays).solve_J(orc.params(I_bdy=0.05), origins=o)
+        d = J[o] / Jo - 1.0
+        print(dvw, chi, d.mean(), d.std(), np.abs(d).max())
+        assert abs(d.mean()) < 2e-15

@@ -136,6 +136,48 @@ __host__ __device__ __forceinline__ float far_profile(double cc, double ec, doub
     return fminf(sqrtf(fmaxf(54.1f + x, 0.f)) * 1.0001f + 1e-3f, 31.f);
 }
 
+// 1 / x and 1 / sqrt x as the device approximates them (documented within 1 and 2
+// ulp).  On the host, for the tests, the rounded values moved by MGX_HOST_ULPS.
+#ifndef MGX_HOST_ULPS
+#define MGX_HOST_ULPS 0
+#endif
+__host__ __device__ __forceinline__ float moved(float r, int ulps) {
+    uint32_t b;
+    memcpy(&b, &r, 4);
+    b += uint32_t(ulps);
+    memcpy(&r, &b, 4);
+    return r;
+}
+
+__host__ __device__ __forceinline__ float rcp_approx(float x) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return moved(1.0f / x, MGX_HOST_ULPS);
+#endif
+}
+
+__host__ __device__ __forceinline__ float rsqrt_approx(float x) {
+#ifdef __CUDA_ARCH__
+    return rsqrtf(x);
+#else
+    return moved(float(1.0 / sqrt(double(x))), 2 * MGX_HOST_ULPS);
+#endif
+}
+
+// sqrt(a) for a >= 0 within 0.51 ulp; outside the range of the single-precision
+// root the library's.
+__host__ __device__ __forceinline__ double root(double a) {
+    if (!(a > 1e-36 && a < 1e36)) return sqrt(a);
+    const double y = double(rsqrt_approx(float(a)));  // 2^-21.4
+    double s = a * y;
+    const double h = 0.5 * y;
+    s = fma(fma(-s, s, a), h, s);         // 2^-42
+    return fma(fma(-s, s, a), h, s);
+}
+
 // e / t for finite e >= 0, t > 0: the mantissas' quotient from a
 // single-precision reciprocal and one fixed-point correction with its square.
 __host__ __device__ __forceinline__ double div_pos(double e, double t) {
@@ -146,15 +188,9 @@ __host__ __device__ __forceinline__ double div_pos(double e, double t) {
     const uint64_t me = ((be << 10) & man) | hid, mt = ((bt << 10) & man) | hid;  // Q1.62
     const uint32_t tb = 0x3f800000u | (uint32_t(bt >> 29) & 0x7fffffu);
     // the reciprocal of t's leading bits, lowered by 2^-21 so that 1 - t x is not negative
-#ifdef __CUDA_ARCH__
-    float x;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(__uint_as_float(tb)));
-    const uint32_t X = __float2uint_rz(x * 2147482624.0f);  // Q1.31
-#else
     float x;
     memcpy(&x, &tb, 4);
-    const uint32_t X = uint32_t(1.0f / x * 2147482624.0f);
-#endif
+    const uint32_t X = uint32_t(rcp_approx(x) * 2147482624.0f);  // Q1.31
     const uint64_t tx = uint64_t(uint32_t(mt >> 32)) * X + mul_hi32(uint32_t(mt), X);  // t x in Q2.61
     const uint64_t qe = uint64_t(uint32_t(me >> 32)) * X + mul_hi32(uint32_t(me), X);
     uint64_t d = (uint64_t(1) << 61) - tx;  // 1 - t x in [0, 2^-20)
@@ -241,13 +277,7 @@ __host__ __device__ __forceinline__ uint64_t pivot_q(uint64_t t, uint64_t b, uin
     const uint64_t F = b + Y;
     const uint64_t den = (uint64_t(1) << 59) + mul_hi63(t, F);  // Q4.59, in [1, 4)
     const uint32_t top = uint32_t(den >> 30);                   // Q2.29
-#ifdef __CUDA_ARCH__
-    float x;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(float(top)));  // 2^-29 / den
-    const uint32_t X = __float2uint_rz(x * 1152920954851033088.0f);  // Q0.31, low by up to 2^-20
-#else
-    const uint32_t X = uint32_t(1.0f / float(top) * 1152920954851033088.0f);
-#endif
+    const uint32_t X = uint32_t(rcp_approx(float(top)) * 1152920954851033088.0f);  // Q0.31, low by up to 2^-20
     const uint64_t dx = uint64_t(uint32_t(den >> 32)) * X + mul_hi32(uint32_t(den), X);  // den X in Q.58
     uint64_t d = (uint64_t(1) << 58) - dx;  // 1 - den X in [0, 2^-20.5)
     const uint32_t dh = uint32_t((d + (1u << 21)) >> 22);

@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 #include <mma.h>
 
+#include "f64_int.cuh"
 #include "mgx_internal.cuh"
 
 namespace mgx {
@@ -253,22 +254,11 @@ __global__ void k_mlp_adam(float *__restrict__ theta, float *__restrict__ m, flo
 // pass of its own (a logarithm per edge was a third of the time), the largest
 // velocity difference is compared squared (the square root is monotone), as
 // bits, and the distances' square roots are a single-precision reciprocal root
-// with two corrections (seven operations).  200 000 points, 5.1e6 edges: 0.77 ->
+// with two corrections (root, seven operations).  200 000 points, 5.1e6 edges: 0.77 ->
 // 0.36 ms.
 __global__ void k_log(const double *__restrict__ x, int64_t n, double *__restrict__ y) {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i < n) y[i] = log(x[i]);
-}
-
-// sqrt(a) for a >= 0 within an ulp; outside the range of the single-precision
-// root the library's.
-__device__ __forceinline__ double root(double a) {
-    if (!(a > 1e-36 && a < 1e36)) return sqrt(a);
-    const double y = double(rsqrtf(float(a)));  // 2^-22
-    double s = a * y;
-    const double h = 0.5 * y;
-    s = fma(fma(-s, s, a), h, s);         // 2^-44
-    return fma(fma(-s, s, a), h, s);
 }
 
 // The larger of two non-negative doubles (their bits order as they do).

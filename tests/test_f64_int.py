@@ -33,6 +33,7 @@ extern "C" double t_piv(double t, double b, uint64_t *Y) {
 extern "C" void t_pivot(double dt, double dtb, uint64_t *Y, float *D, float *bD) { mgx::pivot(dt, dtb, *Y, *D, *bD); }
 extern "C" double t_held(uint64_t Y) { return mgx::held_y(Y); }
 extern "C" uint64_t t_hold(double y) { return mgx::hold_y(y); }
+extern "C" double t_root(double a) { return mgx::root(a); }
 extern "C" uint64_t t_arg(uint64_t alpha, uint64_t g, uint64_t u) { return mgx::arg_magnitude(alpha, g, u); }
 extern "C" float t_far(double cc, double ec, double c0, double e0) { return mgx::far_profile(cc, ec, c0, e0); }
 extern "C" float t_prod(double b, uint64_t D) { return mgx::narrow_product(b, D); }
@@ -43,10 +44,21 @@ extern "C" uint64_t t_tab(int j) { return tab.v[j]; }
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
+    return compiled(tmp_path_factory, 0)
+
+
+@pytest.fixture(scope="module", params=[-1, 1])
+def moved(request, tmp_path_factory):
+    """With the approximate reciprocals as far off as the device's may be."""
+    return compiled(tmp_path_factory, request.param)
+
+
+def compiled(tmp_path_factory, ulps):
     d = tmp_path_factory.mktemp("f64")
     (d / "t.cpp").write_text(SRC)
     so = str(d / "t.so")
-    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I",
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC",
+                    f"-DMGX_HOST_ULPS={ulps}", "-I",
                     os.path.join(ROOT, "paper_2011_14998_gb300", "csrc"), str(d / "t.cpp"), "-o", so], check=True)
     L = C.CDLL(so)
     L.t_exp.restype, L.t_exp.argtypes = C.c_double, [C.c_uint64]
@@ -55,6 +67,7 @@ def lib(tmp_path_factory):
     L.t_pivot.restype, L.t_pivot.argtypes = None, [C.c_double, C.c_double, C.POINTER(C.c_uint64)] + [C.POINTER(C.c_float)] * 2
     L.t_held.restype, L.t_held.argtypes = C.c_double, [C.c_uint64]
     L.t_hold.restype, L.t_hold.argtypes = C.c_uint64, [C.c_double]
+    L.t_root.restype, L.t_root.argtypes = C.c_double, [C.c_double]
     L.t_arg.restype, L.t_arg.argtypes = C.c_uint64, [C.c_uint64] * 3
     L.t_far.restype, L.t_far.argtypes = C.c_float, [C.c_double] * 4
     L.t_prod.restype, L.t_prod.argtypes = C.c_float, [C.c_double, C.c_uint64]
@@ -211,3 +224,30 @@ def test_profile_argument(lib):
             assert got >= 31 << 57
         else:
             assert abs(got - exact) <= 3
+
+
+def test_division_and_pivot_with_other_reciprocals(moved):
+    test_division(moved)
+    test_pivot(moved)
+    test_pivot_of_any_increment(moved, "thick_thin")
+
+
+def check_root(L):
+    mp.mp.dps = 40
+    rng = np.random.default_rng(17)
+    a = np.concatenate([10.0 ** rng.uniform(-36, 36, 6000), rng.uniform(1, 4, 2000), np.arange(1, 200.0) ** 2])
+    for x in a:
+        ref = mp.sqrt(mp.mpf(float(x)))
+        ulp = mp.mpf(2) ** (int(mp.floor(mp.log(ref, 2))) - 52)
+        # two corrections leave 2^-64 before the last rounding
+        assert abs(mp.mpf(L.t_root(float(x))) - ref) <= (0.5 + 2.0 ** -10) * ulp
+    for x in (0.0, 1e-300, 5e-324, 1e300):
+        assert L.t_root(x) == np.sqrt(x)
+
+
+def test_root(lib):
+    check_root(lib)
+
+
+def test_root_with_other_reciprocals(moved):
+    check_root(moved)

@@ -17,8 +17,9 @@ int solve_bins_per_lane(int precision, int order, int32_t n_lines, int32_t n_bin
 
 // Warps per origin and tile.  A warp takes all pairs of an item one after the
 // other, which leaves the chip idle when there are few items, and its last wave
-// nearly empty when there are a few waves: with fewer than four waves of
-// resident warps (28 per SM in single precision, 16 in the forms with double)
+// nearly empty when there are a few waves: with fewer items than about four
+// waves of warps (a line on their number, 152 SMs with 28 warps in single
+// precision and 16 in the forms with double; the forms hold 12 to 36)
 // the pairs of an item are dealt to several warps, which store u, and J is
 // summed from u in the same order (400 points, 33 pairs: 1.95 -> 0.34 ms;
 // 12 000 points, 96 pairs, Hermitian: 50.8 -> 48.2 ms; 4001 points in double

@@ -164,7 +164,7 @@ __device__ __forceinline__ void vput(float2 &x, int c, float v) { (c ? x.y : x.x
 // the branch-free runs of consume_chunk and the lines left out (line_is_far) the
 // solve of the 50 000-point wind fell from 86.1 to 70.8 ms, of a batch of five
 // four-line models from 136.4 to 95.2 ms, J the same bit for bit.  What bounds it
-// now is latency (issue 56 % busy): the reciprocal and exp2 on the recurrence's
+// now is latency (issue 61 % busy): the reciprocal and exp2 on the recurrence's
 // path and the staging's gathers, at 8 resident CTAs.
 template <typename R_, int NL_, int BPL_, int ORD_, typename P_ = R_>
 struct Form {

@@ -168,6 +168,8 @@ def test_pivot_of_any_increment(lib, kind):
 
 def test_single_precision_results(lib):
     """D and dtb D come out as the nearest floats of the fixed-point D's exact multiples."""
+    from fractions import Fraction
+
     rng = np.random.default_rng(12)
     D = [int(x) for x in rng.integers(1 << 60, 1 << 62, 4000)] + [1 << 62, (1 << 62) - 1, 3 << 60, (1 << 61) + (1 << 37)]
     b = [float(x) for x in 10.0 ** rng.uniform(-40, 0, len(D))]

@@ -278,8 +278,11 @@ enum {
  *           later calls with the same models, parameters, outputs, flags and
  *           tuning replay the graph without host work.  A replay whose traced
  *           lists no longer fit the planned layout fails with MGX_ERANGE and
- *           drops the plan.  Freeing a model, or giving one of the plan's models
- *           lines or rays again, drops the plan: the next call plans anew.
+ *           drops the plan.  Freeing a model drops the plan; so does giving one
+ *           of its models another number of lines or bins, other line centres or
+ *           span, or a ray set of other levels or sample size (new values in
+ *           arrays of the same size do not), and a set of finer rays than any
+ *           before: the next call plans anew.
  * A batch of few items deals the pairs of an origin to several warps; its plan
  * then also holds every pair's u (8 n_k pairs_k n_lines_k n_freq_k bytes, at most
  * 1 GiB in all), unless there is no room for it.

@@ -763,14 +763,20 @@ mgx_status mgx_set_lines(mgx_ctx *ctx, int32_t model, int32_t n_lines, const dou
     for (int l = 0; l < n_lines; ++l)
         if (!std::isfinite(nu0[l]) || !(nu0[l] > 0.0)) return fail(ctx, MGX_EINVAL, "set_lines: nu0[%d] must be > 0", l);
     DeviceGuard g(ctx->device);
-    drop_plan_of(ctx, model);
-    free_lines(ctx, *m);
     const size_t n = size_t(m->n), nl = n * size_t(n_lines);
-    CK(dalloc(ctx, &m->chi0, nl)); CK(dalloc(ctx, &m->eta0, nl));
-    CK(dalloc(ctx, &m->dvw, n)); CK(dalloc(ctx, &m->chic, n)); CK(dalloc(ctx, &m->etac, n));
-    CK(dalloc(ctx, &m->chi0f, nl)); CK(dalloc(ctx, &m->eta0f, nl));
-    CK(dalloc(ctx, &m->dvwf, n)); CK(dalloc(ctx, &m->chicf, n)); CK(dalloc(ctx, &m->etacf, n));
-    CK(dalloc(ctx, &m->pt, 4 * n));
+    // as many lines as before: the arrays stay, and a plan stays good if what it holds by value does
+    const bool keep = m->has_lines && m->L == n_lines;
+    if (!keep || m->F != n_freq || m->x_span != x_span || !std::equal(nu0, nu0 + n_lines, m->nu0))
+        drop_plan_of(ctx, model);
+    if (!keep) {
+        free_lines(ctx, *m);
+        CK(dalloc(ctx, &m->chi0, nl)); CK(dalloc(ctx, &m->eta0, nl));
+        CK(dalloc(ctx, &m->dvw, n)); CK(dalloc(ctx, &m->chic, n)); CK(dalloc(ctx, &m->etac, n));
+        CK(dalloc(ctx, &m->chi0f, nl)); CK(dalloc(ctx, &m->eta0f, nl));
+        CK(dalloc(ctx, &m->dvwf, n)); CK(dalloc(ctx, &m->chicf, n)); CK(dalloc(ctx, &m->etacf, n));
+        CK(dalloc(ctx, &m->pt, 4 * n));
+    }
+    m->has_lines = false;  // until the new values are in
     CK(cudaMemcpyAsync(m->chi0, chi0, nl * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(m->eta0, eta0, nl * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(m->dvw, dvw, n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
@@ -789,6 +795,7 @@ mgx_status mgx_set_lines(mgx_ctx *ctx, int32_t model, int32_t n_lines, const dou
     for (int l = 0; l < n_lines; ++l) m->nu0[l] = nu0[l];
     const mgx_status s = sync_status(ctx);
     if (s != MGX_OK) {
+        drop_plan_of(ctx, model);
         free_lines(ctx, *m);
         return s;
     }
@@ -812,8 +819,10 @@ mgx_status mgx_set_rays(mgx_ctx *ctx, int32_t model, int32_t l_min, int32_t l_ma
             if (sample[s] < 0 || sample[s] >= m->n) return fail(ctx, MGX_EINVAL, "set_rays: sample[%lld] out of range", (long long)s);
     }
     DeviceGuard g(ctx->device);
+    // a set of the same levels and sample size is made in the old one's arrays, and a plan stays good
+    const bool keep_sample = adaptive && m->sample && m->split && m->n_sample == n_sample;
     if (l_max > ctx->tab_level) free_plan(ctx, ctx->plan);  // its models' directions are replaced
-    else drop_plan_of(ctx, model);
+    else if (!m->has_rays || m->lmin != l_min || m->lmax != l_max || (adaptive && !keep_sample)) drop_plan_of(ctx, model);
     mgx_status s = ensure_tables(ctx, l_max);
     if (s != MGX_OK) return s;
     drop_offsets(ctx, *m);
@@ -830,11 +839,13 @@ mgx_status mgx_set_rays(mgx_ctx *ctx, int32_t model, int32_t l_min, int32_t l_ma
         launch_rays_fixed(m->n, l_min, m->npairs, ctx->pair_lists_dev[size_t(l_min)], m->rays, ctx->stream);
         CK(cudaGetLastError());
     } else {
-        dfree(ctx, m->sample);
-        dfree(ctx, m->split);
-        CK(dalloc(ctx, &m->sample, size_t(n_sample)));
-        CK(dalloc(ctx, &m->split, size_t(n_sample) * 2));
-        m->n_sample = n_sample;
+        if (!keep_sample) {
+            dfree(ctx, m->sample);
+            dfree(ctx, m->split);
+            CK(dalloc(ctx, &m->sample, size_t(n_sample)));
+            CK(dalloc(ctx, &m->split, size_t(n_sample) * 2));
+            m->n_sample = n_sample;
+        }
         if (n_sample > 0)
             CK(cudaMemcpyAsync(m->sample, sample, size_t(n_sample) * sizeof(int32_t), cudaMemcpyHostToDevice,
                                ctx->stream));

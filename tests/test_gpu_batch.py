@@ -239,11 +239,12 @@ def test_failed_set_rays_leaves_no_ray_set():
         ctx.close()
 
 
-@pytest.mark.parametrize("what", ["lines", "rays", "deeper tables"])
-def test_changed_model_is_planned_anew(what):
-    """A captured step whose model is given other lines or another ray set, or whose direction tables are
-    replaced for another model's finer rays, another model having taken the freed memory: the next call
-    gives what a new context gives."""
+@pytest.mark.parametrize("what", ["lines", "more bins", "span", "rays", "sample", "deeper tables"])
+def test_step_of_a_changed_model(what):
+    """A captured step whose model is given other lines (in the same arrays; of another span; with more
+    bins) or another ray set (of as many sample points; of fewer), or whose direction tables are replaced for
+    another model's finer rays, another model having taken what was freed: the next calls give what a
+    new context gives."""
     import synth
 
     import paper_2011_14998_gb300 as mgx
@@ -253,18 +254,26 @@ def test_changed_model_is_planned_anew(what):
     flags = mgx.MGX_BATCH_GRAPH | mgx.MGX_BATCH_RAYS
 
     def set_lines(ctx, mid, m):
-        mgx.mgx_set_lines(ctx.ptr, mid, m["nu0"], m["chi0"], m["eta0"], m["dvw"], m["chi_c"], m["eta_c"], 20, 4.0)
+        mgx.mgx_set_lines(ctx.ptr, mid, m["nu0"], m["chi0"], m["eta0"], m["dvw"], m["chi_c"], m["eta_c"], m["n_freq"],
+                          m["x_span"])
 
-    changed = dict(a, x_span=4.0, chi0=0.1 * a["chi0"], eta0=0.2 * a["eta0"])
-    half = a["sample"][::2].copy()
+    bins = 40 if what == "more bins" else 20
+    lines = dict(a, chi0=0.1 * a["chi0"], eta0=0.2 * a["eta0"], n_freq=bins, x_span=2.0 if what == "span" else a["x_span"])
+    sample = np.random.default_rng(1).integers(0, 300, 150 if what == "rays" else 300).astype(np.int32)
+    changed = dict(a) if what in ("rays", "sample", "deeper tables") else lines
+    if what in ("rays", "sample"):
+        changed["sample"] = sample
+    import torch
+
+    outs = [torch.empty((300, bins), dtype=torch.float64, device="cuda")]
     ctx = mgx.Context(0)
     try:
-        mid = ctx.load(dict(a, x_span=4.0))
-        outs = ctx.solve_J_batch([mid], flags=flags)
-        if what == "lines":
+        mid = ctx.load(dict(a, n_freq=bins) if what != "more bins" else a)
+        ctx.solve_J_batch([mid], outs=outs, flags=flags)
+        if what in ("rays", "sample"):
+            ctx.set_rays(mid, 0, 1, sample)
+        elif what != "deeper tables":
             set_lines(ctx, mid, changed)
-        elif what == "rays":
-            ctx.set_rays(mid, 0, 1, half)
         ctx.load(b, l_min=0 if what != "deeper tables" else 2, l_max=1 if what != "deeper tables" else 2)
         J = ctx.solve_J_batch([mid], outs=outs, flags=flags)[0].cpu().numpy()
         again = ctx.solve_J_batch([mid], outs=outs, flags=flags)[0].cpu().numpy()
@@ -272,8 +281,7 @@ def test_changed_model_is_planned_anew(what):
         ctx.close()
     ctx = mgx.Context(0)
     try:
-        mid = ctx.load(changed if what == "lines" else dict(a, x_span=4.0), sample=half if what == "rays" else None)
-        ref = ctx.solve_J_batch([mid], flags=flags)[0].cpu().numpy()
+        ref = ctx.solve_J_batch([ctx.load(changed)], flags=flags)[0].cpu().numpy()
     finally:
         ctx.close()
     np.testing.assert_array_equal(J, ref)

@@ -16,7 +16,7 @@ __global__ void k_ingest_points(int32_t n, const double *__restrict__ pos,
     if (i > n) return;
     const int64_t o = off64[i];
     if (o < 0 || o > E || (i < n && off64[i + 1] < o)) dev_fail(status, kDevBadCsr);
-    off32[i] = int32_t(o);
+    off32[i] = int32_t(o < 0 ? 0 : o > E ? E : o);  // within the array also where it is refused
     if (i == n) return;
     const double px = pos[3 * i], py = pos[3 * i + 1], pz = pos[3 * i + 2];
     const double ux = vel[3 * i], uy = vel[3 * i + 1], uz = vel[3 * i + 2];
@@ -40,7 +40,7 @@ __global__ void k_ingest_points(int32_t n, const double *__restrict__ pos,
 __global__ void k_check_nbr(int32_t n, const int32_t *__restrict__ off, const int32_t *__restrict__ nbr,
                             int *status) {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *status != 0) return;  // (offsets refused: rows could be of any length)
     for (int32_t e = off[i]; e < off[i + 1]; ++e) {
         const int32_t j = nbr[e];
         if (j < 0 || j >= n || j == i) dev_fail(status, kDevBadCsr);
@@ -80,9 +80,9 @@ void launch_ingest_mesh(int32_t n, const double *pos_aos, const double *vel_aos,
 // position of nbr[e] minus the float position of its point, next to its id, in
 // CSR order (the spare record after the last stays zero)
 __global__ void k_pack_neighbours(int32_t n, const int32_t *__restrict__ off, const int32_t *__restrict__ nbr,
-                                  float4 *__restrict__ phi, float4 *__restrict__ nrec) {
+                                  float4 *__restrict__ phi, float4 *__restrict__ nrec, const int *status) {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *status != 0) return;  // a mesh that is refused has no records
     const float4 hi = phi[i];
     float smax = 0.0f;
     for (int32_t e = off[i]; e < off[i + 1]; ++e) {
@@ -97,9 +97,9 @@ __global__ void k_pack_neighbours(int32_t n, const int32_t *__restrict__ off, co
 }
 
 void launch_pack_neighbours(int32_t n, const int32_t *off, const int32_t *nbr, float4 *phi, float4 *nrec,
-                            cudaStream_t st) {
+                            const int *status, cudaStream_t st) {
     const int tb = 256;
-    k_pack_neighbours<<<unsigned((n + tb - 1) / tb), tb, 0, st>>>(n, off, nbr, phi, nrec);
+    k_pack_neighbours<<<unsigned((n + tb - 1) / tb), tb, 0, st>>>(n, off, nbr, phi, nrec, status);
 }
 
 __global__ void k_ingest_lines(int32_t n, int32_t L, const double *__restrict__ chi0,

@@ -713,7 +713,7 @@ mgx_status mgx_load_mesh(mgx_ctx *ctx, int64_t n, const double *pos, const doubl
         Timed t(ctx, MGX_K_OTHER);
         launch_ingest_mesh(m.n, pos_d, vel_d, off64, E, m.x, m.y, m.z, m.vx, m.vy, m.vz, m.vxf, m.vyf,
                            m.vzf, m.off, m.nbr, m.phi, xmax, ctx->d_status, ctx->stream);
-        launch_pack_neighbours(m.n, m.off, m.nbr, m.phi, m.nrec, ctx->stream);
+        launch_pack_neighbours(m.n, m.off, m.nbr, m.phi, m.nrec, ctx->d_status, ctx->stream);
     }
     CK(cudaGetLastError());
     unsigned int xmax_h = 0;

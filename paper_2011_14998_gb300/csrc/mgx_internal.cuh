@@ -101,7 +101,7 @@ void launch_ingest_mesh(int32_t n, const double *pos_aos, const double *vel_aos,
                         const int32_t *nbr, float4 *phi, unsigned int *xmax_bits, int *status,
                         cudaStream_t st);
 void launch_pack_neighbours(int32_t n, const int32_t *off, const int32_t *nbr, float4 *phi,
-                            float4 *nrec, cudaStream_t st);
+                            float4 *nrec, const int *status, cudaStream_t st);
 void launch_ingest_lines(int32_t n, int32_t L, const double *chi0, const double *eta0,
                          const double *dvw, const double *chic, const double *etac, float *chi0f,
                          float *eta0f, float *dvwf, float *chicf, float *etacf, int *status,

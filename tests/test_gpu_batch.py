@@ -286,3 +286,32 @@ def test_step_of_a_changed_model(what):
         ctx.close()
     np.testing.assert_array_equal(J, ref)
     np.testing.assert_array_equal(again, ref)
+
+
+@pytest.mark.parametrize("bad", ["id", "negative id", "offset", "negative offset", "falling offsets"])
+def test_graphs_out_of_range_are_refused(bad):
+    """Neighbour ids and offsets far outside the arrays: MGX_EINVAL, and the context works on."""
+    import synth
+
+    import paper_2011_14998_gb300 as mgx
+
+    m = synth.random_cloud(60, seed=1, l_min=0, l_max=0)
+    off, nbr = m["nbr_off"].astype(np.int64).copy(), m["nbr_idx"].copy()
+    if bad == "id":
+        nbr[7] = 2 ** 31 - 1
+    elif bad == "negative id":
+        nbr[7] = -2 ** 31
+    elif bad == "offset":
+        off[9] = 2 ** 40
+    elif bad == "negative offset":
+        off[9] = -2 ** 40
+    else:
+        off[9] = off[8] - 1
+    ctx = mgx.Context(0)
+    try:
+        with pytest.raises(mgx.MgxError) as e:
+            ctx.load(dict(m, nbr_off=off, nbr_idx=nbr))
+        assert e.value.status == mgx.MGX_EINVAL
+        assert np.isfinite(ctx.solve_J(ctx.load(m))).all()
+    finally:
+        ctx.close()

@@ -11,7 +11,7 @@ __global__ void k_ingest_points(int32_t n, const double *__restrict__ pos,
                                 const double *__restrict__ vel, const int64_t *__restrict__ off64,
                                 int64_t E, double *x, double *y, double *z, double *vx, double *vy,
                                 double *vz, float *vxf, float *vyf, float *vzf, int32_t *off32,
-                                float4 *phi, unsigned int *xmax_bits, int *status) {
+                                unsigned int *xmax_bits, int *status) {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i > n) return;
     const int64_t o = off64[i];
@@ -32,9 +32,17 @@ __global__ void k_ingest_points(int32_t n, const double *__restrict__ pos,
     vxf[i] = float(ux);
     vyf[i] = float(uy);
     vzf[i] = float(uz);
-    phi[i] = make_float4(__double2float_rn(px), __double2float_rn(py), __double2float_rn(pz), 0.0f);
     const float s = __double2float_ru(fabs(px) + fabs(py) + fabs(pz));
     if (isfinite(s)) atomicMax(xmax_bits, __float_as_uint(s));  // non-negative: bit order = value order
+}
+
+// The positions in single precision, scaled.
+__global__ void k_screen_points(int32_t n, const double *__restrict__ x, const double *__restrict__ y,
+                                const double *__restrict__ z, const unsigned int *xmax_bits, float4 *__restrict__ phi) {
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (i >= n) return;
+    const double s = screen_scale(*xmax_bits);
+    phi[i] = make_float4(__double2float_rn(s * x[i]), __double2float_rn(s * y[i]), __double2float_rn(s * z[i]), 0.0f);
 }
 
 __global__ void k_check_nbr(int32_t n, const int32_t *__restrict__ off, const int32_t *__restrict__ nbr,
@@ -72,7 +80,8 @@ void launch_ingest_mesh(int32_t n, const double *pos_aos, const double *vel_aos,
                         cudaStream_t st) {
     const int tb = 256;
     k_ingest_points<<<unsigned((n + 1 + tb - 1) / tb), tb, 0, st>>>(
-        n, pos_aos, vel_aos, off64, E, x, y, z, vx, vy, vz, vxf, vyf, vzf, off32, phi, xmax_bits, status);
+        n, pos_aos, vel_aos, off64, E, x, y, z, vx, vy, vz, vxf, vyf, vzf, off32, xmax_bits, status);
+    k_screen_points<<<unsigned((n + tb - 1) / tb), tb, 0, st>>>(n, x, y, z, xmax_bits, phi);
     k_check_nbr<<<unsigned((n + tb - 1) / tb), tb, 0, st>>>(n, off32, nbr, status);
 }
 

@@ -164,14 +164,6 @@ __device__ bool vec2pix_nest_f(int l, float a, float b, float c, int32_t &pix) {
     return true;
 }
 
-// The power of two that brings the mesh's X, which bounds |x|_1, to [1, 2), and X
-// so scaled: the screen then sees the same numbers in any unit of length.
-__device__ __forceinline__ double mesh_scale(const DevMesh &m, float &X) {
-    const uint32_t b = __float_as_uint(m.g0 * 8796093022208.0f);  // g0 >= 2^-43 max |x|_1, and 1e-37
-    X = __uint_as_float((b & 0x7fffffu) | 0x3f800000u);
-    return __longlong_as_double((long long)(1150u - (b >> 23)) << 52);
-}
-
 // A position's coordinate, scaled, as two floats.
 __device__ __forceinline__ void split_coordinate(double x, double scale, float &hi, float &lo) {
     x = __dmul_rn(x, scale);
@@ -220,13 +212,11 @@ __global__ void k_split_sample(DevMesh m, int64_t n_sample, const int32_t *__res
     if (s >= n_sample) return;
     const int32_t j = sample[s];
     const bool ok = j >= 0 && j < m.n;
-    float X;
-    const double scale = mesh_scale(m, X);
     float4 h = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(ok ? j : -1)), l = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (ok) {
-        split_coordinate(m.x[j], scale, h.x, l.x);
-        split_coordinate(m.y[j], scale, h.y, l.y);
-        split_coordinate(m.z[j], scale, h.z, l.z);
+        split_coordinate(m.x[j], m.scale, h.x, l.x);
+        split_coordinate(m.y[j], m.scale, h.y, l.y);
+        split_coordinate(m.z[j], m.scale, h.z, l.z);
     }
     sp[2 * s] = h;
     sp[2 * s + 1] = l;
@@ -316,12 +306,11 @@ k_rays_adaptive(DevMesh m, int32_t lmin, int32_t lmax, int32_t npairs, int64_t n
         }
         if (push(open, n_open, left, j)) take_open();
     };
-    float X;
-    const double scale = mesh_scale(m, X);
+    const float X = m.g0 * 8796093022208.0f;  // bounds |x|_1, scaled: g0 >= 2^-43 of its largest
     float4 oh, ol;
-    split_coordinate(xo, scale, oh.x, ol.x);
-    split_coordinate(yo, scale, oh.y, ol.y);
-    split_coordinate(zo, scale, oh.z, ol.z);
+    split_coordinate(xo, m.scale, oh.x, ol.x);
+    split_coordinate(yo, m.scale, oh.y, ol.y);
+    split_coordinate(zo, m.scale, oh.z, ol.z);
     for (int64_t s0 = tid - lane; s0 < n_sample; s0 += nt) {
         int32_t j = -1;
         bool is_far = false, is_open = false;

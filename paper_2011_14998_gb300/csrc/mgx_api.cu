@@ -33,6 +33,7 @@ struct Model {
     int32_t *off = nullptr, *nbr = nullptr;
     float4 *phi = nullptr, *nrec = nullptr;
     float g0 = 0.0f;
+    double scale = 1.0;
     // lines
     bool has_lines = false;
     int32_t L = 0, F = 0;
@@ -263,6 +264,7 @@ DevMesh mesh_view(const Model &m) {
     d.phi = m.phi;
     d.nrec = m.nrec;
     d.g0 = m.g0;
+    d.scale = m.scale;
     return d;
 }
 
@@ -732,7 +734,8 @@ mgx_status mgx_load_mesh(mgx_ctx *ctx, int64_t n, const double *pos, const doubl
         float xm;
         std::memcpy(&xm, &xmax_h, sizeof xm);
         const double u = 1.0 / 16777216.0;  // 2^-24
-        m.g0 = float(32.0 * u * u * double(xm) * (1.0 + 1e-6)) + 1e-37f;
+        m.scale = screen_scale(xmax_h);
+        m.g0 = float(32.0 * u * u * (m.scale * double(xm)) * (1.0 + 1e-6)) + 1e-37f;
     }
     ctx->models.push_back(m);
     *model_id = int32_t(ctx->models.size() - 1);

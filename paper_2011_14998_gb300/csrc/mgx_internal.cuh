@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/mgx.h"
 
@@ -42,10 +43,27 @@ struct DevMesh {
     const float *vxf, *vyf, *vzf;
     const int32_t *off;  // [n+1]
     const int32_t *nbr;  // [E]
+    // what the single-precision screens of the tracer and the ray sets work on, in units 1 / scale
+    // (screen_scale): their squares then neither overflow nor vanish, whatever the unit of length
     const float4 *phi;        // positions rounded to float; w: the largest |x_n - x|_1 over the neighbours (float)
     const float4 *nrec;       // [E + 1] neighbour records: fl32 position of nbr[e] minus that of its point, id in w (int bits)
     float g0;                 // 32 u^2 max_n (|x|+|y|+|z|) + 1e-37: floor of the screen's error bounds
+    double scale;
 };
+
+// The power of two that brings the largest |x|_1 of a mesh (as float bits, rounded
+// up) to [1, 2); a power of two, so that scaled values round as the plain ones do.
+__host__ __device__ __forceinline__ double screen_scale(uint32_t xmax_bits) {
+    const uint32_t e = xmax_bits >> 23;
+    const uint64_t b = uint64_t(1150u - (e > 0 ? e : 1u)) << 52;
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double d;
+    memcpy(&d, &b, sizeof d);
+    return d;
+#endif
+}
 
 struct DevLines {
     int32_t L, F;

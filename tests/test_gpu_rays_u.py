@@ -119,3 +119,35 @@ def test_adaptive_ray_sets_in_any_unit(ctx, orc, kind, unit):
     rays = ctx.rays(mid)
     ctx.free(mid)
     np.testing.assert_array_equal(rays, orc.rayset(pos, 0, 3, m["sample"]))
+
+
+@pytest.mark.parametrize("unit", [-97, -75, -30, 53, 66, 86])
+@pytest.mark.parametrize("kind", ["cloud", "far", "wind"])
+def test_lists_and_J_in_any_unit(ctx, orc, kind, unit):
+    """A mesh in units of 2^-unit, opacities per that unit: the same traced lists (the oracle's), the
+    distances and J in FP64 to the last bit in plain units, J in FP32 within its rounding."""
+    import synth
+
+    import paper_2011_14998_gb300 as mgx
+
+    m = (synth.wind_model(400, seed=3, n_freq=9, level=1) if kind == "wind"
+         else synth.random_cloud(150, seed=6, n_lines=1, n_freq=9, l_min=1, l_max=1))
+    if kind == "far":
+        m = dict(m, pos=m["pos"] + 2.0 ** 10)
+    s = 2.0 ** unit
+    q = dict(m, pos=m["pos"] * s, **{k: m[k] / s for k in ("chi0", "eta0", "chi_c", "eta_c")})
+    got = []
+    for k in (m, q):
+        mid = ctx.load(k)
+        off, idx, Z, _ = ctx.trace(mid, 0, len(k["pos"]), with_delta=True)
+        got.append((off, idx, Z, ctx.solve_J(mid), ctx.solve_J(mid, precision=mgx.MGX_FP32),
+                    ctx.solve_J_batch([mid], precision=mgx.MGX_FP64)[0].cpu().numpy(), ctx.rays(mid)))
+        ctx.free(mid)
+    a, b = got
+    for i in (0, 1, 3, 5, 6):
+        np.testing.assert_array_equal(a[i], b[i])
+    np.testing.assert_array_equal(a[2] * s, b[2])
+    np.testing.assert_allclose(a[4], b[4], rtol=1e-5)
+    o = np.arange(0, len(q["pos"]), 9)
+    Jo = orc.OracleModel(q, rays=b[6]).solve_J(orc.params(), origins=o)
+    assert j_rel_err(b[3][o], Jo)[0] < 1e-12
